@@ -61,7 +61,7 @@ def parse():
     ap.add_argument("--no-batch", action="store_true")
     ap.add_argument("--only-3d", action="store_true",
                     help="time only the 3D (D3Q19, tetrahedra) section and print it as one JSON line")
-    ap.add_argument("--ncu-case", choices=["fp32", "fp32-tiled", "fp64"],
+    ap.add_argument("--ncu-case", choices=["fp32", "fp32-gathered", "fp64"],
                     help="run two steps of the 1024-column rough-wall droplet (1,041,408 nodes, above L2, about "
                          "2 GB on the device) and exit: the small case for ncu captures of the step kernels")
     ap.add_argument("--sweep-parts", type=int, default=2, help="threads per node of the solve steps (--ncu-case)")
@@ -252,7 +252,7 @@ class ClockSampler:
                 "sm_max_mhz": max(mx) if mx else None, "reasons": reasons, "samples": len(self.rows)}
 
 
-SOURCES_2D = ("felbm.cu", "felbm_dev32.cuh", "felbm_adjoint.cuh", "felbm_internal.h", "mesh.cpp", "felbm.h")
+SOURCES_2D = ("felbm.cu", "felbm_dev32.cuh", "felbm_block32.cuh", "felbm_adjoint.cuh", "felbm_internal.h", "mesh.cpp", "felbm.h")
 SOURCES_3D = ("felbm3d.cu", "felbm3d_dev32.cuh", "felbm3d_internal.h", "mesh3d.cpp", "felbm_internal.h",
               "felbm3d.h", "felbm.h")
 
@@ -302,6 +302,15 @@ def recorded_fp64_flops(files=SOURCES_2D):
             if len(parts) >= 4 and not line.startswith("#") and parts[1] == h:
                 out[parts[0]] = (float(parts[2]), parts[3])
     return out
+
+
+def fp32_step_bytes(solve_launches):
+    """Minimum bytes per node-update of the FP32 form's launches:
+    distributions read and written (2 x 18 x 4), right-hand side written and
+    read (2 x 18 x 4), per solve launch an iterate, the right-hand side and
+    the new iterate (3 x 18 x 4; the update's: increment and deviations in,
+    deviations out), about 200 B of nodal and element fields."""
+    return 2 * 18 * 4 + 2 * 18 * 4 + solve_launches * 3 * 18 * 4 + 200
 
 
 def fp64_roofline(r64, n_nodes, n_tri, rate, fp64_peak, flops):
@@ -482,14 +491,12 @@ def time_batch(F, torch, dev, K, flush, barrier, world, dist):
     n = mesh.info()["n_nodes"]
     st.timing_enable(True)
     st.step(1)
-    sweeps = st.timing_get()["solve_launches"] + 1
+    launches = st.timing_get()["solve_launches"]
     st.timing_enable(False)
     st.close()
     value = job_rate(n, K, world, total_ms)
-    # the whole step against the minimum bytes per node-update of the FP32
-    # form, as for the rough wall (distributions and right-hand side written
-    # and read, three 18-float streams per solve step, ~200 B of fields)
-    step_bytes = 2 * 18 * 4 + 2 * 18 * 4 + sweeps * 3 * 18 * 4 + 200
+    # the whole step against the minimum bytes per node-update of its launches, as for the rough wall
+    step_bytes = fp32_step_bytes(launches)
     hbm_peak, peak_src = peaks()
     return {"workload": "64-droplet contact-angle sweep, widths 64..512, FP32 deviation storage",
             "nodes": n, "members": len(b["members"]), "steps": K,
@@ -497,7 +504,7 @@ def time_batch(F, torch, dev, K, flush, barrier, world, dist):
             "ms_per_step": total_ms / K, "schedule": tune,
             "finite": all(d["status"] == 0 for d in dg),
             "max_abs_mass_drift_rel": max(abs(d["mass_drift_rel"]) for d in dg),
-            "step_roofline": {"alg_bytes_per_node_update": step_bytes, "sweeps": sweeps,
+            "step_roofline": {"alg_bytes_per_node_update": step_bytes, "solve_launches": launches,
                               "achieved": value / world * step_bytes / 1e9, "peak": hbm_peak, "unit": "GB/s",
                               "frac": value / world * step_bytes / 1e9 / hbm_peak, "peak_source": peak_src}}
 
@@ -546,7 +553,7 @@ def time_free_droplet(F, torch, dev, K, flush, barrier, world, dist, fp64_peak):
         out[name] = {"value": job_rate(n, K, world, r["total_ms"]), "unit": "node-updates/s",
                      "ms_per_step": r["total_ms"] / K, "steps": K,
                      "phase_ms": {k: round(v, 5) for k, v in r["phase_ms"].items()},
-                     "sweep_ms": r["phase_ms"]["solve_ms"] / r["solve_launches"], "autotune": r["tune"],
+                     "sweep_ms": r["phase_ms"]["solve_ms"] / (r["diag"]["solver_sweeps"] - 1), "autotune": r["tune"],
                      "finite": r["diag"]["status"] == 0}
         if prec == F.FP64:
             out[name]["fp64_roofline"] = fp64_roofline(r, n, len(w["mesh"]["tri"]), out[name]["value"] / world,
@@ -679,23 +686,19 @@ def run_gpu(args):
             raise SystemExit(f"bench: the {name} state is not finite after the timed steps")
     if rank == 0:
         nnz = r32["info"]["nnz"]
-        # dominant kernel of the FP32-deviation step: one step of the FP32
-        # solve of the 18 right-hand sides (the last one also updates the
-        # fields), timed as the solve phase over its launches
-        sweep_ms = r32["phase_ms"]["solve_ms"] / r32["solve_launches"]
-        # algorithmic bytes of one solve step x_{k+1} = x_k + tau m^-1 (b - M x_k):
-        # gathered x_k, b and the new x (3 x 18 floats per node), the mass
-        # row (column index + FP32 value per entry), the inverse lumped mass
-        alg_bytes = N * (3 * 18 * 4 + 4) + nnz * (4 + 4)
+        # the solve phase of the FP32-deviation step: blocked launches (several
+        # steps of the 18 right-hand sides each), then the field update.
+        # Algorithmic bytes of a blocked launch: x in, b, x out (3 x 18 floats
+        # per node), the mass row (column index + FP32 value per entry), the
+        # inverse lumped mass; of the update: the increment and the
+        # deviations in, the deviations out, the fields in and out
+        n_launch = r32["solve_launches"]
+        alg_bytes = (n_launch - 1) * (N * (3 * 18 * 4 + 4) + nnz * (4 + 4)) + N * (3 * 18 * 4 + 2 * 20)
         hbm_peak, peak_src = peaks()
-        achieved = alg_bytes / (sweep_ms * 1e-3) / 1e9
-        # whole step, with the minimum bytes per node-update of the FP32 form:
-        # distributions read and written (2 x 18 x 4), right-hand side written
-        # and read (2 x 18 x 4), per solve step a gathered iterate, the
-        # right-hand side and the new iterate (3 x 18 x 4), about 200 B of
-        # nodal and element fields
-        k_sweeps = r32["solve_launches"] + 1
-        step_bytes = 2 * 18 * 4 + 2 * 18 * 4 + k_sweeps * 3 * 18 * 4 + 200
+        solve_ms = r32["phase_ms"]["solve_ms"]
+        achieved = alg_bytes / (solve_ms * 1e-3) / 1e9
+        step_bytes = fp32_step_bytes(n_launch)
+        k_sweeps = r32["diag"]["solver_sweeps"]
 
         def summary(r, dtype):
             return {"value": job_rate(N, K, world, r["total_ms"]), "ms_per_step": r["total_ms"] / K,
@@ -727,7 +730,7 @@ def run_gpu(args):
             "data": "synthetic",
             "config": dict(workload_config(w, world), precision="FP32 deviation storage (fp32_dev); "
                            "plain FP64 in fp64", solver=f"FP32 Richardson steps at the Chebyshev roots, "
-                                                         f"{r32['solve_launches'] + 1} per step"),
+                                                         f"{k_sweeps} per step"),
             "fp32_dev": s32,
             "fp64": s64,
             "free_droplet_256": rfd,
@@ -735,14 +738,15 @@ def run_gpu(args):
             "adjoint": radj,
             "tetrahedra_3d": r3,
             "step_roofline": {"alg_bytes_per_node_update": step_bytes, "sweeps": k_sweeps,
+                              "solve_launches": n_launch,
                               "achieved": s32["value"] * step_bytes / 1e9, "peak": hbm_peak, "unit": "GB/s",
                               "frac": s32["value"] * step_bytes / 1e9 / hbm_peak,
                               "frac_of_nominal_8TBps": s32["value"] * step_bytes / 1e9 / nominal},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
-                         "frac": achieved / hbm_peak, "traffic": recorded_traffic("k_sweep32"),
-                         "kernel": "k_sweep32 (one step of the FP32 solve of the 18 right-hand sides)",
+                         "frac": achieved / hbm_peak, "traffic": recorded_traffic("solve_phase"),
+                         "kernel": "solve phase: k_block32 launches of the FP32 solve, then k_update32",
                          "source_hash": source_hash(),
-                         "alg_bytes_per_launch": alg_bytes, "launch_ms": sweep_ms,
+                         "alg_bytes": alg_bytes, "phase_ms": solve_ms,
                          "peak_source": peak_src, "frac_of_nominal_8TBps": achieved / nominal},
             "e2e": {"value": s32["e2e_value"], "unit": "node-updates/s",
                     "h2d_bytes_per_step": r32["state_bytes"], "d2h_bytes_per_step": 8 * F.DIAG_SLOTS},
@@ -795,8 +799,8 @@ def ncu_case(args):
     prec = F.FP64 if args.ncu_case == "fp64" else F.FP32_DEV
     st = F.State(F.Mesh.from_dict(w["mesh"]), F.params_derive(w["phys"], precision=prec), w["C0"], device="cuda:0")
     st.sweep_parts(args.sweep_parts)
-    if args.ncu_case == "fp32-tiled":
-        st.sweep_tiled(True)
+    if args.ncu_case == "fp32-gathered":
+        st.sweep_tiled(False)
     st.step(2)
     torch.cuda.synchronize()
     print(json.dumps({"ncu_case": args.ncu_case, "nodes": len(w["mesh"]["xy"]), "status": st.diagnostics()["status"]}))

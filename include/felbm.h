@@ -15,7 +15,8 @@
  *  - Host arrays are owned by the caller and only read (or written) during
  *    the call.  Node numbering is the caller's: the library reorders nodes
  *    internally (compact tiles of at most 1024 nodes by recursive coordinate
- *    bisection, reverse Cuthill-McKee order inside a tile) and converts back
+ *    bisection, halved once more into blocks, reverse Cuthill-McKee order
+ *    inside a block) and converts back
  *    on every exchange.
  *  - Device memory: the library never allocates it.  The caller allocates one
  *    workspace of felbm_workspace_bytes() bytes (any allocator, 256-byte
@@ -289,39 +290,31 @@ int felbm_batch_schedule(felbm_state* state, int32_t cta_max_nodes);
  * rebuilt at the next felbm_step.  Synchronises. */
 int felbm_solver_check(felbm_state* state, int32_t enable, double tol);
 
-/* Threads per node of the FP32 solve sweeps (states with an FP32 solve):
- * 1, 2, 3 or 6, each owning 18 / parts of the node's right-hand sides.  Every
- * choice performs the same arithmetic per row, so the trajectory does not
- * depend on it; felbm_autotune picks one by timing.  Default 2.  The step
- * graph is rebuilt at the next felbm_step.  FELBM_ERR_INVALID_ARG for any
- * other value. */
+/* Threads per node of the gathered FP32 solve sweeps (states with an FP32
+ * solve): 1, 2, 3 or 6, which share the node's right-hand sides.  Every choice
+ * performs the same arithmetic per row, so the trajectory does not depend on
+ * it; felbm_autotune picks one by timing.  Default 2.  Without effect while
+ * the solve runs blocked (felbm_sweep_tiled).  The step graph is rebuilt at
+ * the next felbm_step.  FELBM_ERR_INVALID_ARG for any other value. */
 int felbm_sweep_parts(felbm_state* state, int32_t parts);
 
-/* Where the FP32 store sweeps of the solve read their operands (states with
- * an FP32 solve and an ELL pattern).  0: each thread gathers its row's
- * neighbours from global memory.  1: a persistent grid, one block per SM,
- * walks (node tile, part of the right-hand sides) items through up to four
- * stages of shared memory: 1D TMA bulk copies bring the tile's runs of the iterate,
- * right-hand side, ELL rows and inverse lumped mass, cp.async the tile's
- * halo, while the block computes an earlier item from another stage.
- * The tiled step splits the 18 right-hand sides in 3 or 6 parts (the
- * felbm_sweep_parts value if it is one of those and fits, else 6).  Same
- * arithmetic in the same order: the trajectory does not depend on it.
- * FELBM_ERR_UNSUPPORTED if a tile's halo exceeds the staged rows (504
- * nodes) or the rows are too long for two stages.  On the meshes measured
- * here the gathered form is faster (the autotuner keeps it).  A tiled sweep whose
- * copy has not landed after 0.2 s stops (and later blocks skip their work)
- * and sets an error bit that the next felbm_diagnostics or felbm_get_state
- * reports as FELBM_ERR_CUDA.
- * The step graph is rebuilt at the next felbm_step.  Default 0;
+/* How the FP32 solve (states with an FP32 solve and an ELL pattern) walks its
+ * sweeps.  0: one launch per sweep, each thread gathering its row's
+ * neighbours from global memory.  1: blocked -- a thread block keeps a run of
+ * at most 512 nodes and the layers of nodes around it in shared memory and
+ * advances several sweeps per launch.  Same arithmetic per row in the same
+ * order: the trajectory does not depend on it.  FELBM_ERR_UNSUPPORTED if the
+ * mesh has no ELL copy, rows of more than 12 entries, or a node tile that
+ * references more than 504 nodes outside it (then 0 is used).  The step graph
+ * is rebuilt at the next felbm_step.  Default: 1 where it is supported;
  * felbm_autotune picks one by timing. */
 int felbm_sweep_tiled(felbm_state* state, int32_t on);
 
 typedef struct felbm_tune_result {
     int32_t sweep_parts;     /* chosen threads per node of the FP32 solve sweeps */
     float parts_ms[4];       /* step time with 1, 2, 3, 6 threads per node (0 = not timed) */
-    int32_t sweep_tiled;     /* 1: the tiled store sweeps were chosen (felbm_sweep_tiled) */
-    float tiled_ms[4];       /* step time of the tiled sweeps with 1, 2, 3, 6 parts (0 = not timed) */
+    int32_t sweep_tiled;     /* 1: the blocked sweeps were chosen (felbm_sweep_tiled) */
+    float tiled_ms[4];       /* step time of the blocked sweeps in entry 2 (0 = not timed) */
     int32_t cta_max_nodes;   /* chosen batch threshold (0 = tiled only) */
     int32_t n_candidates;
     int32_t candidates[16];  /* thresholds timed */
@@ -331,7 +324,7 @@ typedef struct felbm_tune_result {
 /* Autotuner: times `trials` steps (after one warm-up step) per candidate and
  * keeps the fastest -- first the threads per node of the FP32 solve sweeps
  * (1, 2, 3 or 6; states with an FP32 solve and an ELL pattern; see
- * felbm_sweep_parts), each gathered and tiled (felbm_sweep_tiled), then, for
+ * felbm_sweep_parts), each gathered, and the blocked form (felbm_sweep_tiled), then, for
  * FP32_DEV batches, each distinct split of the members (tiled only, CTA per
  * member up to 2^11 .. 2^17 nodes).  The state and the step count are saved
  * before and restored after, so the simulation is unchanged.  Synchronises. */

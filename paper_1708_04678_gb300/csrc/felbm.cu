@@ -24,8 +24,10 @@
 //               A_T (Phi - e.grad psi_hat) of eq:galerkin_lbm
 //   k_rhs       node-centric gather of the streaming right-hand side with
 //               weak bounce-back on walls; first Chebyshev iterate
-//   k_cheb      Chebyshev sweeps of the consistent-mass solve with the
-//               lumped-mass preconditioner; the last adds the increment
+//   k_block32   sweeps of the consistent-mass solve with the lumped-mass
+//               preconditioner, several per launch (FP32 corrections; k_sweep32
+//               and k_cheb32 one at a time, k_cheb in FP64); the last adds the
+//               increment
 // No floating-point atomics: every sum is a fixed-order loop or tree.  The one
 // atomic is an integer counter that picks the block of k_diag_fused32 that
 // combines the blocks' partials (in block order, whichever block it is).
@@ -93,12 +95,16 @@ struct DevMesh {
     const float* mval32;      // [nnz] FP32 copy of the mass entries
     int32_t ell_w;            // width of the ELL copy (max row length), 0 = none
     const int32_t* ell_col;   // [ell_w][Np] column-major ELL copy of the pattern
-    const uint16_t* ell_loc;  // [ell_w][Np] the same columns as indices into the node's tile's staged row
-    int32_t n_tiles;          // node tiles (contiguous id ranges, HostMesh::tile_ptr)
-    int32_t tiled_ok;         // every tile and halo fits the staged rows of k_sweep_tile32
-    const int32_t* tile_ptr;  // [n_tiles + 1]
-    const int32_t* halo_ptr;  // [n_tiles + 1]
-    const int32_t* halo;      // [halo_ptr[n_tiles]] nodes outside a tile its rows reference
+    int32_t n_blocks;         // node blocks (contiguous id ranges, HostMesh::blk_ptr)
+    int32_t blk_steps;        // most steps of the blocked solve per launch (layers around the blocks), 0 = not blocked
+    const int32_t* blk_ptr;   // [n_blocks + 1]
+    const int32_t* blk_cnt;   // [n_blocks][kBlockSteps + 1] nodes of a block and its first l layers
+    const int32_t* blk_halo_ptr; // [n_blocks + 1]
+    const int32_t* blk_halo;  // the layers' nodes, layer by layer
+    const int32_t* blk_row;   // [n_blocks + 1] first row of each block in the two tables below
+    const float* blk_val;     // per block [ell_w][rows] FP32 mass entries of the block and all layers but the last
+    const uint32_t* blk_col;  // per block [ell_w / 2][rows] the columns after the first as pairs of 16-bit indices
+                              // in the block's node list
     const float* ell_val;     // [ell_w][Np] FP32 mass entries (padding: own column, 0)
     const double* ell_lval;   // [ell_w][Np] patch-Laplacian coefficients of C (padding 0)
     int32_t iell_w;           // width of the ELL copy of node -> triangle incidence, 0 = none
@@ -154,8 +160,8 @@ struct Bufs {
     double* x1;      // [18][Np] they hold x64 (solution) and rho64 (residual)
     double* x64;     // alias of x0
     double* rho64;   // alias of x1
-    float* r32;      // [18][Np] FP32 residual of the current correction
-    float* e0;       // [18][Np] FP32 Chebyshev iterates
+    float* r32;      // [18 Np] FP32 residual of the current correction (layout: vec_at)
+    float* e0;       // [18 Np] FP32 iterates
     float* e1;
     // FP32-deviation storage (precision FELBM_FP32_DEV); C above stays FP64
     float* dpsi;     // deviations from equilibrium: [Np][16] rows (q = 1..8 of g, h), then [2][Np] (q = 0)
@@ -173,8 +179,66 @@ struct Bufs {
     double* diag_out;  // [kDiagSlots]
     double* Cdiag;     // [Np]
     unsigned* diag_done;   // blocks of k_diag_fused32 finished (0 between launches)
-    unsigned* kerr;        // error bits of the solve kernels (kErrTileWait); 0 at felbm_init
 };
+
+// The FP32 vectors of the solve (r32, e0, e1): the moving populations as four
+// planes of float4 [Np] (q = 1..4 and 5..8 of g, then of h), then the rest
+// populations of g and h as one plane of float2 [Np].  A gathered neighbour is
+// one 16-byte word per four right-hand sides.
+constexpr int kPlanes = 5;
+__device__ __forceinline__ size_t vec_at(int Np, int q18, int i) {
+    const int part = q18 >= 9 ? 1 : 0, q = q18 - 9 * part, s = part * 8 + q - 1;
+    return q == 0 ? (size_t)16 * Np + 2 * (size_t)i + part : ((size_t)(s >> 2) * Np + i) * 4 + (s & 3);
+}
+// q18 of component c of plane p
+__host__ __device__ constexpr int vec_row(int p, int c) {
+    return p == 4 ? 9 * c : 9 * (p >> 1) + 1 + 4 * (p & 1) + c;
+}
+// Plane p of node i as NV values (NV = 4 for p < 4, 2 for p = 4).
+template <int NV>
+__device__ __forceinline__ void load_vec(float (&v)[NV], const float* x, int Np, int p, int i) {
+    if constexpr (NV == 4) {
+        const float4 t = reinterpret_cast<const float4*>(x)[(size_t)p * Np + i];
+        v[0] = t.x;
+        v[1] = t.y;
+        v[2] = t.z;
+        v[3] = t.w;
+    } else {
+        const float2 t = reinterpret_cast<const float2*>(x + (size_t)16 * Np)[i];
+        v[0] = t.x;
+        v[1] = t.y;
+    }
+}
+template <int NV>
+__device__ __forceinline__ void store_vec(float* x, int Np, int p, int i, const float (&v)[NV]) {
+    if constexpr (NV == 4)
+        reinterpret_cast<float4*>(x)[(size_t)p * Np + i] = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        reinterpret_cast<float2*>(x + (size_t)16 * Np)[i] = make_float2(v[0], v[1]);
+}
+// All 18 values of node i, indexed by q18.
+__device__ __forceinline__ void load_all(float (&d)[18], const float* x, int Np, int i) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        float v[4];
+        load_vec(v, x, Np, p, i);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d[vec_row(p, c)] = v[c];
+    }
+    float v[2];
+    load_vec(v, x, Np, 4, i);
+    d[0] = v[0];
+    d[9] = v[1];
+}
+__device__ __forceinline__ void store_all(float* x, int Np, int i, const float (&d)[18]) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const float v[4] = {d[vec_row(p, 0)], d[vec_row(p, 1)], d[vec_row(p, 2)], d[vec_row(p, 3)]};
+        store_vec(x, Np, p, i, v);
+    }
+    const float v[2] = {d[0], d[9]};
+    store_vec(x, Np, 4, i, v);
+}
 
 constexpr int kBlock = 256;
 constexpr int kDiagBlocks = 608;   // fixed grid (4 x 152 SMs): the reduction order never changes
@@ -424,8 +488,8 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
     for (int q = 0; q < 18; ++q) {
         b.rhs[q * Np + i] = acc[q];
         if (kMixed) {
-            b.r32[q * Np + i] = (float)acc[q];
-            b.e1[q * Np + i] = (float)(acc[q] * s);
+            b.r32[vec_at(Np, q, i)] = (float)acc[q];
+            b.e1[vec_at(Np, q, i)] = (float)(acc[q] * s);
         } else {
             b.x1[q * Np + i] = acc[q] * s;
         }
@@ -444,8 +508,8 @@ __global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, double
     for (int q = 0; q < 18; ++q) {
         double r = b.rhs[q * Np + i];
         if (kMixed) {
-            b.r32[q * Np + i] = (float)r;
-            b.e1[q * Np + i] = (float)(r * s);
+            b.r32[vec_at(Np, q, i)] = (float)r;
+            b.e1[vec_at(Np, q, i)] = (float)(r * s);
         } else {
             b.x1[q * Np + i] = r * s;
         }
@@ -502,7 +566,8 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 
 #include "felbm_dev32.cuh"
 #include "felbm_adjoint.cuh"
-#include "felbm_tile32.cuh"
+
+#include "felbm_block32.cuh"
 
 // One step of the FP32 correction solve (CSR rows): Richardson iteration
 // x_{k+1} = x_k + tau_k m^{-1} (b - M x_k) with the Chebyshev step sizes
@@ -526,16 +591,16 @@ __global__ void __launch_bounds__(128) k_cheb32(DevMesh m, Phys c, Bufs b, const
         int j = m.col[k];
         float mv = m.mval32[k];
 #pragma unroll
-        for (int q = 0; q < 18; ++q) acc[q] = fmaf(mv, cur[q * Np + j], acc[q]);
+        for (int q = 0; q < 18; ++q) acc[q] = fmaf(mv, cur[vec_at(Np, q, j)], acc[q]);
     }
     float s = tau * m.inv_lumped32[i];
     float d[18];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        float xk = cur[q * Np + i];
-        float xn = fmaf(s, b.r32[q * Np + i] - acc[q], xk);
+        float xk = cur[vec_at(Np, q, i)];
+        float xn = fmaf(s, b.r32[vec_at(Np, q, i)] - acc[q], xk);
         if (kFinal == kStore) {
-            nxt[q * Np + i] = xn;
+            nxt[vec_at(Np, q, i)] = xn;
         } else if (kFinal == kUpdateDev) {
             d[q] = xn;
         } else {
@@ -554,89 +619,116 @@ __global__ void __launch_bounds__(128) k_cheb32(DevMesh m, Phys c, Bufs b, const
 // the predecessor's results before touching them.  Both instructions are
 // no-ops for a kernel launched without the attribute.
 
+// Planes [vec_first(parts, part), vec_first(parts, part + 1)) of the iterate
+// belong to one of the `parts` threads of a node (6 threads: five own a plane).
+__host__ __device__ constexpr int vec_first(int parts, int part) {
+    return parts == 6 ? (part < 5 ? part : 5) : kPlanes * part / parts;
+}
+
+// The planes [kP, kEnd) of one node's step; g: all gathered values are loaded
+// before the first product (more loads in flight per thread).
+template <int kP, int kEnd, int kFinal, int kW, bool kFromRhs>
+__device__ __forceinline__ void sweep_planes(const DevMesh& m, const Bufs& b, const float* __restrict__ cur, float* nxt,
+                                             int i, const int (&col)[kW], const float (&val)[kW],
+                                             const float (&sc)[kFromRhs ? kW : 1], float s, int have_x64,
+                                             float (&d)[18]) {
+    if constexpr (kP < kEnd) {
+        constexpr int NV = kP < 4 ? 4 : 2;
+        const int Np = m.Np;
+        float g[kW][NV], rr[NV];
+        const float* src = kFromRhs ? b.r32 : cur;
+#pragma unroll
+        for (int k = 0; k < kW; ++k) load_vec(g[k], src, Np, kP, col[k]);
+        if constexpr (kFromRhs) {
+            // the row's first column is the node itself
+#pragma unroll
+            for (int c = 0; c < NV; ++c) rr[c] = g[0][c];
+#pragma unroll
+            for (int k = 0; k < kW; ++k)
+#pragma unroll
+                for (int c = 0; c < NV; ++c) g[k][c] *= sc[k];
+        } else {
+            load_vec(rr, b.r32, Np, kP, i);
+        }
+        float xn[NV];
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+            float acc = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kW; ++k) acc = fmaf(val[k], g[k][c], acc);
+            xn[c] = fmaf(s, rr[c] - acc, g[0][c]);
+        }
+        if constexpr (kFinal == kStore) {
+            store_vec(nxt, Np, kP, i, xn);
+        } else if constexpr (kFinal == kUpdateDev) {
+#pragma unroll
+            for (int c = 0; c < NV; ++c) d[vec_row(kP, c)] = xn[c];
+        } else {
+#pragma unroll
+            for (int c = 0; c < NV; ++c) {
+                const int r = vec_row(kP, c) * Np + i;
+                const double x = have_x64 ? b.x64[r] + (double)xn[c] : (double)xn[c];
+                if (kFinal == kAddPsi)
+                    b.psi[r] += x;
+                else
+                    b.x64[r] = x;
+            }
+        }
+        sweep_planes<kP + 1, kEnd, kFinal, kW, kFromRhs>(m, b, cur, nxt, i, col, val, sc, s, have_x64, d);
+    }
+}
+
+template <int kPart, int kParts, int kFinal, int kW, bool kFromRhs>
+__device__ __forceinline__ void sweep_part(int part, const DevMesh& m, const Bufs& b, const float* __restrict__ cur,
+                                           float* nxt, int i, const int (&col)[kW], const float (&val)[kW],
+                                           const float (&sc)[kFromRhs ? kW : 1], float s, int have_x64, float (&d)[18]) {
+    if constexpr (kPart < kParts) {
+        if (part == kPart)
+            sweep_planes<vec_first(kParts, kPart), vec_first(kParts, kPart + 1), kFinal, kW, kFromRhs>(
+                m, b, cur, nxt, i, col, val, sc, s, have_x64, d);
+        else
+            sweep_part<kPart + 1, kParts, kFinal, kW, kFromRhs>(part, m, b, cur, nxt, i, col, val, sc, s, have_x64, d);
+    }
+}
+
 // The FP32 step of k_cheb32 on the ELL copy of the pattern (kW entries per
-// row, padded with the own column and value 0).  Row indices and values are
-// loaded up front (coalesced, column-major).
-// kParts threads per node, each owning 18/kParts of the node's rows (more
-// threads in flight for this latency-bound gather); the field update needs
-// all 18 in one thread.  The parts of one node block are consecutive blocks
-// (blockIdx.x = kParts * node block + part), so they run together and share
-// the block's matrix rows through L2 instead of fetching them from DRAM
-// once per part.
+// row, the node's own first, padded with the own column and value 0).  Row
+// indices and values are loaded up front (coalesced, column-major).
+// kParts threads per node, each owning some of the iterate's planes; the
+// field update needs all of them in one thread.  The parts of one node block
+// are consecutive blocks (blockIdx.x = kParts * node block + part), so they
+// run together and share the block's matrix rows through L2 instead of
+// fetching them from DRAM once per part.
 template <int kFinal, int kW, int kParts, bool kFromRhs = false>
 __global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, const float* __restrict__ cur,
                                                  float* nxt, float tau, int have_x64, float tau0) {
     pdl_release();
     static_assert(kFinal != kUpdateDev || kParts == 1, "the field update needs the whole node");
-    constexpr int NQ = 18 / kParts;
     const int nb = (int)blockIdx.x / kParts;
     const int i = nb * (int)blockDim.x + (int)threadIdx.x;
-    const int q0 = NQ * ((int)blockIdx.x - nb * kParts);
+    const int part = (int)blockIdx.x - nb * kParts;
     const int Np = m.Np;
-    static_assert(18 % kParts == 0, "parts must divide 18");
     int col[kW];
     float val[kW];
+    // kFromRhs: the first step of the solve, whose iterate x_0 = tau_0 b / m
+    // is formed here from the right-hand side (the RHS kernel stores b only)
+    float sc[kFromRhs ? kW : 1];
     if (i < m.N) {
 #pragma unroll
         for (int k = 0; k < kW; ++k) {
             col[k] = m.ell_col[k * Np + i];
             val[k] = m.ell_val[k * Np + i];
         }
-    }
-    const float s = tau * (i < m.N ? m.inv_lumped32[i] : 0.0f);
-    // kFromRhs: the first step of the solve, whose iterate x_0 = tau_0 b / m
-    // is formed here from the right-hand side (the RHS kernel stores b only)
-    float sc[kFromRhs ? kW : 1];
-    float s0 = 0.0f;
-    if constexpr (kFromRhs) {
-        if (i < m.N) {
+        if constexpr (kFromRhs) {
 #pragma unroll
             for (int k = 0; k < kW; ++k) sc[k] = m.inv_lumped32[col[k]] * tau0;
-            s0 = m.inv_lumped32[i] * tau0;
         }
     }
+    const float s = tau * (i < m.N ? m.inv_lumped32[i] : 0.0f);
     pdl_wait();
     if (i >= m.N) return;
-    // every gathered value is loaded before the first product (more loads in
-    // flight per thread for this latency-bound gather: 15 % faster sweeps on
-    // the 2.08M-node rough wall than interleaving loads and products)
-    float g[kW][NQ], xk[NQ], rr[NQ];
-    const float* src = kFromRhs ? b.r32 : cur;
-#pragma unroll
-    for (int k = 0; k < kW; ++k)
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) g[k][q] = src[(q0 + q) * Np + col[k]];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        rr[q] = b.r32[(q0 + q) * Np + i];
-        xk[q] = kFromRhs ? rr[q] * s0 : cur[(q0 + q) * Np + i];
-    }
-    if constexpr (kFromRhs) {
-#pragma unroll
-        for (int k = 0; k < kW; ++k)
-#pragma unroll
-            for (int q = 0; q < NQ; ++q) g[k][q] *= sc[k];
-    }
-    float d[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int k = 0; k < kW; ++k) acc = fmaf(val[k], g[k][q], acc);
-        const int r = (q0 + q) * Np + i;
-        float xn = fmaf(s, rr[q] - acc, xk[q]);
-        if (kFinal == kStore) {
-            nxt[r] = xn;
-        } else if (kFinal == kUpdateDev) {
-            d[q] = xn;
-        } else {
-            double x = have_x64 ? b.x64[r] + (double)xn : (double)xn;
-            if (kFinal == kAddPsi)
-                b.psi[r] += x;
-            else
-                b.x64[r] = x;
-        }
-    }
+    float d[18];
+    sweep_part<0, kParts, kFinal, kW, kFromRhs>(part, m, b, cur, nxt, i, col, val, sc, s, have_x64, d);
     if constexpr (kFinal == kUpdateDev) dev32_update(m, c, b, i, d);
 }
 
@@ -654,7 +746,7 @@ __global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* 
         int j = m.col[k];
         double mv = m.mval[k];
 #pragma unroll
-        for (int q = 0; q < 18; ++q) acc[q] += mv * (double)e[q * Np + j];
+        for (int q = 0; q < 18; ++q) acc[q] += mv * (double)e[vec_at(Np, q, j)];
     }
     double s = m.inv_lumped[i] * tau0;
 #pragma unroll
@@ -662,10 +754,10 @@ __global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* 
         double xo = first_round ? 0.0 : b.x64[q * Np + i];
         double ro = first_round ? b.rhs[q * Np + i] : b.rho64[q * Np + i];
         double rn = ro - acc[q];
-        b.x64[q * Np + i] = xo + (double)e[q * Np + i];
+        b.x64[q * Np + i] = xo + (double)e[vec_at(Np, q, i)];
         b.rho64[q * Np + i] = rn;
-        b.r32[q * Np + i] = (float)rn;
-        next_first[q * Np + i] = (float)(rn * s);
+        b.r32[vec_at(Np, q, i)] = (float)rn;
+        next_first[vec_at(Np, q, i)] = (float)(rn * s);
     }
 }
 
@@ -685,10 +777,10 @@ __global__ void __launch_bounds__(kBlock) k_solve_resid(DevMesh m, Bufs b, const
         const int k0 = m.row_ptr[i], k1 = m.row_ptr[i + 1];
         for (int q = 0; q < 18; ++q) {
             float acc = 0.0f;
-            for (int k = k0; k < k1; ++k) acc = fmaf(m.mval32[k], x[q * Np + m.col[k]], acc);
-            const float r = b.r32[q * Np + i] - acc;
+            for (int k = k0; k < k1; ++k) acc = fmaf(m.mval32[k], x[vec_at(Np, q, m.col[k])], acc);
+            const float r = b.r32[vec_at(Np, q, i)] - acc;
             rr += (double)r * (double)r;
-            const double bq = kRhs64 ? b.rhs[q * Np + i] : (double)b.r32[q * Np + i];
+            const double bq = kRhs64 ? b.rhs[q * Np + i] : (double)b.r32[vec_at(Np, q, i)];
             bb += bq * bq;
         }
     }
@@ -1065,26 +1157,26 @@ __device__ __forceinline__ void sweep32_node(const DevMesh& m, const Phys& c, co
             const int j = m.ell_col[k * Np + i];
             const float v = m.ell_val[k * Np + i];
 #pragma unroll
-            for (int q = 0; q < 18; ++q) acc[q] = fmaf(v, cur[q * Np + j], acc[q]);
+            for (int q = 0; q < 18; ++q) acc[q] = fmaf(v, cur[vec_at(Np, q, j)], acc[q]);
         }
     } else {
         for (int k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
             const int j = m.col[k];
             const float v = m.mval32[k];
 #pragma unroll
-            for (int q = 0; q < 18; ++q) acc[q] = fmaf(v, cur[q * Np + j], acc[q]);
+            for (int q = 0; q < 18; ++q) acc[q] = fmaf(v, cur[vec_at(Np, q, j)], acc[q]);
         }
     }
     const float s = tau * m.inv_lumped32[i];
     float d[18];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        float xk = cur[q * Np + i];
-        float xn = fmaf(s, b.r32[q * Np + i] - acc[q], xk);
+        float xk = cur[vec_at(Np, q, i)];
+        float xn = fmaf(s, b.r32[vec_at(Np, q, i)] - acc[q], xk);
         if (update)
             d[q] = xn;
         else
-            nxt[q * Np + i] = xn;
+            nxt[vec_at(Np, q, i)] = xn;
     }
     if (update) dev32_update(m, c, b, i, d);
 }
@@ -1192,11 +1284,10 @@ struct felbm_state {
     bool dev32 = false;   // FELBM_FP32_DEV storage
     bool use_pdl = true;  // programmatic dependent launch between solve sweeps
     int sweep_parts = 2;  // threads per node of the FP32 store sweeps (1, 2, 3, 6)
-    bool sweep_tiled = false;  // store sweeps stage each node tile in shared memory (k_sweep_tile32)
+    bool sweep_tiled = false;  // the solve runs several steps of a node block per launch (k_block32)
     bool check = false;        // felbm_solver_check: residual of every solve before its last step
     double check_tol = 0.0;
-    int n_sm = 1;              // multiprocessors of the device (grid of the persistent tiled step)
-    int smem_optin = 0;        // largest dynamic shared memory a block may opt into
+    int n_sm = 1;              // multiprocessors of the device
     felbm::GroupTables gt{};
     felbm::AdjBufs adj{};         // adjoint buffers (FP64 states)
     std::vector<double> gmass0;   // per-group mass at felbm_init
@@ -1204,7 +1295,7 @@ struct felbm_state {
     // CTA each (k_step_cta32); the rest, a prefix of the node and triangle
     // ranges, run the tiled kernels.  cta_max_nodes = 0: tiled only.
     int32_t cta_max_nodes = 0;
-    int32_t n_cta = 0, tiled_N = 0, tiled_T = 0;
+    int32_t n_cta = 0, tiled_N = 0, tiled_T = 0, tiled_blocks = 0;
     int32_t* d_cta_groups = nullptr;   // [G] in the workspace
     cudaStream_t side_stream = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -1235,6 +1326,27 @@ static int inc_width(const HostMesh& h) {
     return 0;
 }
 
+// Meshes felbm_sweep_tiled takes: an ELL width with a compiled blocked solve (a
+// thread keeps its nodes' rows in registers; 16 entries do not fit) and tiles
+// whose first layer is small.
+static bool tiled_ok(const HostMesh& h, int ell_w) {
+    return (ell_w == 7 || ell_w == 9 || ell_w == 12) && h.max_halo <= kHaloMax;
+}
+
+// Rows of the blocked solve's tables: per block its own nodes and all layers
+// but the last, rounded up to 32.  first (blocks + 1 entries): where each
+// block's rows start.
+static int64_t block_rows(const HostMesh& h, int32_t* first) {
+    const int32_t nb = (int32_t)h.blk_ptr.size() - 1;
+    int64_t rows = 0;
+    for (int32_t t = 0; t < nb; ++t) {
+        if (first) first[t] = (int32_t)rows;
+        rows += (h.layer_cnt[(size_t)t * (kBlockSteps + 1) + h.n_layers - 1] + 31) & ~31;
+    }
+    if (first) first[nb] = (int32_t)rows;
+    return rows;
+}
+
 // Layout of the workspace; with base == nullptr only the size is computed.
 static size_t carve(const HostMesh& h, bool dev32, void* base, DevMesh* dm, Bufs* b,
                     GroupTables* gtab = nullptr, AdjBufs* adj = nullptr) {
@@ -1259,13 +1371,17 @@ static size_t carve(const HostMesh& h, bool dev32, void* base, DevMesh* dm, Bufs
     const int ellw = ell_width(h);
     d.ell_w = ellw;
     d.ell_col = cv.take<int32_t>((size_t)std::max(ellw, 1) * Np);
-    d.ell_loc = cv.take<uint16_t>((size_t)std::max(ellw, 1) * Np);
     d.ell_val = cv.take<float>((size_t)std::max(ellw, 1) * Np);
-    d.n_tiles = (int32_t)h.tile_ptr.size() - 1;
-    d.tiled_ok = ellw > 0 && h.max_halo <= kHaloMax;
-    d.tile_ptr = cv.take<int32_t>(h.tile_ptr.size());
-    d.halo_ptr = cv.take<int32_t>(h.halo_ptr.size());
-    d.halo = cv.take<int32_t>(std::max<size_t>(h.halo.size(), 1));
+    d.n_blocks = (int32_t)h.blk_ptr.size() - 1;
+    d.blk_steps = tiled_ok(h, ellw) ? h.n_layers : 0;
+    const size_t brows = d.blk_steps > 0 ? (size_t)block_rows(h, nullptr) : 1;
+    d.blk_ptr = cv.take<int32_t>(h.blk_ptr.size());
+    d.blk_cnt = cv.take<int32_t>(h.layer_cnt.size());
+    d.blk_halo_ptr = cv.take<int32_t>(h.halo_ptr.size());
+    d.blk_halo = cv.take<int32_t>(std::max<size_t>(h.halo.size(), 1));
+    d.blk_row = cv.take<int32_t>(h.blk_ptr.size());
+    d.blk_val = cv.take<float>(brows * std::max(ellw, 1));
+    d.blk_col = cv.take<uint32_t>(brows * std::max(ellw / 2, 1));
     d.ell_lval = cv.take<double>((size_t)std::max(ellw, 1) * Np);
     const int iw = inc_width(h);
     d.iell_w = iw;
@@ -1330,7 +1446,6 @@ static size_t carve(const HostMesh& h, bool dev32, void* base, DevMesh* dm, Bufs
     bb.diag_out = cv.take<double>(kDiagSlots);
     bb.Cdiag = cv.take<double>(Np);
     bb.diag_done = cv.take<unsigned>(1);
-    bb.kerr = cv.take<unsigned>(1);
     GroupTables g{};
     const size_t G = std::max<int32_t>(h.G, 1);
     g.node_begin = cv.take<int32_t>(G);
@@ -1405,11 +1520,12 @@ static unsigned grid_for(int n, int block) { return (unsigned)((n + block - 1) /
 
 // Launch with or without programmatic dependent launch (PDL).
 template <typename... KArgs, typename... Args>
-static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, Args&&... args) {
+static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                     Args&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1419,93 +1535,67 @@ static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, cu
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// One FP32 Chebyshev sweep: the ELL kernel of the mesh's width, else CSR.
-// pdl: the previous launch on the stream is a sweep (a kernel that waits).
-// parts: threads per node for the store sweeps (1, 2, 3 or 6; autotuned).
-// The tiled store step (k_sweep_tile32): a persistent grid of one block per
-// SM walking the (tile, part) items through its pipeline stages.
-template <int kW, int kParts>
-static void launch_tile_w(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                          float* nxt, float tau, bool pdl) {
-    cudaLaunchConfig_t cfg{};
-    const int items = m.n_tiles * kParts;
-    cfg.gridDim = dim3((unsigned)std::min(items, st->n_sm));
-    cfg.blockDim = dim3(kTileThreads);
-    cfg.dynamicSmemBytes = tile_stages(18 / kParts, kW) * tile_stage_bytes(18 / kParts, kW);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    if constexpr (tile_stages(18 / kParts, kW) >= 2) cudaLaunchKernelEx(&cfg, k_sweep_tile32<kW, kParts>, m, b, cur, nxt, tau);
+// One blocked launch: K steps from cur (or from b) to nxt or the final
+// destination.  All planes of a block in one thread block; one plane each
+// where that would leave multiprocessors idle.
+template <int kFinal, int kW, bool kFromRhs>
+static void launch_block_w(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
+                           float* nxt, const BlockTau& bt, int K, float tau0, int have_x64, bool pdl) {
+    const int ny = m.n_blocks >= kSplitPlanesBelow * st->n_sm ? 1 : kPlanes;
+    launch_k(pdl, k_block32<kW, kFinal, kFromRhs>, dim3((unsigned)m.n_blocks, ny), dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur,
+             nxt, bt, K, tau0, have_x64);
 }
 
-// Parts of the 18 right-hand sides per work item of the tiled step: 3 if
-// requested (1, 2 or 3) and two or more stages fit the shared memory of a
-// block, else 6; 0 if not even that fits.
-static bool tile_fits(int parts, int ell_w, int smem_optin) {
-    const int nq = 18 / parts;
-    return tile_stages(nq, ell_w) >= 2 &&
-           tile_stages(nq, ell_w) * tile_stage_bytes(nq, ell_w) + 1024 <= (size_t)smem_optin;
-}
-static int tile_parts(const felbm_state* st, int ell_w) {
-    for (int p : {3, 6})
-        if (p >= st->sweep_parts && tile_fits(p, ell_w, st->smem_optin)) return p;
-    return 0;
+template <int kFinal, bool kFromRhs>
+static void launch_block(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
+                         float* nxt, const BlockTau& bt, int K, float tau0, int have_x64, bool pdl) {
+    pdl = pdl && st->use_pdl;
+    switch (m.ell_w) {
+        case 7: launch_block_w<kFinal, 7, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl); break;
+        case 9: launch_block_w<kFinal, 9, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl); break;
+        default: launch_block_w<kFinal, 12, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl);
+    }
 }
 
+// Shared memory beyond the default 48 KB for the blocked kernels.
 template <int kW>
-static void launch_tile(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                        float* nxt, float tau, bool pdl) {
-    if (tile_parts(st, kW) == 3)
-        launch_tile_w<kW, 3>(st, m, b, s, cur, nxt, tau, pdl);
-    else
-        launch_tile_w<kW, 6>(st, m, b, s, cur, nxt, tau, pdl);
-}
-
-// Shared memory beyond the default 48 KB for the tiled steps that fit.
-template <int kW>
-static cudaError_t allow_tile_smem(int smem_optin) {
+static cudaError_t allow_block_smem() {
     cudaError_t e = cudaSuccess;
-    auto set = [&](auto kern, int parts) {
-        const size_t bytes = tile_stages(18 / parts, kW) * tile_stage_bytes(18 / parts, kW);
-        if (e == cudaSuccess && tile_fits(parts, kW, smem_optin))
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const auto set = [&](auto kern) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSmem));
     };
-    if constexpr (tile_stages(6, kW) >= 2) set(k_sweep_tile32<kW, 3>, 3);
-    if constexpr (tile_stages(3, kW) >= 2) set(k_sweep_tile32<kW, 6>, 6);
+    set(k_block32<kW, kStore, false>);
+    set(k_block32<kW, kStore, true>);
+    set(k_block32<kW, kAddPsi, false>);
+    set(k_block32<kW, kAddX64, false>);
     return e;
 }
 
+// One FP32 Chebyshev sweep: the ELL kernel of the mesh's width, else CSR.
+// pdl: the previous launch on the stream is a sweep (a kernel that waits).
+// parts: threads per node for the store sweeps (1, 2, 3 or 6; autotuned).
 template <int kFinal, int kW>
 static void launch_sweep_w(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
                            float* nxt, float tau, int have_x64, bool pdl) {
-    if constexpr (kFinal == kStore) {
-        // the tiled form covers whole meshes (not the tiled prefix of a hybrid batch schedule)
-        if (st->sweep_tiled && m.tiled_ok && m.N == st->dm.N && tile_parts(st, kW) > 0) {
-            launch_tile<kW>(st, m, b, s, cur, nxt, tau, pdl);
-            return;
-        }
-    }
     const dim3 block(128);
     const int parts = kFinal == kUpdateDev ? 1 : st->sweep_parts;
     const dim3 grid(grid_for(m.N, 128) * parts);
     switch (parts) {
         case 1:
-            launch_k(pdl, k_sweep32<kFinal, kW, 1>, grid, block, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
+            launch_k(pdl, k_sweep32<kFinal, kW, 1>, grid, block, 0, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
             break;
         case 3:
             if constexpr (kFinal != kUpdateDev)
-                launch_k(pdl, k_sweep32<kFinal, kW, 3>, grid, block, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
+                launch_k(pdl, k_sweep32<kFinal, kW, 3>, grid, block, 0, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
             break;
         case 6:
             if constexpr (kFinal != kUpdateDev)
-                launch_k(pdl, k_sweep32<kFinal, kW, 6>, grid, block, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
+                launch_k(pdl, k_sweep32<kFinal, kW, 6>, grid, block, 0, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
             break;
         default:
             if constexpr (kFinal != kUpdateDev)
-                launch_k(pdl, k_sweep32<kFinal, kW, 2>, grid, block, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
+                launch_k(pdl, k_sweep32<kFinal, kW, 2>, grid, block, 0, s, m, st->phys, b, cur, nxt, tau, have_x64, 0.0f);
     }
 }
 
@@ -1543,10 +1633,10 @@ static void launch_first_w(felbm_state* st, const DevMesh& m, const Bufs& b, cud
     const int parts = st->sweep_parts;
     const dim3 grid(grid_for(m.N, 128) * parts);
     switch (parts) {
-        case 1: launch_k(pdl, k_sweep32<kStore, kW, 1, true>, grid, block, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
-        case 3: launch_k(pdl, k_sweep32<kStore, kW, 3, true>, grid, block, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
-        case 6: launch_k(pdl, k_sweep32<kStore, kW, 6, true>, grid, block, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
-        default: launch_k(pdl, k_sweep32<kStore, kW, 2, true>, grid, block, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0);
+        case 1: launch_k(pdl, k_sweep32<kStore, kW, 1, true>, grid, block, 0, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
+        case 3: launch_k(pdl, k_sweep32<kStore, kW, 3, true>, grid, block, 0, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
+        case 6: launch_k(pdl, k_sweep32<kStore, kW, 6, true>, grid, block, 0, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0); break;
+        default: launch_k(pdl, k_sweep32<kStore, kW, 2, true>, grid, block, 0, s, m, st->phys, b, nullptr, nxt, tau, 0, tau0);
     }
 }
 
@@ -1562,12 +1652,50 @@ static void launch_first(felbm_state* st, const DevMesh& m, const Bufs& b, cudaS
     }
 }
 
+// Whether the solve on m runs blocked.
+static bool blocked(const felbm_state* st, const DevMesh& m) { return st->sweep_tiled && m.blk_steps > 0; }
+
+// The steps [k, end) of one correction in as few blocked launches as the
+// layers allow, of about equal length; the last goes to `final` unless it is
+// kStore.  Returns the buffer with the last stored iterate.
+static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, float* cur, float* prv,
+                              int k, int end, int final, int have_x64, bool from_rhs, bool pdl) {
+    int left = (end - k + m.blk_steps - 1) / m.blk_steps;
+    for (; left > 0; --left) {
+        const int K = (end - k + left - 1) / left;
+        BlockTau bt{};
+        for (int j = 0; j < K; ++j) bt.tau[j] = (float)st->tau[k + j];
+        const float tau0 = (float)st->tau[0];
+        if (from_rhs)
+            launch_block<kStore, true>(st, m, b, s, nullptr, prv, bt, K, tau0, have_x64, pdl);
+        else if (left > 1 || final == kStore)
+            launch_block<kStore, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
+        else if (final == kAddPsi)
+            launch_block<kAddPsi, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
+        else
+            launch_block<kAddX64, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
+        from_rhs = false;
+        pdl = true;
+        k += K;
+        std::swap(cur, prv);
+    }
+    return cur;
+}
+
+// The checked solve's residual of the iterate cur (felbm_solver_check).
+static void enqueue_resid(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur) {
+    if (st->dev32)
+        k_solve_resid<false><<<kDiagBlocks, kBlock, 0, s>>>(m, b, cur, b.diag_part);
+    else
+        k_solve_resid<true><<<kDiagBlocks, kBlock, 0, s>>>(m, b, cur, b.diag_part);
+    k_solve_resid_final<<<1, 1, 0, s>>>(b.diag_part, kDiagBlocks, b.diag_out + kSolveResSlot);
+}
+
 // Whether the FP32 time step forms x_0 inside its first solve step (then the
 // RHS kernel stores b only): one correction round, gathered steps, at least
 // two steps after the first, no residual check, an ELL width with kernels.
 static bool first_from_rhs(const felbm_state* st, const DevMesh& m) {
-    return st->dev32 && st->rounds == 1 && st->sweeps > 2 && !st->check && !st->sweep_tiled &&
-           gathered_width(m.ell_w);
+    return st->dev32 && st->rounds == 1 && st->sweeps > 2 && !st->check && (blocked(st, m) || gathered_width(m.ell_w));
 }
 
 // Enqueue the mass solve for the right-hand side in b.rhs (first iterate
@@ -1595,17 +1723,32 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
     for (int r = 0; r < st->rounds; ++r) {
         float* cur = A;
         float* prv = B;
-        for (int k = 1; k < st->sweeps; ++k) {
+        const bool last_round = r == st->rounds - 1;
+        if (blocked(st, m)) {
+            const int final = !last_round || (into_psi && st->dev32) ? kStore : (into_psi ? kAddPsi : kAddX64);
+            bool pdl = r == 0 && after_release;
+            int k = 1;
+            if (last_round && st->check) {
+                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, kStore, have_x64, false, pdl);
+                prv = x == cur ? prv : cur;
+                cur = x;
+                enqueue_resid(st, m, b, s, cur);
+                k = st->sweeps - 1;
+                pdl = false;
+            }
+            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, final, have_x64, from_rhs && r == 0, pdl);
+            prv = x == cur ? prv : cur;
+            cur = x;
+            if (last_round && into_psi && st->dev32)
+                launch_k(st->use_pdl, k_update32, dim3(grid_for(m.N, 128)), dim3(128), 0, s, m, st->phys, b, (const float*)cur);
+        }
+        for (int k = 1; k < st->sweeps && !blocked(st, m); ++k) {
             const float tau = (float)st->tau[k];
-            const bool last = r == st->rounds - 1 && k == st->sweeps - 1;
+            const bool last = last_round && k == st->sweeps - 1;
             // the previous launch is a sweep of this round, or a kernel that released its dependents
             bool pdl = k > 1 || (k == 1 && r == 0 && after_release);
             if (last && st->check) {
-                if (st->dev32)
-                    k_solve_resid<false><<<kDiagBlocks, kBlock, 0, s>>>(m, b, cur, b.diag_part);
-                else
-                    k_solve_resid<true><<<kDiagBlocks, kBlock, 0, s>>>(m, b, cur, b.diag_part);
-                k_solve_resid_final<<<1, 1, 0, s>>>(b.diag_part, kDiagBlocks, b.diag_out + kSolveResSlot);
+                enqueue_resid(st, m, b, s, cur);
                 pdl = false;
             }
             if (from_rhs && r == 0 && k == 1)
@@ -1620,7 +1763,7 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
                 launch_sweep<kAddPsi>(st, m, b, s, cur, prv, tau, have_x64, pdl);
             std::swap(cur, prv);
         }
-        if (r < st->rounds - 1) {
+        if (!last_round) {
             k_refine<<<grid, 128, 0, s>>>(m, b, cur, prv, r == 0, st->tau[0]);
             A = prv;
             B = cur;
@@ -1630,8 +1773,13 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
 }
 
 static int solve_launches(const felbm_state* st) {
-    return st->mode == FELBM_SOLVER_FP64 ? st->sweeps - 1
-                                         : st->rounds * (st->sweeps - 1) + (st->rounds - 1);
+    if (st->mode == FELBM_SOLVER_FP64) return st->sweeps - 1;
+    const int refines = st->rounds - 1;
+    if (!blocked(st, st->dm)) return st->rounds * (st->sweeps - 1) + refines;
+    const int most = st->dm.blk_steps;
+    const auto groups = [&](int steps) { return (steps + most - 1) / most; };
+    const int last = st->check ? groups(st->sweeps - 2) + 1 : groups(st->sweeps - 1);
+    return refines * (groups(st->sweeps - 1) + 1) + last + (st->dev32 ? 1 : 0);
 }
 
 static int step_launches(const felbm_state* st) { return (st->dev32 ? 4 : 5) + solve_launches(st); }
@@ -1662,6 +1810,7 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
         DevMesh mt = m;
         mt.N = st->tiled_N;
         mt.T = st->tiled_T;
+        mt.n_blocks = st->tiled_blocks;
         // collision is folded into the element, RHS and update kernels
         mark(1);
         if (mt.N > 0) {
@@ -1677,27 +1826,27 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
             }
             mark(2);
             if (st->phys.lapmu_nodal)
-                launch_k(chain, k_lmu32, dim3(grid_for(mt.N, kBlock)), dim3(kBlock), s, mt, st->phys, b);
+                launch_k(chain, k_lmu32, dim3(grid_for(mt.N, kBlock)), dim3(kBlock), 0, s, mt, st->phys, b);
             else
-                launch_k(chain, k_gradmu32, dim3(grid_for(mt.T, kBlock)), dim3(kBlock), s, mt, b);
+                launch_k(chain, k_gradmu32, dim3(grid_for(mt.T, kBlock)), dim3(kBlock), 0, s, mt, b);
             mark(3);
-            launch_k(chain, k_element32, dim3(grid_for(mt.T, 128)), dim3(128), s, mt, st->phys, b);
+            launch_k(chain, k_element32, dim3(grid_for(mt.T, 128)), dim3(128), 0, s, mt, st->phys, b);
             mark(4);
             const bool from_rhs = first_from_rhs(st, mt);
             const float tau0 = (float)st->tau[0];
             const dim3 gn(grid_for(mt.N, 128)), bn(128);
             switch (mt.iell_w * 2 + (from_rhs ? 1 : 0)) {
-                case 12: launch_k(chain, k_rhs32<6, true>, gn, bn, s, mt, st->phys, b, tau0); break;
-                case 13: launch_k(chain, k_rhs32<6, false>, gn, bn, s, mt, st->phys, b, tau0); break;
-                case 16: launch_k(chain, k_rhs32<8, true>, gn, bn, s, mt, st->phys, b, tau0); break;
-                case 17: launch_k(chain, k_rhs32<8, false>, gn, bn, s, mt, st->phys, b, tau0); break;
-                case 24: launch_k(chain, k_rhs32<12, true>, gn, bn, s, mt, st->phys, b, tau0); break;
-                case 25: launch_k(chain, k_rhs32<12, false>, gn, bn, s, mt, st->phys, b, tau0); break;
+                case 12: launch_k(chain, k_rhs32<6, true>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
+                case 13: launch_k(chain, k_rhs32<6, false>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
+                case 16: launch_k(chain, k_rhs32<8, true>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
+                case 17: launch_k(chain, k_rhs32<8, false>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
+                case 24: launch_k(chain, k_rhs32<12, true>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
+                case 25: launch_k(chain, k_rhs32<12, false>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
                 default:
                     if (from_rhs)
-                        launch_k(chain, k_rhs32<0, false>, gn, bn, s, mt, st->phys, b, tau0);
+                        launch_k(chain, k_rhs32<0, false>, gn, bn, 0, s, mt, st->phys, b, tau0);
                     else
-                        launch_k(chain, k_rhs32<0, true>, gn, bn, s, mt, st->phys, b, tau0);
+                        launch_k(chain, k_rhs32<0, true>, gn, bn, 0, s, mt, st->phys, b, tau0);
             }
             mark(5);
             enqueue_solve(st, mt, st->buf, s, true, chain, from_rhs);
@@ -1851,44 +2000,68 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
         for (int32_t k = h.row_ptr[i]; k < h.row_ptr[i + 1]; ++k) lval[k] = -2.0 * h.stiff[k] * inv_vol[i];
     }
     for (int32_t i = 0; i < h.N && ellw > 0; ++i) {
-        int32_t r0 = h.row_ptr[i], len = h.row_ptr[i + 1] - r0;
-        for (int k = 0; k < ellw; ++k) {
-            size_t at = (size_t)k * st->dm.Np + i;
-            ell_col[at] = k < len ? h.col[r0 + k] : i;
-            ell_val[at] = k < len ? (float)h.mass[r0 + k] : 0.0f;
-            ell_lval[at] = k < len ? lval[r0 + k] : 0.0;
+        // the diagonal first (the solve steps hold the node's own value already),
+        // then the other columns in order
+        const int32_t r0 = h.row_ptr[i], len = h.row_ptr[i + 1] - r0;
+        int at_k = 1;
+        for (int k = 0; k < len; ++k) {
+            const int32_t c = h.col[r0 + k];
+            const size_t at = (size_t)(c == i ? 0 : at_k++) * st->dm.Np + i;
+            ell_col[at] = c;
+            ell_val[at] = (float)h.mass[r0 + k];
+            ell_lval[at] = lval[r0 + k];
         }
+        for (int k = len; k < ellw; ++k) ell_col[(size_t)k * st->dm.Np + i] = i;
     }
-    // the ELL columns as indices into the staged row of the node's tile:
-    // [0, span) the 16-byte aligned run a0 = tile start rounded down to 4,
-    // then the tile's halo in its sorted order
-    std::vector<uint16_t> ell_loc((size_t)std::max(ellw, 1) * st->dm.Np, 0);
-    if (st->dm.tiled_ok) {
-        const int32_t ntile = st->dm.n_tiles;
-        for (int32_t t = 0; t < ntile; ++t) {
-            const int32_t s0 = h.tile_ptr[t], s1 = h.tile_ptr[t + 1], a0 = s0 & ~3;
-            const int32_t span = ((s1 + 3) & ~3) - a0;
-            const int32_t* hb = h.halo.data() + h.halo_ptr[t];
-            const int32_t* he = h.halo.data() + h.halo_ptr[t + 1];
-            for (int32_t i = s0; i < s1; ++i)
+    // the blocked solve's rows: a block's node list is its own run, then its
+    // layers; every node but the last layer's gets its ELL row with columns as
+    // indices into that list (padding: the node itself with entry 0)
+    const int32_t nblk = st->dm.n_blocks;
+    std::vector<int32_t> blk_row(nblk + 1, 0);
+    std::vector<float> blk_val;
+    std::vector<uint32_t> blk_col;
+    if (st->dm.blk_steps > 0) {
+        const int wc = ellw / 2;
+        const int64_t rows = block_rows(h, blk_row.data());
+        blk_val.assign((size_t)rows * ellw, 0.0f);
+        blk_col.assign((size_t)rows * wc, 0);
+        std::atomic<int> stray{0};
+        const int32_t Np = st->dm.Np;
+        struct Index {
+            std::vector<int32_t> blk, at;      // a node's index in the list of the block that saw it last
+        };
+        const auto make = [&]() { return Index{std::vector<int32_t>(h.N, -1), std::vector<int32_t>(h.N)}; };
+        parallel_for(nblk, 32, make, [&](int32_t t, Index& ix) {
+            const int32_t s0 = h.blk_ptr[t], ni = h.blk_ptr[t + 1] - s0;
+            const int32_t* cnt = h.layer_cnt.data() + (size_t)t * (kBlockSteps + 1);
+            const int32_t* halo = h.halo.data() + h.halo_ptr[t];
+            const int32_t nr = cnt[h.n_layers - 1], stride = blk_row[t + 1] - blk_row[t];
+            float* val = blk_val.data() + (size_t)ellw * blk_row[t];
+            uint32_t* col = blk_col.data() + (size_t)wc * blk_row[t];
+            for (int32_t r = 0; r < cnt[h.n_layers]; ++r) {
+                const int32_t i = r < ni ? s0 + r : halo[r - ni];
+                ix.blk[i] = t;
+                ix.at[i] = r;
+            }
+            for (int32_t r = 0; r < nr; ++r) {
+                const int32_t i = r < ni ? s0 + r : halo[r - ni];
                 for (int k = 0; k < ellw; ++k) {
-                    const size_t at = (size_t)k * st->dm.Np + i;
-                    const int32_t c = ell_col[at];
-                    int32_t loc;
-                    if (c >= s0 && c < s1) {
-                        loc = c - a0;
-                    } else {
-                        const int32_t* f = std::lower_bound(hb, he, c);
-                        if (f == he || *f != c) {
-                            set_error("felbm_init: internal error, a row entry outside its tile's halo");
-                            delete st;
-                            return FELBM_ERR_BAD_MESH;
-                        }
-                        loc = span + (int32_t)(f - hb);
-                    }
-                    ell_loc[at] = (uint16_t)loc;
+                    val[(size_t)k * stride + r] = ell_val[(size_t)k * Np + i];
+                    if (k == 0) continue;
+                    const int32_t c = ell_col[(size_t)k * Np + i];
+                    if (ix.blk[c] != t) stray = 1;
+                    const uint32_t at = ix.blk[c] == t ? (uint32_t)ix.at[c] : (uint32_t)r;
+                    uint32_t& pair = col[(size_t)((k - 1) / 2) * stride + r];
+                    pair = (k & 1) ? at | (uint32_t)r << 16 : (pair & 0xffffu) | at << 16;
                 }
+            }
+        });
+        if (stray) {
+            set_error("felbm_init: internal error, a row entry outside its block's layers");
+            delete st;
+            return FELBM_ERR_BAD_MESH;
         }
+        st->sweep_tiled = st->mode != FELBM_SOLVER_FP64;
     }
     auto pad_tri = [&](const std::vector<int32_t>& src, int rows) {
         std::vector<int32_t> outv((size_t)rows * st->dm.Tp, 0);
@@ -1933,23 +2106,21 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     UP(d.mval32, mval32);
     UP(d.ell_col, ell_col);
     UP(d.ell_val, ell_val);
-    UP(d.ell_loc, ell_loc);
-    UP(d.tile_ptr, h.tile_ptr);
-    UP(d.halo_ptr, h.halo_ptr);
-    UP(d.halo, h.halo);
-    if (e == cudaSuccess) e = cudaMemsetAsync(st->buf.kerr, 0, sizeof(unsigned), s);
+    UP(d.blk_ptr, h.blk_ptr);
+    UP(d.blk_cnt, h.layer_cnt);
+    UP(d.blk_halo_ptr, h.halo_ptr);
+    UP(d.blk_halo, h.halo);
+    UP(d.blk_row, blk_row);
+    UP(d.blk_val, blk_val);
+    UP(d.blk_col, blk_col);
     int cur_dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&cur_dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&st->n_sm, cudaDevAttrMultiProcessorCount, cur_dev);
-    if (e == cudaSuccess)
-        e = cudaDeviceGetAttribute(&st->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, cur_dev);
-    if (e == cudaSuccess && st->dm.tiled_ok) {
+    if (e == cudaSuccess && st->dm.blk_steps > 0) {
         switch (ellw) {
-            case 7: e = allow_tile_smem<7>(st->smem_optin); break;
-            case 9: e = allow_tile_smem<9>(st->smem_optin); break;
-            case 12: e = allow_tile_smem<12>(st->smem_optin); break;
-            case 16: e = allow_tile_smem<16>(st->smem_optin); break;
-            default: break;
+            case 7: e = allow_block_smem<7>(); break;
+            case 9: e = allow_block_smem<9>(); break;
+            default: e = allow_block_smem<12>();
         }
     }
     UP(d.ell_lval, ell_lval);
@@ -2094,6 +2265,7 @@ int set_schedule(felbm_state* st, int32_t max_nodes) {
     st->n_cta = (int32_t)cta.size();
     st->tiled_N = tiled_N;
     st->tiled_T = tiled_T;
+    st->tiled_blocks = (int32_t)(std::upper_bound(h.blk_ptr.begin(), h.blk_ptr.end(), tiled_N) - h.blk_ptr.begin()) - 1;
     return FELBM_OK;
 }
 
@@ -2286,19 +2458,6 @@ static felbm_diag fill_diag(const felbm_state* st, const double* v, double mass0
 
 extern "C" {
 
-// Error bits the solve kernels left since felbm_init (read after the stream
-// has been synchronised by the caller of this check).
-static int solve_status(felbm_state* st, const char* who) {
-    unsigned bits = 0;
-    FELBM_CUDA(cudaMemcpyAsync(&bits, st->buf.kerr, sizeof bits, cudaMemcpyDeviceToHost, st->stream));
-    FELBM_CUDA(cudaStreamSynchronize(st->stream));
-    if (bits & kErrTileWait) {
-        set_error(std::string(who) + ": a tiled solve step gave up waiting for its tile copy");
-        return FELBM_ERR_CUDA;
-    }
-    return FELBM_OK;
-}
-
 int felbm_diagnostics(felbm_state* st, const felbm_diag_request* req, felbm_diag* out) {
     if (!st || !out) {
         set_error("felbm_diagnostics: invalid argument");
@@ -2311,7 +2470,6 @@ int felbm_diagnostics(felbm_state* st, const felbm_diag_request* req, felbm_diag
     double v[kDiagSlots];
     FELBM_CUDA(cudaMemcpyAsync(v, st->buf.diag_out, sizeof v, cudaMemcpyDeviceToHost, s));
     FELBM_CUDA(cudaStreamSynchronize(s));
-    if (int rc = solve_status(st, "felbm_diagnostics")) return rc;
     *out = fill_diag(st, v, st->mass0, st->hm.N, rq.substrate, nullptr, st->hm.E, st->step, v + kSolveResSlot);
     if (out->status == FELBM_ERR_NOT_CONVERGED) {
         set_error("felbm_diagnostics: the last solve's residual is above the tolerance of felbm_solver_check");
@@ -2419,7 +2577,7 @@ int felbm_get_state(felbm_state* st, double* g, double* h) {
     FELBM_CUDA(cudaMemcpyAsync(g, st->buf.stage, sizeof(double) * 9 * N, cudaMemcpyDeviceToHost, s));
     FELBM_CUDA(cudaMemcpyAsync(h, st->buf.stage + (size_t)9 * N, sizeof(double) * 9 * N, cudaMemcpyDeviceToHost, s));
     FELBM_CUDA(cudaStreamSynchronize(s));
-    return solve_status(st, "felbm_get_state");
+    return FELBM_OK;
 }
 
 int felbm_set_state(felbm_state* st, const double* g, const double* h) {
@@ -2638,9 +2796,9 @@ int felbm_sweep_tiled(felbm_state* st, int32_t on) {
         set_error("felbm_sweep_tiled: invalid argument (0 or 1)");
         return FELBM_ERR_INVALID_ARG;
     }
-    if (on && (!st->dm.tiled_ok || tile_parts(st, st->dm.ell_w) == 0)) {
-        set_error("felbm_sweep_tiled: this mesh has no ELL copy, a tile halo beyond the staged rows, or "
-                  "rows too long for two pipeline stages in shared memory");
+    if (on && !tiled_ok(st->hm, st->dm.ell_w)) {
+        set_error("felbm_sweep_tiled: this mesh has no ELL copy, rows of more than 12 entries, or a tile "
+                  "with more than 504 nodes in its first layer");
         return FELBM_ERR_UNSUPPORTED;
     }
     FELBM_CUDA(cudaStreamSynchronize(st->stream));
@@ -2707,12 +2865,11 @@ int felbm_autotune(felbm_state* st, int32_t trials, felbm_tune_result* out) {
     if (st->mode != FELBM_SOLVER_FP64 && st->dm.ell_w > 0) {
         rc = set_schedule(st, 0);
         for (int tiled = 0; tiled < 2 && rc == FELBM_OK; ++tiled) {
-            if (tiled && !st->dm.tiled_ok) break;
+            if (tiled && st->dm.blk_steps == 0) break;
             for (int k = 0; k < 4 && rc == FELBM_OK; ++k) {
                 st->sweep_parts = parts_c[k];
                 st->sweep_tiled = tiled != 0;
-                // the tiled step runs 3 or 6 parts (two stages of 1 or 2 parts do not fit)
-                if (tiled && (tile_parts(st, st->dm.ell_w) != parts_c[k])) continue;
+                if (tiled && parts_c[k] != 3) continue;   // the blocked solve has one form
                 drop_graph(st);
                 float ms = 0.0f;
                 if ((rc = time_steps(st, trials, e0, e1, &ms)) != FELBM_OK) break;

@@ -342,10 +342,11 @@ __device__ __forceinline__ void rhs32_node(const DevMesh& m, const Phys& c, cons
         }
     }
     float s = m.inv_lumped32[i] * tau0;
+    store_all(b.r32, Np, i, acc);
+    if (kFirst) {
 #pragma unroll
-    for (int q = 0; q < 18; ++q) {
-        b.r32[q * Np + i] = acc[q];
-        if (kFirst) b.e1[q * Np + i] = acc[q] * s;
+        for (int q = 0; q < 18; ++q) acc[q] *= s;
+        store_all(b.e1, Np, i, acc);
     }
 }
 

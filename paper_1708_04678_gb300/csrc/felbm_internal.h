@@ -1,8 +1,13 @@
 // Internal host-side structures of the FE-LBM library (not part of the ABI).
 #pragma once
 
+#include <algorithm>
+#include <atomic>
 #include <cstdint>
+#include <exception>
+#include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "felbm.h"
@@ -16,8 +21,41 @@ void set_error(const std::string& msg);
 std::vector<int32_t> rcm_order(int32_t N, const std::vector<int32_t>& adj_ptr,
                                const std::vector<int32_t>& adj);
 
-// Most nodes in one tile of the tiled solve step (see HostMesh::tile_ptr).
+// Most nodes in one node tile and in one block of the blocked solve (half a
+// tile), most nodes of a block and the layers around it, and most layers.
 constexpr int32_t kTileNodes = 1024;
+constexpr int32_t kBlockCore = 512;
+constexpr int32_t kBlockNodes = 1024;
+constexpr int32_t kBlockSteps = 8;
+
+// f(k, scratch) for k in [0, n) on the host's cores, at least `grain` of them a
+// thread (on the calling thread alone where no other can be started); every
+// thread works with its own make().  The first exception is rethrown on the
+// calling thread.
+template <class Make, class F>
+void parallel_for(int32_t n, int32_t grain, const Make& make, const F& f) {
+    const int32_t nt = std::min<int32_t>(std::max(1u, std::thread::hardware_concurrency()), n / grain);
+    std::vector<std::thread> pool;
+    std::atomic<int32_t> next{0};
+    std::exception_ptr failed;
+    std::mutex mu;
+    const auto work = [&]() {
+        try {
+            auto scratch = make();
+            for (int32_t k; (k = next.fetch_add(1)) < n;) f(k, scratch);
+        } catch (...) {
+            std::lock_guard<std::mutex> lock(mu);
+            if (!failed) failed = std::current_exception();
+        }
+    };
+    try {
+        for (int32_t t = 1; t < nt; ++t) pool.emplace_back(work);
+    } catch (...) {
+    }
+    work();
+    for (auto& t : pool) t.join();
+    if (failed) std::rethrow_exception(failed);
+}
 
 // Host mesh after preprocessing.  Node ids are the internal ids (node tiles
 // of recursive coordinate bisection, reverse Cuthill-McKee order inside a
@@ -50,11 +88,20 @@ struct HostMesh {
     double min_area = 0.0, total_area = 0.0;
     int32_t max_degree = 0, bandwidth = 0;
     // node tiles: tile k holds the internal nodes [tile_ptr[k], tile_ptr[k+1]),
-    // at most kTileNodes, all in one component; its halo is the sorted list
-    // of nodes outside it that share a matrix row entry with one inside
+    // at most kTileNodes, all in one component
     std::vector<int32_t> tile_ptr;
+    int32_t max_halo = 0;                     // most nodes outside a tile that its matrix rows reference
+    // blocks of the blocked solve: a tile, or each half of one of more than
+    // kBlockCore nodes.  halo[halo_ptr[k] ...] lists the nodes around block k
+    // layer by layer (layer 1: the nodes outside that share a matrix row entry
+    // with one inside, layer 2: those that share one with layer 1, ...; each
+    // layer sorted); layer_cnt[k][l] counts the block's nodes and those up to
+    // layer l.  n_layers layers, the same for every block: as many as keep
+    // every block's count within kBlockNodes (at most kBlockSteps; 0: none do).
+    std::vector<int32_t> blk_ptr;
     std::vector<int32_t> halo_ptr, halo;
-    int32_t max_halo = 0;
+    std::vector<int32_t> layer_cnt;           // [blocks][kBlockSteps + 1]
+    int32_t n_layers = 0;
     // connected components ("groups"), numbered by their lowest caller node
     // id; each occupies a contiguous range of internal nodes and triangles
     int32_t G = 0;

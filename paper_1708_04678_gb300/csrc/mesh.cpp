@@ -102,13 +102,13 @@ std::vector<int32_t> rcm_order(int32_t N, const std::vector<int32_t>& adj_ptr,
     return order;
 }
 
-// Cut the nodes nodes[lo, hi) into tiles of at most kTileNodes by recursive
+// Cut the nodes nodes[lo, hi) into runs of at most `most` by recursive
 // coordinate bisection: split at the median of the longer side of their
-// bounding box, recurse into both halves in turn (so consecutive tiles are
-// neighbours in space), and record the end of every tile in `ends`.
-static void bisect_tiles(std::vector<int32_t>& nodes, int64_t lo, int64_t hi, const double* xy,
+// bounding box, recurse into both halves in turn (so consecutive runs are
+// neighbours in space), and record the end of every run in `ends`.
+static void bisect_tiles(std::vector<int32_t>& nodes, int64_t lo, int64_t hi, int64_t most, const double* xy,
                          std::vector<int64_t>& ends) {
-    if (hi - lo <= kTileNodes) {
+    if (hi - lo <= most) {
         ends.push_back(hi);
         return;
     }
@@ -126,8 +126,8 @@ static void bisect_tiles(std::vector<int32_t>& nodes, int64_t lo, int64_t hi, co
         const double ca = xy[2 * (size_t)a + axis], cb = xy[2 * (size_t)b + axis];
         return ca < cb || (ca == cb && a < b);
     });
-    bisect_tiles(nodes, lo, mid, xy, ends);
-    bisect_tiles(nodes, mid, hi, xy, ends);
+    bisect_tiles(nodes, lo, mid, most, xy, ends);
+    bisect_tiles(nodes, mid, hi, most, xy, ends);
 }
 
 // node_px / node_py: periodic lengths of the sub-mesh each node belongs to
@@ -308,15 +308,17 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
                 return csize[comp_of[a]] > csize[comp_of[b]];
             });
         // Node tiles within each component's run.  Recursive coordinate
-        // bisection makes compact tiles, the nodes of a tile keep their
-        // reverse Cuthill-McKee order; FELBM_ORDER=rcm keeps the plain
-        // reverse Cuthill-McKee order and cuts it into runs of kTileNodes.
+        // bisection makes compact tiles and, one level further, the blocks of
+        // the blocked solve; the nodes of a block keep their reverse
+        // Cuthill-McKee order.  FELBM_ORDER=rcm keeps the plain reverse
+        // Cuthill-McKee order and cuts it into runs.
         const char* env = std::getenv("FELBM_ORDER");
         const bool plain_rcm = env && std::string(env) == "rcm";
         std::vector<int32_t> rank(N);
         for (int32_t n = 0; n < N; ++n) rank[m.perm[n]] = n;
         m.tile_ptr.assign(1, 0);
-        std::vector<int64_t> ends;
+        m.blk_ptr.assign(1, 0);
+        std::vector<int64_t> ends, halves;
         for (int64_t a = 0; a < N;) {
             int64_t b = a;
             while (b < N && comp_of[m.perm[b]] == comp_of[m.perm[a]]) ++b;
@@ -325,15 +327,28 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
                 for (int64_t e = a + kTileNodes; e < b; e += kTileNodes) ends.push_back(e);
                 ends.push_back(b);
             } else {
-                bisect_tiles(m.perm, a, b, xy, ends);
+                bisect_tiles(m.perm, a, b, kTileNodes, xy, ends);
+            }
+            halves.clear();
+            int64_t t0 = a;
+            for (int64_t e : ends) {
+                if (plain_rcm && e - t0 > kBlockCore) halves.push_back(t0 + kBlockCore);
+                if (plain_rcm)
+                    halves.push_back(e);
+                else
+                    bisect_tiles(m.perm, t0, e, kBlockCore, xy, halves);
+                t0 = e;
+            }
+            if (!plain_rcm) {
                 int64_t s0 = a;
-                for (int64_t e : ends) {
+                for (int64_t e : halves) {
                     std::sort(m.perm.begin() + s0, m.perm.begin() + e,
                               [&](int32_t u, int32_t v) { return rank[u] < rank[v]; });
                     s0 = e;
                 }
             }
             for (int64_t e : ends) m.tile_ptr.push_back((int32_t)e);
+            for (int64_t e : halves) m.blk_ptr.push_back((int32_t)e);
             a = b;
         }
     }
@@ -447,25 +462,61 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
         }
     }
 
-    // ---- halo of every node tile ---------------------------------------
+    // ---- first layer of every tile (its size only), layers of every block ----
     {
-        const int32_t ntile = (int32_t)m.tile_ptr.size() - 1;
-        m.halo_ptr.assign(ntile + 1, 0);
-        m.halo.clear();
-        m.max_halo = 0;
-        std::vector<int32_t> h;
-        for (int32_t k = 0; k < ntile; ++k) {
-            const int32_t s0 = m.tile_ptr[k], s1 = m.tile_ptr[k + 1];
-            h.clear();
-            for (int32_t i = s0; i < s1; ++i)
-                for (int32_t p = m.row_ptr[i]; p < m.row_ptr[i + 1]; ++p)
-                    if (m.col[p] < s0 || m.col[p] >= s1) h.push_back(m.col[p]);
-            std::sort(h.begin(), h.end());
-            h.erase(std::unique(h.begin(), h.end()), h.end());
-            m.halo.insert(m.halo.end(), h.begin(), h.end());
-            m.halo_ptr[k + 1] = (int32_t)m.halo.size();
-            m.max_halo = std::max(m.max_halo, (int32_t)h.size());
+        const int32_t ntile = (int32_t)m.tile_ptr.size() - 1, nblk = (int32_t)m.blk_ptr.size() - 1;
+        using Marks = std::vector<int32_t>;                  // the run that saw a node last
+        const auto unmarked = [&]() { return Marks(N, -1); };
+        // the nodes outside run k = [s0, s1) that row i references and that it has not seen
+        const auto visit = [&](int32_t i, int32_t k, int32_t s0, int32_t s1, Marks& mark, std::vector<int32_t>& out) {
+            for (int32_t p = m.row_ptr[i]; p < m.row_ptr[i + 1]; ++p) {
+                const int32_t c = m.col[p];
+                if ((c >= s0 && c < s1) || mark[c] == k) continue;
+                mark[c] = k;
+                out.push_back(c);
+            }
+        };
+        std::vector<int32_t> first(ntile);
+        parallel_for(ntile, 64, unmarked, [&](int32_t k, Marks& mark) {
+            std::vector<int32_t> out;
+            for (int32_t i = m.tile_ptr[k]; i < m.tile_ptr[k + 1]; ++i)
+                visit(i, k, m.tile_ptr[k], m.tile_ptr[k + 1], mark, out);
+            first[k] = (int32_t)out.size();
+        });
+        m.max_halo = *std::max_element(first.begin(), first.end());
+        const int32_t stride = kBlockSteps + 1;
+        m.layer_cnt.assign((size_t)nblk * stride, 0);
+        std::vector<std::vector<int32_t>> ring(nblk);
+        std::vector<int32_t> fits(nblk);
+        parallel_for(nblk, 32, unmarked, [&](int32_t k, Marks& mark) {
+            const int32_t s0 = m.blk_ptr[k], s1 = m.blk_ptr[k + 1];
+            std::vector<int32_t>& h = ring[k];
+            h.reserve(kBlockNodes);
+            int32_t* cnt = m.layer_cnt.data() + (size_t)k * stride;
+            cnt[0] = s1 - s0;
+            size_t from = 0;
+            for (int32_t l = 1; l <= kBlockSteps; ++l) {
+                const size_t to = h.size();
+                if (l == 1)
+                    for (int32_t i = s0; i < s1; ++i) visit(i, k, s0, s1, mark, h);
+                for (size_t q = from; l > 1 && q < to; ++q) visit(h[q], k, s0, s1, mark, h);
+                if (s1 - s0 + (int64_t)h.size() > kBlockNodes) break;
+                std::sort(h.begin() + to, h.end());
+                from = to;
+                cnt[l] = s1 - s0 + (int32_t)h.size();
+                fits[k] = l;
+            }
+        });
+        m.n_layers = *std::min_element(fits.begin(), fits.end());
+        m.halo_ptr.assign(nblk + 1, 0);
+        for (int32_t k = 0; k < nblk; ++k) {
+            const int32_t* cnt = m.layer_cnt.data() + (size_t)k * stride;
+            m.halo_ptr[k + 1] = m.halo_ptr[k] + cnt[m.n_layers] - cnt[0];
         }
+        m.halo.resize(m.halo_ptr[nblk]);
+        for (int32_t k = 0; k < nblk; ++k)
+            std::copy(ring[k].begin(), ring[k].begin() + (m.halo_ptr[k + 1] - m.halo_ptr[k]),
+                      m.halo.begin() + m.halo_ptr[k]);
     }
 
     // ---- wall edges: new ids, length and unit normal out of the fluid ----
