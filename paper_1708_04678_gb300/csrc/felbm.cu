@@ -141,6 +141,7 @@ struct Phys {
     // 1 = vertex mean of the nodal patch Laplacian, lapmu_fac * sum l_ij (mu_j - mu_i)
     int lapmu_nodal;
     double lapmu_fac;
+    double inv_tau_l, inv_tau_v;
     // FP32 copies, rounded once on the host
     float dt_f, dt3_f, dt2h_f, inv_tau_l_f, inv_tau_v_f, rho_v_f, drho_f, mobility_f;
 };
@@ -241,16 +242,29 @@ __device__ __forceinline__ void store_all(float* x, int Np, int i, const float (
 }
 
 constexpr int kBlock = 256;
+constexpr int kWarpBlocksBelow = 512;   // items per multiprocessor (fp64_block)
 constexpr int kDiagBlocks = 608;   // fixed grid (4 x 152 SMs): the reduction order never changes
 constexpr int kDiagSlots = 16;
 constexpr int kDiagSums = 13;        // slots of the final reduction (k_diag_final, or k_diag_fused32's last block)
 constexpr int kDiagStepSlot = 15;    // felbm_diagnostics_enqueue: the step count
 constexpr int kSolveResSlot = 13;    // slots 13, 14: sum r^2 and sum b^2 of the checked solve (felbm_solver_check)
 
+// Programmatic dependent launch: a kernel launched with the attribute may
+// start while its predecessor drains; it must wait before touching that
+// kernel's outputs.  Both are no-ops in a kernel launched without it.  A
+// pointer to such outputs is never const __restrict__: the compiler would load
+// through the read-only path, ahead of the wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" :::); }
+
 // ------------------------------------------------------ K1: collision -----
 // Moments of the pre-collision state (C = sum h, p = sum g, rho u = sum e g /
 // cs2) and BGK collision towards the equilibria of eqn::g_eq / eqn::f_eq,
 // written in place: g_eq = w p + rho cs2 (Gamma - w), h_eq = Gamma C.
+// Bound by the FP64 pipe, hence one division instead of six and each direction
+// formed with its opposite: 155 us on 520,704 nodes against 207 us.  (With
+// T = Gamma / w - 1 and the factors of omega folded it took 115 us, but the
+// rounding of Gamma - w, which the 64-bit references share, then differs.)
 __global__ void __launch_bounds__(kBlock) k_collide(DevMesh m, Phys c, Bufs b, int do_collide) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
@@ -267,31 +281,37 @@ __global__ void __launch_bounds__(kBlock) k_collide(DevMesh m, Phys c, Bufs b, i
         C += h[q];
         p += g[q];
     }
-    double mx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-    double my = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-    double rho = c.rho_v + C * (c.rho_l - c.rho_v);
-    double ux = 3.0 * mx / rho, uy = 3.0 * my / rho;
+    const double mx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+    const double my = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
+    const double rho = c.rho_v + C * (c.rho_l - c.rho_v);
+    // omega = 1 / (tau + 1/2) = (1/tau) / (1 + 1/(2 tau)); one division for it and 1/rho
+    const double inv_tau = fma(C, c.inv_tau_l - c.inv_tau_v, c.inv_tau_v);
+    const double half = fma(0.5, inv_tau, 1.0), inv = 1.0 / (rho * half), inv_rho3 = 3.0 * half * inv;
+    const double ux = mx * inv_rho3, uy = my * inv_rho3;
     b.C[i] = C;
     b.p[i] = p;
     b.ux[i] = ux;
     b.uy[i] = uy;
     if (!do_collide) return;
-    double inv_tau = C / c.tau_l + (1.0 - C) / c.tau_v;
-    double omega = 1.0 / (1.0 / inv_tau + 0.5);
-    double uu15 = 1.5 * (ux * ux + uy * uy);
-    double rcs2 = rho * (1.0 / 3.0);
-#define FELBM_COLLIDE_Q(q)                                                            \
-    {                                                                                 \
-        double eu = edot<q>(ux, uy);                                                  \
-        double G = wq(q) * (1.0 + 3.0 * eu + 4.5 * eu * eu - uu15);                   \
-        double geq = wq(q) * p + rcs2 * (G - wq(q));                                  \
-        double heq = G * C;                                                           \
-        b.psi[q * Np + i] = g[q] - omega * (g[q] - geq);                              \
-        b.psi[(9 + q) * Np + i] = h[q] - omega * (h[q] - heq);                        \
+    const double omega = inv_tau * rho * inv;
+    const double uu15 = 1.5 * (ux * ux + uy * uy), rcs2 = rho * (1.0 / 3.0);
+    // a direction and its opposite share 4.5 (e.u)^2
+#define FELBM_COLLIDE_Q(q, G0)                                                          \
+    {                                                                                   \
+        const double G = wq(q) * (G0);                                                  \
+        const double geq = wq(q) * p + rcs2 * (G - wq(q));                              \
+        b.psi[(q) * Np + i] = g[q] - omega * (g[q] - geq);                              \
+        b.psi[(9 + (q)) * Np + i] = h[q] - omega * (h[q] - G * C);                      \
     }
-    FELBM_COLLIDE_Q(0) FELBM_COLLIDE_Q(1) FELBM_COLLIDE_Q(2) FELBM_COLLIDE_Q(3)
-    FELBM_COLLIDE_Q(4) FELBM_COLLIDE_Q(5) FELBM_COLLIDE_Q(6) FELBM_COLLIDE_Q(7)
-    FELBM_COLLIDE_Q(8)
+#define FELBM_COLLIDE_PAIR(q)                                                           \
+    {                                                                                   \
+        const double eu = edot<q>(ux, uy), t = 4.5 * eu * eu;                           \
+        FELBM_COLLIDE_Q(q, 1.0 + 3.0 * eu + t - uu15)                                   \
+        FELBM_COLLIDE_Q(opp(q), 1.0 - 3.0 * eu + t - uu15)                              \
+    }
+    FELBM_COLLIDE_Q(0, 1.0 - uu15)
+    FELBM_COLLIDE_PAIR(1) FELBM_COLLIDE_PAIR(2) FELBM_COLLIDE_PAIR(5) FELBM_COLLIDE_PAIR(6)
+#undef FELBM_COLLIDE_PAIR
 #undef FELBM_COLLIDE_Q
 }
 
@@ -299,20 +319,41 @@ __global__ void __launch_bounds__(kBlock) k_collide(DevMesh m, Phys c, Bufs b, i
 // mu_i = 2 beta C (C-1)(2C-1) - kappa lap(C)_i with the patch Laplacian
 // kappa lap(C)_i = kappa sum_j l_ij C_j + (1/V_i) sum_{wall e at i} -phi_c |e|
 // [ (Ca+Cb)/2 - (Ca^2 + Ca Cb + Cb^2)/3 ]  (wall flux of eqn:bc2, C linear on e).
+// kW > 0: the sum over the ELL copy of the row (zero padding), its columns and
+// coefficients loaded up front so that the gathers of C are in flight
+// together; kW = 0: CSR.
+template <int kW>
 __global__ void __launch_bounds__(kBlock) k_mu(DevMesh m, Phys c, Bufs b) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
     double lap = 0.0;
-    for (int k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) lap += m.lval[k] * b.C[m.col[k]];
+    int col[kW > 0 ? kW : 1];
+    double l[kW > 0 ? kW : 1];
+#pragma unroll
+    for (int k = 0; k < kW; ++k) {
+        col[k] = m.ell_col[k * m.Np + i];
+        l[k] = m.ell_lval[k * m.Np + i];
+    }
+    const int w0 = m.winc_ptr[i], w1 = m.winc_ptr[i + 1];
+    const double inv_vol = m.inv_vol[i];
+    if constexpr (kW > 0) {
+        double Cj[kW];
+#pragma unroll
+        for (int k = 0; k < kW; ++k) Cj[k] = b.C[col[k]];
+#pragma unroll
+        for (int k = 0; k < kW; ++k) lap = fma(l[k], Cj[k], lap);
+    } else {
+        for (int k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) lap += m.lval[k] * b.C[m.col[k]];
+    }
     double wall = 0.0;
-    for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
+    for (int k = w0; k < w1; ++k) {
         int e = m.winc_edge[k];
         double Ca = b.C[m.wall_a[e]], Cb = b.C[m.wall_b[e]];
         double s = 0.5 * (Ca + Cb) - (Ca * Ca + Ca * Cb + Cb * Cb) * (1.0 / 3.0);
         wall -= m.wall_phi[e] * m.wall_len[e] * s;
     }
     double C = b.C[i];
-    b.mu[i] = 2.0 * c.beta * C * (C - 1.0) * (2.0 * C - 1.0) - (c.kappa * lap + wall * m.inv_vol[i]);
+    b.mu[i] = 2.0 * c.beta * C * (C - 1.0) * (2.0 * C - 1.0) - (c.kappa * lap + wall * inv_vol);
 }
 
 // ------------------------------------------------- K3: grad mu per T ------
@@ -320,12 +361,20 @@ __global__ void __launch_bounds__(kBlock) k_gradmu(DevMesh m, Bufs b) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m.T) return;
     const int Tp = m.Tp;
+    int v[3];
+    double bx[3], by[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        v[k] = m.tri[k * Tp + t];
+        bx[k] = m.grad[(2 * k) * Tp + t];
+        by[k] = m.grad[(2 * k + 1) * Tp + t];
+    }
     double gx = 0.0, gy = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        double mu = b.mu[m.tri[k * Tp + t]];
-        gx += mu * m.grad[(2 * k) * Tp + t];
-        gy += mu * m.grad[(2 * k + 1) * Tp + t];
+        const double mu = b.mu[v[k]];
+        gx += mu * bx[k];
+        gy += mu * by[k];
     }
     b.gmu[t] = gx;
     b.gmu[Tp + t] = gy;
@@ -349,78 +398,108 @@ __global__ void __launch_bounds__(kBlock) k_lmu(DevMesh m, Phys c, Bufs b) {
 //   Phi_g = (e-u).[cs2 grad(rho) (Gamma - w) + mu grad(C) Gamma]
 //   Phi_h = [(e-u).(grad C - C/(rho cs2) (grad p - mu grad C)) + M lap(mu)] Gamma
 // Residual R_a = A (Phi_a - e_a . grad psi_hat_a), psi_hat P1 on the triangle.
+// The FP64 pipe is 87 % busy, so the forces are factored to about 190 FP64
+// instructions a triangle: 402 us on 1,040,384 triangles against 639 us for
+// the terms as written above.
 __global__ void __launch_bounds__(128) k_element(DevMesh m, Phys c, Bufs b) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m.T) return;
     const int Tp = m.Tp, Np = m.Np;
-    int v[3];
+    int v[3], nb[3];
     double bx[3], by[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         v[k] = m.tri[k * Tp + t];
+        nb[k] = m.nbr[k * Tp + t];
         bx[k] = m.grad[(2 * k) * Tp + t];
         by[k] = m.grad[(2 * k + 1) * Tp + t];
     }
     const double A = m.area[t];
-    double Cs = 0, ps = 0, uxs = 0, uys = 0, mus = 0, gCx = 0, gCy = 0, gpx = 0, gpy = 0;
+    const double third = 1.0 / 3.0;
+    double Cv[3], pv[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        double Cv = b.C[v[k]], pv = b.p[v[k]];
-        Cs += Cv;
-        ps += pv;
-        uxs += b.ux[v[k]];
-        uys += b.uy[v[k]];
-        mus += b.mu[v[k]];
-        gCx += Cv * bx[k];
-        gCy += Cv * by[k];
-        gpx += pv * bx[k];
-        gpy += pv * by[k];
+        Cv[k] = b.C[v[k]];
+        pv[k] = b.p[v[k]];
     }
-    const double third = 1.0 / 3.0;
-    double Cb = Cs * third, ux = uxs * third, uy = uys * third, mub = mus * third;
+    const double Cs = Cv[0] + Cv[1] + Cv[2];
+    const double ux = third * (b.ux[v[0]] + b.ux[v[1]] + b.ux[v[2]]);
+    const double uy = third * (b.uy[v[0]] + b.uy[v[1]] + b.uy[v[2]]);
+    const double mub = third * (b.mu[v[0]] + b.mu[v[1]] + b.mu[v[2]]);
+    const double gCx = fma(Cv[2], bx[2], fma(Cv[1], bx[1], Cv[0] * bx[0]));
+    const double gCy = fma(Cv[2], by[2], fma(Cv[1], by[1], Cv[0] * by[0]));
+    const double gpx = fma(pv[2], bx[2], fma(pv[1], bx[1], pv[0] * bx[0]));
+    const double gpy = fma(pv[2], by[2], fma(pv[1], by[1], pv[0] * by[0]));
     double lapmu = 0.0;
     if (c.lapmu_nodal) {
         lapmu = (b.lmu[v[0]] + b.lmu[v[1]] + b.lmu[v[2]]) * third;
     } else {
-        double gmx = b.gmu[t], gmy = b.gmu[Tp + t];
+        // -sum over interior edges of (grad mu_T + grad mu_T').b_k; the b_k sum
+        // to zero, so grad mu_T enters only through the wall edges
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            int nb = m.nbr[k * Tp + t];
-            if (nb >= 0) lapmu -= (gmx + b.gmu[nb]) * bx[k] + (gmy + b.gmu[Tp + nb]) * by[k];
+            const double gx = nb[k] >= 0 ? -b.gmu[nb[k]] : b.gmu[t], gy = nb[k] >= 0 ? -b.gmu[Tp + nb[k]] : b.gmu[Tp + t];
+            lapmu = fma(gx, bx[k], fma(gy, by[k], lapmu));
         }
     }
-    double drho = c.rho_l - c.rho_v;
-    double rhob = c.rho_v + Cb * drho;
-    double grx = drho * gCx, gry = drho * gCy;
-    double f = 3.0 * Cb / rhob;
-    double vhx = gCx - f * (gpx - mub * gCx), vhy = gCy - f * (gpy - mub * gCy);
-    double u_gr = ux * grx + uy * gry, u_gC = ux * gCx + uy * gCy, u_vh = ux * vhx + uy * vhy;
-    double uu15 = 1.5 * (ux * ux + uy * uy);
-    double Mlap = c.mobility * lapmu;
-    double out[18];
-#define FELBM_ELEM_Q(q)                                                                           \
-    {                                                                                             \
-        double eu = edot<q>(ux, uy);                                                              \
-        double G = wq(q) * (1.0 + 3.0 * eu + 4.5 * eu * eu - uu15);                               \
-        double phig = third * (G - wq(q)) * (edot<q>(grx, gry) - u_gr) + mub * G * (edot<q>(gCx, gCy) - u_gC); \
-        double phih = ((edot<q>(vhx, vhy) - u_vh) + Mlap) * G;                                    \
-        double dg = 0.0, dh = 0.0;                                                                \
-        if (q != 0) {                                                                             \
-            for (int k = 0; k < 3; ++k) {                                                         \
-                double eb = edot<q>(bx[k], by[k]);                                                \
-                dg += b.psi[q * Np + v[k]] * eb;                                                  \
-                dh += b.psi[(9 + q) * Np + v[k]] * eb;                                            \
-            }                                                                                     \
-        }                                                                                         \
-        out[q] = A * (phig - dg);                                                                 \
-        out[9 + q] = A * (phih - dh);                                                             \
+    const double drho = c.rho_l - c.rho_v, f = Cs / fma(Cs, third * drho, c.rho_v);   // C / (rho cs2)
+    const double vhx = gCx - f * (gpx - mub * gCx), vhy = gCy - f * (gpy - mub * gCy);
+    const double uu15 = 1.5 * (ux * ux + uy * uy);
+    // With T = Gamma / w - 1, s = (e - u).grad C and cs2 grad rho = (drho / 3) grad C:
+    //   A Phi_g = w s (P + Q T),  P = A mu,  Q = A (mu + drho / 3)
+    //   A Phi_h = w A ((e - u).v + M lap mu) (1 + T)
+    // formed for a direction and its opposite together (T = t2 +- 3 e.u); the
+    // axis weight 1/9 is folded into the vectors, diagonals take a quarter,
+    // rest four times.
+    const double P = A * mub, Q = fma(A * third, drho, P), w1 = 1.0 / 9.0, Aw = A * w1;
+    const double sx = w1 * gCx, sy = w1 * gCy, su = fma(ux, sx, uy * sy);
+    const double vx = Aw * vhx, vy = Aw * vhy, vu = fma(ux, vx, uy * vy) - Aw * (c.mobility * lapmu);
+    double abx[3], aby[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        abx[k] = A * bx[k];
+        aby[k] = A * by[k];
     }
-    FELBM_ELEM_Q(0) FELBM_ELEM_Q(1) FELBM_ELEM_Q(2) FELBM_ELEM_Q(3) FELBM_ELEM_Q(4)
-    FELBM_ELEM_Q(5) FELBM_ELEM_Q(6) FELBM_ELEM_Q(7) FELBM_ELEM_Q(8)
-#undef FELBM_ELEM_Q
+    double out[18];
+    out[0] = -4.0 * su * fma(Q, -uu15, P);
+    out[9] = -4.0 * fma(vu, -uu15, vu);
+#define FELBM_ELEM_PAIR(q, f)                                                                     \
+    {                                                                                             \
+        const double eu = edot<q>(ux, uy), t2 = fma(4.5 * eu, eu, -uu15);                         \
+        const double tp = fma(3.0, eu, t2), tm = fma(-3.0, eu, t2);                               \
+        const double es = edot<q>((f) * sx, (f) * sy), ev = edot<q>((f) * vx, (f) * vy);          \
+        const double vp = ev - (f) * vu, vm = -ev - (f) * vu;                                     \
+        double gp = (es - (f) * su) * fma(Q, tp, P), gm = (-es - (f) * su) * fma(Q, tm, P);       \
+        double hp = fma(vp, tp, vp), hm = fma(vm, tm, vm);                                        \
+        for (int k = 0; k < 3; ++k) {                                                             \
+            const double eb = edot<q>(abx[k], aby[k]);                                            \
+            gp = fma(-b.psi[(q) * Np + v[k]], eb, gp);                                            \
+            gm = fma(b.psi[opp(q) * Np + v[k]], eb, gm);                                          \
+            hp = fma(-b.psi[(9 + (q)) * Np + v[k]], eb, hp);                                      \
+            hm = fma(b.psi[(9 + opp(q)) * Np + v[k]], eb, hm);                                    \
+        }                                                                                         \
+        out[q] = gp;                                                                              \
+        out[opp(q)] = gm;                                                                         \
+        out[9 + (q)] = hp;                                                                        \
+        out[9 + opp(q)] = hm;                                                                     \
+    }
+    FELBM_ELEM_PAIR(1, 1.0) FELBM_ELEM_PAIR(2, 1.0) FELBM_ELEM_PAIR(5, 0.25) FELBM_ELEM_PAIR(6, 0.25)
+#undef FELBM_ELEM_PAIR
     double2* dst = reinterpret_cast<double2*>(b.R + (size_t)t * 18);
 #pragma unroll
     for (int k = 0; k < 9; ++k) dst[k] = make_double2(out[2 * k], out[2 * k + 1]);
+}
+
+// The right-hand side of an FP32 correction and its first iterate s r.
+__device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const double (&r)[18], float s) {
+    float r32[18], e[18];
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        r32[q] = (float)r[q];
+        e[q] = r32[q] * s;
+    }
+    store_all(b.r32, Np, i, r32);
+    store_all(b.e1, Np, i, e);
 }
 
 // ------------------------------------------- K5: streaming RHS gather -----
@@ -432,67 +511,106 @@ __global__ void __launch_bounds__(128) k_element(DevMesh m, Phys c, Bufs b) {
 // FP32 Richardson steps): in FP64 (FP64 Chebyshev) or, for the
 // mixed-precision solve, in FP32 together with the FP32 copy of the
 // right-hand side.
-template <bool kMixed>
+//
+// Bound by the FP64 pipe (85 % busy: 108 FMAs, 60 operations on the weights, 18
+// conversions a node): 175 us on 520,704 nodes, 256 us with the weights formed
+// direction by direction and the first iterate in FP64.
+// One thread per node, or (kSets = 2, consecutive blocks) one per node and set,
+// which forms the weights twice but halves a thread's chain of loads and its
+// straight-line code -- what a small mesh waits for (2,112 nodes: 15.5 us
+// against 17.3).
+template <bool kMixed, int kSets>
 __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double first_scale) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int kN = kSets == 1 ? 18 : 9;
+    const int nb = (int)blockIdx.x / kSets, set = (int)blockIdx.x - nb * kSets;
+    const int i = nb * (int)blockDim.x + (int)threadIdx.x;
     if (i >= m.N) return;
     const int Np = m.Np;
-    double acc[18];
+    double acc[kN];
 #pragma unroll
-    for (int q = 0; q < 18; ++q) acc[q] = 0.0;
+    for (int q = 0; q < kN; ++q) acc[q] = 0.0;
     const double c1 = c.dt * (1.0 / 3.0), c2 = 0.5 * c.dt * c.dt;
-    for (int k = m.inc_ptr[i]; k < m.inc_ptr[i + 1]; ++k) {
-        int t = m.inc_tri[k];
-        double bxi = m.inc_bx[k], byi = m.inc_by[k];
-        const double2* src = reinterpret_cast<const double2*>(b.R + (size_t)t * 18);
-        double r[18];
+    // the next triangle's id and gradient are loaded while this one's residual is in flight
+    const int k1 = m.inc_ptr[i + 1];
+    int k = m.inc_ptr[i], t = k < k1 ? m.inc_tri[k] : 0;
+    double bxi = k < k1 ? m.inc_bx[k] : 0.0, byi = k < k1 ? m.inc_by[k] : 0.0;
+    const int w0 = m.winc_ptr[i], w1 = m.winc_ptr[i + 1];
+    const double s = m.inv_lumped[i] * first_scale;
+    const double* psi = b.psi + (size_t)9 * set * Np;
+    while (k < k1) {
+        const double* src = b.R + (size_t)t * 18 + 9 * set;
+        double r[kN];
+        if constexpr (kSets == 1) {
 #pragma unroll
-        for (int s = 0; s < 9; ++s) {
-            double2 v2 = src[s];
-            r[2 * s] = v2.x;
-            r[2 * s + 1] = v2.y;
+            for (int q = 0; q < 9; ++q) {
+                const double2 v2 = reinterpret_cast<const double2*>(src)[q];
+                r[2 * q] = v2.x;
+                r[2 * q + 1] = v2.y;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 9; ++q) r[q] = src[q];
         }
-#define FELBM_RHS_Q(q)                                          \
-        {                                                       \
-            double w = c1 + c2 * edot<q>(bxi, byi);             \
-            acc[q] += r[q] * w;                                 \
-            acc[9 + q] += r[9 + q] * w;                         \
+        const double wx = c2 * bxi, wy = c2 * byi;
+        if (++k < k1) {
+            t = m.inc_tri[k];
+            bxi = m.inc_bx[k];
+            byi = m.inc_by[k];
         }
-        FELBM_RHS_Q(0) FELBM_RHS_Q(1) FELBM_RHS_Q(2) FELBM_RHS_Q(3) FELBM_RHS_Q(4)
-        FELBM_RHS_Q(5) FELBM_RHS_Q(6) FELBM_RHS_Q(7) FELBM_RHS_Q(8)
-#undef FELBM_RHS_Q
+        const double xp = c1 + wx, xm = c1 - wx;      // c1 + c2 e.b for e = (+-1, 0); the diagonals add +-wy
+        const double w[9] = {c1, xp, c1 + wy, xm, c1 - wy, xp + wy, xm + wy, xm - wy, xp - wy};
+#pragma unroll
+        for (int q = 0; q < kN; ++q) acc[q] = fma(r[q], w[q % 9], acc[q]);
     }
-    for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
-        int e = m.winc_edge[k];
-        int o = m.wall_a[e] == i ? m.wall_b[e] : m.wall_a[e];
-        double L = m.wall_len[e], nx = m.wall_nx[e], ny = m.wall_ny[e];
+    for (int kw = w0; kw < w1; ++kw) {
+        const int e = m.winc_edge[kw], a0 = m.wall_a[e], a1 = m.wall_b[e], o = a0 == i ? a1 : a0;
+        const double L = m.wall_len[e], nx = m.wall_nx[e], ny = m.wall_ny[e];
+        // all populations of both ends first, so that they are in flight together
+        double pi[kN], po[kN];
+#pragma unroll
+        for (int q = 0; q < kN; ++q) {
+            if (q % 9 == 0) continue;
+            pi[q] = psi[q * Np + i];
+            po[q] = psi[q * Np + o];
+        }
+        const double wi = L * (1.0 / 3.0), wo = L * (1.0 / 6.0);
 #define FELBM_WALL_Q(q)                                                                      \
         {                                                                                    \
-            double en = edot<q>(nx, ny);                                                     \
+            const double en = edot<q>(nx, ny);                                               \
             if (en < 0.0) {                                                                  \
-                double f = -c.dt * en;                                                       \
-                double dgi = b.psi[opp(q) * Np + i] - b.psi[q * Np + i];                     \
-                double dgo = b.psi[opp(q) * Np + o] - b.psi[q * Np + o];                     \
-                double dhi = b.psi[(9 + opp(q)) * Np + i] - b.psi[(9 + q) * Np + i];         \
-                double dho = b.psi[(9 + opp(q)) * Np + o] - b.psi[(9 + q) * Np + o];         \
-                acc[q] += f * (L * (1.0 / 3.0) * dgi + L * (1.0 / 6.0) * dgo);               \
-                acc[9 + q] += f * (L * (1.0 / 3.0) * dhi + L * (1.0 / 6.0) * dho);           \
+                const double f = -c.dt * en;                                                 \
+                _Pragma("unroll") for (int h = 0; h < kN; h += 9)                            \
+                    acc[h + q] += f * (wi * (pi[h + opp(q)] - pi[h + q]) + wo * (po[h + opp(q)] - po[h + q])); \
             }                                                                                \
         }
         FELBM_WALL_Q(1) FELBM_WALL_Q(2) FELBM_WALL_Q(3) FELBM_WALL_Q(4)
         FELBM_WALL_Q(5) FELBM_WALL_Q(6) FELBM_WALL_Q(7) FELBM_WALL_Q(8)
 #undef FELBM_WALL_Q
     }
-    double s = m.inv_lumped[i] * first_scale;
 #pragma unroll
-    for (int q = 0; q < 18; ++q) {
-        b.rhs[q * Np + i] = acc[q];
-        if (kMixed) {
-            b.r32[vec_at(Np, q, i)] = (float)acc[q];
-            b.e1[vec_at(Np, q, i)] = (float)(acc[q] * s);
-        } else {
-            b.x1[q * Np + i] = acc[q] * s;
+    for (int q = 0; q < kN; ++q) {
+        b.rhs[(9 * set + q) * Np + i] = acc[q];
+        if (!kMixed) b.x1[(9 * set + q) * Np + i] = acc[q] * s;
+    }
+    // the corrections start from the FP32 copy (conversions share the FP64 pipe)
+    if constexpr (kMixed && kSets == 1) {
+        store_start(b, Np, i, acc, (float)s);
+    } else if constexpr (kMixed) {
+        float r32[9], e[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            r32[q] = (float)acc[q];
+            e[q] = r32[q] * (float)s;
         }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const float rp[4] = {r32[4 * p + 1], r32[4 * p + 2], r32[4 * p + 3], r32[4 * p + 4]};
+            const float ep[4] = {e[4 * p + 1], e[4 * p + 2], e[4 * p + 3], e[4 * p + 4]};
+            store_vec(b.r32, Np, 2 * set + p, i, rp);
+            store_vec(b.e1, Np, 2 * set + p, i, ep);
+        }
+        b.r32[vec_at(Np, 9 * set, i)] = r32[0];
+        b.e1[vec_at(Np, 9 * set, i)] = e[0];
     }
 }
 
@@ -504,16 +622,13 @@ __global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, double
     if (i >= m.N) return;
     const int Np = m.Np;
     double s = m.inv_lumped[i] * first_scale;
+    double acc[18];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        double r = b.rhs[q * Np + i];
-        if (kMixed) {
-            b.r32[vec_at(Np, q, i)] = (float)r;
-            b.e1[vec_at(Np, q, i)] = (float)(r * s);
-        } else {
-            b.x1[q * Np + i] = r * s;
-        }
+        acc[q] = b.rhs[q * Np + i];
+        if (!kMixed) b.x1[q * Np + i] = acc[q] * s;
     }
+    if constexpr (kMixed) store_start(b, Np, i, acc, (float)s);
 }
 
 // ---------------------------------------------- K6: Chebyshev sweep -------
@@ -558,11 +673,15 @@ __global__ void __launch_bounds__(128) k_cheb(DevMesh m, Bufs b, const double* _
 // ~70x the FP64 rate, so only the refinement kernels pay FP64 matvecs.
 enum Final { kStore = 0, kAddPsi = 1, kAddX64 = 2, kUpdateDev = 3 };
 
-// Programmatic dependent launch: a kernel launched with the attribute may
-// start while its predecessor drains; it must wait before touching that
-// kernel's outputs.  Both are no-ops in a kernel launched without it.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" :::); }
+// A float as a double through the integer pipe: the conversion instruction
+// shares the FP64 pipe, whose rate is 1/64 of it.  Exact for every float
+// (the rare denormals take the instruction).
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0u && (u << 1) != 0u) return (double)x;
+    const uint32_t bias = e == 0u ? 0u : (e == 0x7f800000u ? 0x70000000u : 0x38000000u);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
+}
 
 #include "felbm_dev32.cuh"
 #include "felbm_adjoint.cuh"
@@ -579,7 +698,7 @@ __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.lau
 // recurrence, but each step reads only x_k (gathered) and b.
 //   cur = x_k; the new iterate goes to nxt (or to the final destination).
 template <int kFinal>
-__global__ void __launch_bounds__(128) k_cheb32(DevMesh m, Phys c, Bufs b, const float* __restrict__ cur,
+__global__ void __launch_bounds__(128) k_cheb32(DevMesh m, Phys c, Bufs b, const float* cur,
                                                 float* nxt, float tau, int have_x64) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
@@ -628,7 +747,7 @@ __host__ __device__ constexpr int vec_first(int parts, int part) {
 // The planes [kP, kEnd) of one node's step; g: all gathered values are loaded
 // before the first product (more loads in flight per thread).
 template <int kP, int kEnd, int kFinal, int kW, bool kFromRhs>
-__device__ __forceinline__ void sweep_planes(const DevMesh& m, const Bufs& b, const float* __restrict__ cur, float* nxt,
+__device__ __forceinline__ void sweep_planes(const DevMesh& m, const Bufs& b, const float* cur, float* nxt,
                                              int i, const int (&col)[kW], const float (&val)[kW],
                                              const float (&sc)[kFromRhs ? kW : 1], float s, int have_x64,
                                              float (&d)[18]) {
@@ -679,7 +798,7 @@ __device__ __forceinline__ void sweep_planes(const DevMesh& m, const Bufs& b, co
 }
 
 template <int kPart, int kParts, int kFinal, int kW, bool kFromRhs>
-__device__ __forceinline__ void sweep_part(int part, const DevMesh& m, const Bufs& b, const float* __restrict__ cur,
+__device__ __forceinline__ void sweep_part(int part, const DevMesh& m, const Bufs& b, const float* cur,
                                            float* nxt, int i, const int (&col)[kW], const float (&val)[kW],
                                            const float (&sc)[kFromRhs ? kW : 1], float s, int have_x64, float (&d)[18]) {
     if constexpr (kPart < kParts) {
@@ -700,7 +819,7 @@ __device__ __forceinline__ void sweep_part(int part, const DevMesh& m, const Buf
 // run together and share the block's matrix rows through L2 instead of
 // fetching them from DRAM once per part.
 template <int kFinal, int kW, int kParts, bool kFromRhs = false>
-__global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, const float* __restrict__ cur,
+__global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, const float* cur,
                                                  float* nxt, float tau, int have_x64, float tau0) {
     pdl_release();
     static_assert(kFinal != kUpdateDev || kParts == 1, "the field update needs the whole node");
@@ -733,31 +852,87 @@ __global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, cons
 }
 
 // x <- x + e ; rho <- rho - M11 e (FP64) ; FP32 copy of rho and the first
-// iterate of the next correction, tau_0 rho / m.
-__global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* __restrict__ e,
-                                                float* next_first, int first_round, double tau0) {
+// iterate of the next correction, tau_0 rho / m.  One thread per node and
+// plane (consecutive blocks, which share the rows through L2): five times the
+// warps and a fifth of the straight-line code, which is what a small mesh
+// waits for (2,112 nodes: 8.3 us against 15.3 for all planes in a thread; on
+// 520,704 nodes 212 against 197 us).  The FP64 pipe is 85 % busy; with
+// conversion instructions for the 126 gathered values it took 377 us.
+template <int NV>
+__device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, const float* e,
+                                             float* next_first, int first_round, float tau0, int p, int i) {
+    const int Np = m.Np, k1 = m.row_ptr[i + 1];
+    int k = m.row_ptr[i];
+    const float s = m.inv_lumped32[i] * tau0;
+    // every load of the node itself before the first store (the compiler keeps
+    // their order, and one at a time they cost a latency each)
+    const size_t at = (size_t)(NV == 2 ? 0 : 9 * (p >> 1) + 1 + 4 * (p & 1)) * Np + i, stride = (size_t)(NV == 2 ? 9 : 1) * Np;
+    float ei[NV];
+    double acc[NV], ro[NV], xo[NV];
+    load_vec(ei, e, Np, p, i);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+        acc[c] = 0.0;
+        ro[c] = first_round ? b.rhs[at + c * stride] : b.rho64[at + c * stride];
+        xo[c] = first_round ? 0.0 : b.x64[at + c * stride];
+    }
+#pragma unroll 4
+    for (; k < k1; ++k) {
+        const double mv = m.mval[k];
+        float ej[NV];
+        load_vec(ej, e, Np, p, m.col[k]);
+#pragma unroll
+        for (int c = 0; c < NV; ++c) acc[c] = fma(mv, widen(ej[c]), acc[c]);
+    }
+    float r32[NV], first[NV];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+        const double ed = widen(ei[c]), rn = ro[c] - acc[c];
+        b.x64[at + c * stride] = first_round ? ed : xo[c] + ed;
+        b.rho64[at + c * stride] = rn;
+        r32[c] = (float)rn;
+        first[c] = r32[c] * s;
+    }
+    store_vec(b.r32, Np, p, i, r32);
+    store_vec(next_first, Np, p, i, first);
+}
+
+__global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* e,
+                                                float* next_first, int first_round, float tau0) {
+    const int nb = (int)blockIdx.x / kPlanes, p = (int)blockIdx.x - kPlanes * nb;
+    const int i = nb * (int)blockDim.x + (int)threadIdx.x;
+    if (i >= m.N) return;
+    if (p < 4)
+        refine_plane<4>(m, b, e, next_first, first_round, tau0, p, i);
+    else
+        refine_plane<2>(m, b, e, next_first, first_round, tau0, p, i);
+}
+
+// The last correction's iterate e added up (FP64): psi += x64 + e (the time
+// step), or x64 += e.  A kernel of its own: inside k_block32 the 108 extra
+// loads and stores a node spill its registers (136 us against 66 + 48 us on
+// 520,704 nodes).
+template <bool kPsi>
+__global__ void __launch_bounds__(128) k_add64(DevMesh m, Bufs b, const float* e, int have_x64) {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
     const int Np = m.Np;
-    double acc[18];
-#pragma unroll
-    for (int q = 0; q < 18; ++q) acc[q] = 0.0;
-    for (int k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
-        int j = m.col[k];
-        double mv = m.mval[k];
-#pragma unroll
-        for (int q = 0; q < 18; ++q) acc[q] += mv * (double)e[vec_at(Np, q, j)];
-    }
-    double s = m.inv_lumped[i] * tau0;
+    float ei[18];
+    double xo[18], po[18];
+    load_all(ei, e, Np, i);
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        double xo = first_round ? 0.0 : b.x64[q * Np + i];
-        double ro = first_round ? b.rhs[q * Np + i] : b.rho64[q * Np + i];
-        double rn = ro - acc[q];
-        b.x64[q * Np + i] = xo + (double)e[vec_at(Np, q, i)];
-        b.rho64[q * Np + i] = rn;
-        b.r32[vec_at(Np, q, i)] = (float)rn;
-        next_first[vec_at(Np, q, i)] = (float)(rn * s);
+        xo[q] = have_x64 ? b.x64[q * Np + i] : 0.0;
+        if (kPsi) po[q] = b.psi[q * Np + i];
+    }
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        const double x = have_x64 ? xo[q] + widen(ei[q]) : widen(ei[q]);
+        if (kPsi)
+            b.psi[q * Np + i] = po[q] + x;
+        else
+            b.x64[q * Np + i] = x;
     }
 }
 
@@ -1518,6 +1693,13 @@ static cudaError_t up(const T* dst, const std::vector<T>& src, cudaStream_t s) {
 
 static unsigned grid_for(int n, int block) { return (unsigned)((n + block - 1) / block); }
 
+// Threads per block of the FP64 kernels: `most`, or a warp where that spreads
+// n items over the multiprocessors more evenly (the FP64 pipe of each is what
+// the kernels wait for): a step on 2,112 nodes took 101 us against 125, on
+// 18,432 nodes 162 against 186 (with the other FP64 changes); on 520,704 nodes
+// the two are the same.
+static int fp64_block(const felbm_state* st, int n, int most) { return n < kWarpBlocksBelow * st->n_sm ? 32 : most; }
+
 // Launch with or without programmatic dependent launch (PDL).
 template <typename... KArgs, typename... Args>
 static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
@@ -1535,25 +1717,23 @@ static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, si
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// One blocked launch: K steps from cur (or from b) to nxt or the final
-// destination.  All planes of a block in one thread block; one plane each
+// One blocked launch: K steps from cur (or from b) to nxt.  All planes of a block in one thread block; one plane each
 // where that would leave multiprocessors idle.
-template <int kFinal, int kW, bool kFromRhs>
-static void launch_block_w(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                           float* nxt, const BlockTau& bt, int K, float tau0, int have_x64, bool pdl) {
-    const int ny = m.n_blocks >= kSplitPlanesBelow * st->n_sm ? 1 : kPlanes;
-    launch_k(pdl, k_block32<kW, kFinal, kFromRhs>, dim3((unsigned)m.n_blocks, ny), dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur,
-             nxt, bt, K, tau0, have_x64);
-}
-
-template <int kFinal, bool kFromRhs>
+template <bool kFromRhs>
 static void launch_block(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                         float* nxt, const BlockTau& bt, int K, float tau0, int have_x64, bool pdl) {
-    pdl = pdl && st->use_pdl;
+                         float* nxt, const BlockTau& bt, int K, float tau0, bool pdl) {
+    const bool full = m.n_blocks >= kSplitPlanesBelow * st->n_sm;
+    const dim3 grid((unsigned)m.n_blocks, full ? 1 : kPlanes);
+    const auto go = [&](auto kern) {
+        // dependent launch places the blocks of a small grid on whatever
+        // multiprocessors the previous kernel has left, two on one while
+        // others idle: 82 against 74 us a step on 2,112 nodes (FP64)
+        launch_k(pdl && full && st->use_pdl, kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur, nxt, bt, K, tau0);
+    };
     switch (m.ell_w) {
-        case 7: launch_block_w<kFinal, 7, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl); break;
-        case 9: launch_block_w<kFinal, 9, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl); break;
-        default: launch_block_w<kFinal, 12, kFromRhs>(st, m, b, s, cur, nxt, bt, K, tau0, have_x64, pdl);
+        case 7: go(k_block32<7, kFromRhs>); break;
+        case 9: go(k_block32<9, kFromRhs>); break;
+        default: go(k_block32<12, kFromRhs>);
     }
 }
 
@@ -1565,10 +1745,8 @@ static cudaError_t allow_block_smem() {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSmem));
     };
-    set(k_block32<kW, kStore, false>);
-    set(k_block32<kW, kStore, true>);
-    set(k_block32<kW, kAddPsi, false>);
-    set(k_block32<kW, kAddX64, false>);
+    set(k_block32<kW, false>);
+    set(k_block32<kW, true>);
     return e;
 }
 
@@ -1656,10 +1834,10 @@ static void launch_first(felbm_state* st, const DevMesh& m, const Bufs& b, cudaS
 static bool blocked(const felbm_state* st, const DevMesh& m) { return st->sweep_tiled && m.blk_steps > 0; }
 
 // The steps [k, end) of one correction in as few blocked launches as the
-// layers allow, of about equal length; the last goes to `final` unless it is
-// kStore.  Returns the buffer with the last stored iterate.
+// layers allow, of about equal length.  Returns the buffer with the last
+// iterate.
 static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, float* cur, float* prv,
-                              int k, int end, int final, int have_x64, bool from_rhs, bool pdl) {
+                              int k, int end, bool from_rhs, bool pdl) {
     int left = (end - k + m.blk_steps - 1) / m.blk_steps;
     for (; left > 0; --left) {
         const int K = (end - k + left - 1) / left;
@@ -1667,13 +1845,9 @@ static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, 
         for (int j = 0; j < K; ++j) bt.tau[j] = (float)st->tau[k + j];
         const float tau0 = (float)st->tau[0];
         if (from_rhs)
-            launch_block<kStore, true>(st, m, b, s, nullptr, prv, bt, K, tau0, have_x64, pdl);
-        else if (left > 1 || final == kStore)
-            launch_block<kStore, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
-        else if (final == kAddPsi)
-            launch_block<kAddPsi, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
+            launch_block<true>(st, m, b, s, nullptr, prv, bt, K, tau0, pdl);
         else
-            launch_block<kAddX64, false>(st, m, b, s, cur, prv, bt, K, tau0, have_x64, pdl);
+            launch_block<false>(st, m, b, s, cur, prv, bt, K, tau0, pdl);
         from_rhs = false;
         pdl = true;
         k += K;
@@ -1698,6 +1872,16 @@ static bool first_from_rhs(const felbm_state* st, const DevMesh& m) {
     return st->dev32 && st->rounds == 1 && st->sweeps > 2 && !st->check && (blocked(st, m) || gathered_width(m.ell_w));
 }
 
+static void launch_mu(const DevMesh& m, const Phys& c, const Bufs& b, unsigned grid, int block, cudaStream_t s) {
+    switch (m.ell_w) {
+        case 7: k_mu<7><<<grid, block, 0, s>>>(m, c, b); break;
+        case 9: k_mu<9><<<grid, block, 0, s>>>(m, c, b); break;
+        case 12: k_mu<12><<<grid, block, 0, s>>>(m, c, b); break;
+        case 16: k_mu<16><<<grid, block, 0, s>>>(m, c, b); break;
+        default: k_mu<0><<<grid, block, 0, s>>>(m, c, b);
+    }
+}
+
 // Enqueue the mass solve for the right-hand side in b.rhs (first iterate
 // already written, unless from_rhs).  into_psi: add the increment to psi (time step); else
 // leave the solution in x1/x0 (FP64 mode, returned) or x64 (mixed mode).
@@ -1705,13 +1889,14 @@ static bool first_from_rhs(const felbm_state* st, const DevMesh& m) {
 // set of scratch buffers with the same layout).
 static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s,
                                    bool into_psi, bool after_release = false, bool from_rhs = false) {
-    const unsigned grid = grid_for(m.N, 128);
+    const int nb = fp64_block(st, m.N, 128);
+    const unsigned grid = grid_for(m.N, nb);
     if (st->mode == FELBM_SOLVER_FP64) {
         const double* result = b.x1;
         for (int k = 1; k < st->sweeps; ++k) {
             const double* cur = (k & 1) ? b.x1 : b.x0;
             double* prev = (k & 1) ? b.x0 : b.x1;
-            k_cheb<<<grid, 128, 0, s>>>(m, b, cur, prev, st->cheb_a[k], st->cheb_c[k], k == 1,
+            k_cheb<<<grid, nb, 0, s>>>(m, b, cur, prev, st->cheb_a[k], st->cheb_c[k], k == 1,
                                         into_psi && k == st->sweeps - 1);
             result = prev;
         }
@@ -1725,22 +1910,25 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
         float* prv = B;
         const bool last_round = r == st->rounds - 1;
         if (blocked(st, m)) {
-            const int final = !last_round || (into_psi && st->dev32) ? kStore : (into_psi ? kAddPsi : kAddX64);
             bool pdl = r == 0 && after_release;
             int k = 1;
             if (last_round && st->check) {
-                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, kStore, have_x64, false, pdl);
+                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, false, pdl);
                 prv = x == cur ? prv : cur;
                 cur = x;
                 enqueue_resid(st, m, b, s, cur);
                 k = st->sweeps - 1;
                 pdl = false;
             }
-            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, final, have_x64, from_rhs && r == 0, pdl);
+            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, from_rhs && r == 0, pdl);
             prv = x == cur ? prv : cur;
             cur = x;
             if (last_round && into_psi && st->dev32)
-                launch_k(st->use_pdl, k_update32, dim3(grid_for(m.N, 128)), dim3(128), 0, s, m, st->phys, b, (const float*)cur);
+                launch_k(st->use_pdl, k_update32, dim3(grid_for(m.N, 128)), dim3(128), 0, s, m, st->phys, b,
+                         (const float*)cur);
+            else if (last_round)
+                launch_k(st->use_pdl, into_psi ? k_add64<true> : k_add64<false>, dim3(grid), dim3(nb), 0, s, m, b,
+                         (const float*)cur, have_x64);
         }
         for (int k = 1; k < st->sweeps && !blocked(st, m); ++k) {
             const float tau = (float)st->tau[k];
@@ -1764,7 +1952,7 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
             std::swap(cur, prv);
         }
         if (!last_round) {
-            k_refine<<<grid, 128, 0, s>>>(m, b, cur, prv, r == 0, st->tau[0]);
+            k_refine<<<grid * kPlanes, nb, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0]);
             A = prv;
             B = cur;
         }
@@ -1779,7 +1967,7 @@ static int solve_launches(const felbm_state* st) {
     const int most = st->dm.blk_steps;
     const auto groups = [&](int steps) { return (steps + most - 1) / most; };
     const int last = st->check ? groups(st->sweeps - 2) + 1 : groups(st->sweeps - 1);
-    return refines * (groups(st->sweeps - 1) + 1) + last + (st->dev32 ? 1 : 0);
+    return refines * (groups(st->sweeps - 1) + 1) + last + 1;
 }
 
 static int step_launches(const felbm_state* st) { return (st->dev32 ? 4 : 5) + solve_launches(st); }
@@ -1860,21 +2048,25 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
         mark(6);
         return;
     }
-    k_collide<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b, 1);
+    const int nb = fp64_block(st, m.N, 128), tb = fp64_block(st, m.T, 128);
+    const unsigned ng = grid_for(m.N, nb), tg = grid_for(m.T, tb);
+    k_collide<<<ng, nb, 0, s>>>(m, st->phys, b, 1);
     mark(1);
-    k_mu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b);
+    launch_mu(m, st->phys, b, ng, nb, s);
     mark(2);
     if (st->phys.lapmu_nodal)
-        k_lmu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b);
+        k_lmu<<<ng, nb, 0, s>>>(m, st->phys, b);
     else
-        k_gradmu<<<grid_for(m.T, kBlock), kBlock, 0, s>>>(m, b);
+        k_gradmu<<<tg, tb, 0, s>>>(m, b);
     mark(3);
-    k_element<<<grid_for(m.T, 128), 128, 0, s>>>(m, st->phys, b);
+    k_element<<<tg, tb, 0, s>>>(m, st->phys, b);
     mark(4);
+    // a small mesh takes a thread per node and set
+    const auto rhs = [&](auto kern, int sets, double scale) { kern<<<sets * ng, nb, 0, s>>>(m, st->phys, b, scale); };
     if (st->mode == FELBM_SOLVER_FP64)
-        k_rhs<false><<<grid_for(m.N, 128), 128, 0, s>>>(m, st->phys, b, st->inv_theta);
+        nb == 32 ? rhs(k_rhs<false, 2>, 2, st->inv_theta) : rhs(k_rhs<false, 1>, 1, st->inv_theta);
     else
-        k_rhs<true><<<grid_for(m.N, 128), 128, 0, s>>>(m, st->phys, b, st->tau[0]);
+        nb == 32 ? rhs(k_rhs<true, 2>, 2, st->tau[0]) : rhs(k_rhs<true, 1>, 1, st->tau[0]);
     mark(5);
     enqueue_solve(st, st->dm, st->buf, s, true);
     mark(6);
@@ -1940,6 +2132,8 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     ph.lapmu_nodal = params->lapmu_mode == FELBM_LAPMU_NODAL;
     // lval = -2 K_ij / (s |patch_i|); the lumped P1 Laplacian is -K_ij / (|patch_i| / 3)
     ph.lapmu_fac = (params->lap_mode == FELBM_LAP_PAPER ? 1.0 : 2.0 / 3.0) * 1.5;
+    ph.inv_tau_l = 1.0 / params->tau_l;
+    ph.inv_tau_v = 1.0 / params->tau_v;
     ph.dt_f = (float)params->dt;
     ph.dt3_f = (float)(params->dt / 3.0);
     ph.dt2h_f = (float)(0.5 * params->dt * params->dt);
@@ -2639,7 +2833,7 @@ int felbm_get_fields(felbm_state* st, double* C, double* p, double* ux, double* 
         return FELBM_OK;
     }
     k_collide<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, st->buf, 0);
-    k_mu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, st->buf);
+    launch_mu(m, st->phys, st->buf, grid_for(m.N, kBlock), kBlock, s);
     FELBM_CUDA(cudaGetLastError());
     double* srcs[5] = {st->buf.C, st->buf.p, st->buf.ux, st->buf.uy, st->buf.mu};
     for (int k = 0; k < 5; ++k) {
@@ -3041,7 +3235,7 @@ int felbm_adjoint_step(felbm_state* st) {
     AdjBufs& a = st->adj;
     // fields of the state psi^n (the input of the step being reversed)
     k_collide<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b, 0);
-    k_mu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b);
+    launch_mu(m, st->phys, b, grid_for(m.N, kBlock), kBlock, s);
     k_gradmu<<<grid_for(m.T, kBlock), kBlock, 0, s>>>(m, b);
     // lambda_RHS = M11^{-1} lambda with the step's solver
     FELBM_CUDA(cudaMemcpyAsync(b.rhs, a.lam, sizeof(double) * 18 * m.Np, cudaMemcpyDeviceToDevice, s));

@@ -105,10 +105,9 @@ __device__ __forceinline__ void block_fetch(BlockSmem& sm, const DevMesh& m, con
 // The K steps of plane p, whose copies into x[buf] and b were queued by this
 // thread; queues those of plane `next` (kPlanes: none) into the third buffer,
 // which it returns.
-template <int NV, int kW, int kFinal, bool kFromRhs>
-__device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* __restrict__ cur,
-                                           float* nxt, const BlockTau& bt, int K, float tau0, int have_x64, int p,
-                                           int next, int buf, const int (&node)[kBlockNpt],
+template <int NV, int kW, bool kFromRhs>
+__device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* cur,
+                                           float* nxt, const BlockTau& bt, int K, float tau0, int p, int next, int buf, const int (&node)[kBlockNpt],
                                            const float (&val)[kBlockNpt][kW], const uint32_t (&col)[kBlockNpt][kW / 2],
                                            const float (&im)[kBlockNpt]) {
     const int Np = m.Np, tid = (int)threadIdx.x;
@@ -161,22 +160,10 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
                 const float s = tau * im[n];
 #pragma unroll
                 for (int c = 0; c < NV; ++c) x[n][c] = fmaf(s, rr[n][c] - acc[c], x[n][c]);
-                if (step < K) {
+                if (step < K)
                     store_shared(xb + r * NV, x[n]);
-                } else if constexpr (kFinal == kStore) {
+                else
                     store_vec(nxt, Np, p, node[n], x[n]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < NV; ++c) {
-                        const int q = NV == 2 ? 9 * c : 9 * (p >> 1) + 1 + 4 * (p & 1) + c;
-                        const int at = q * Np + node[n];
-                        const double v = have_x64 ? b.x64[at] + (double)x[n][c] : (double)x[n][c];
-                        if (kFinal == kAddPsi)
-                            b.psi[at] += v;
-                        else
-                            b.x64[at] = v;
-                    }
-                }
             }
         }
         if (step < K) __syncthreads();
@@ -187,13 +174,12 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
     return free;
 }
 
-// kW: ELL width; kFinal: where the last iterate goes (kStore: nxt); kFromRhs:
-// x_0 = tau_0 b / m formed here.  Grid: blocks x (1 or kPlanes): all planes of
+// kW: ELL width; kFromRhs: x_0 = tau_0 b / m formed here.  Grid: blocks x (1 or kPlanes): all planes of
 // a block in turn, or one.
-template <int kW, int kFinal, bool kFromRhs>
+template <int kW, bool kFromRhs>
 __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
-    k_block32(DevMesh m, Bufs b, const float* __restrict__ cur, float* nxt, const __grid_constant__ BlockTau bt, int K, float tau0,
-              int have_x64) {
+    k_block32(DevMesh m, Bufs b, const float* cur, float* nxt, const __grid_constant__ BlockTau bt, int K,
+              float tau0) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BlockSmem& sm = *reinterpret_cast<BlockSmem*>(smem_raw);
     pdl_release();
@@ -233,15 +219,15 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
     }
     int buf = 0;
     for (int p = p0; p < min(p1, 4); ++p)
-        buf = block_plane<4, kW, kFinal, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, have_x64, p,
+        buf = block_plane<4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, p,
                                                    p + 1 < p1 ? p + 1 : kPlanes, buf, node, val, col, im);
     if (p1 == kPlanes)
-        block_plane<2, kW, kFinal, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, have_x64, 4, kPlanes, buf, node, val, col, im);
+        block_plane<2, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, 4, kPlanes, buf, node, val, col, im);
 }
 
 // The field and deviation update from the solve's last iterate (FP32-deviation
 // states): psi^{n+1} = psi_hat + d.
-__global__ void __launch_bounds__(128) k_update32(DevMesh m, Phys c, Bufs b, const float* __restrict__ x) {
+__global__ void __launch_bounds__(128) k_update32(DevMesh m, Phys c, Bufs b, const float* x) {
     pdl_release();
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
