@@ -614,10 +614,11 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
     }
 }
 
-// First iterate for a standalone solve: x1 = first_scale * B / m_i
-// (1/theta for the FP64 recurrence, tau_0 for the FP32 steps).
+// Start of a standalone solve for the right-hand sides src ([18][Np], copied
+// to rhs): x1 = first_scale * B / m_i (1/theta for the FP64 recurrence, tau_0
+// for the FP32 steps).
 template <bool kMixed>
-__global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, double first_scale) {
+__global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, const double* src, double first_scale) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
     const int Np = m.Np;
@@ -625,7 +626,11 @@ __global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, double
     double acc[18];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        acc[q] = b.rhs[q * Np + i];
+        acc[q] = src[q * Np + i];
+    }
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        if (src != b.rhs) b.rhs[q * Np + i] = acc[q];
         if (!kMixed) b.x1[q * Np + i] = acc[q] * s;
     }
     if constexpr (kMixed) store_start(b, Np, i, acc, (float)s);
@@ -2858,9 +2863,9 @@ int felbm_mass_solve(felbm_state* st, const double* B, double* X, int32_t k) {
     k_scatter_in<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b.stage, b.rhs, k);
     if (k < 18) k_zero_rows<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b.rhs, k, 18);
     if (st->mode == FELBM_SOLVER_FP64)
-        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, st->inv_theta);
+        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, b.rhs, st->inv_theta);
     else
-        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, st->tau[0]);
+        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, b.rhs, st->tau[0]);
     const double* result = enqueue_solve(st, st->dm, b, s, false);
     k_gather_out<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, result, b.stage, k);
     FELBM_CUDA(cudaGetLastError());
@@ -2946,9 +2951,9 @@ int felbm_mass_solve_static(felbm_state* st, const double* d_B, double* d_X, int
     k_scatter_in<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, d_B, sb.rhs, k);
     if (k < 18) k_zero_rows<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb.rhs, k, 18);
     if (st->mode == FELBM_SOLVER_FP64)
-        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, st->inv_theta);
+        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, sb.rhs, st->inv_theta);
     else
-        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, st->tau[0]);
+        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, sb.rhs, st->tau[0]);
     const double* result = enqueue_solve(st, st->dm, sb, s, false);
     k_gather_out<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, result, d_X, k);
     FELBM_CUDA(cudaGetLastError());
@@ -3233,21 +3238,22 @@ int felbm_adjoint_step(felbm_state* st) {
     const DevMesh& m = st->dm;
     Bufs& b = st->buf;
     AdjBufs& a = st->adj;
+    const int nb = fp64_block(st, m.N, 128), tb = fp64_block(st, m.T, 128);
+    const unsigned ng = grid_for(m.N, nb), tg = grid_for(m.T, tb);
     // fields of the state psi^n (the input of the step being reversed)
-    k_collide<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b, 0);
-    launch_mu(m, st->phys, b, grid_for(m.N, kBlock), kBlock, s);
-    k_gradmu<<<grid_for(m.T, kBlock), kBlock, 0, s>>>(m, b);
+    k_collide<<<ng, nb, 0, s>>>(m, st->phys, b, 0);
+    launch_mu(m, st->phys, b, ng, nb, s);
+    k_gradmu<<<tg, tb, 0, s>>>(m, b);
     // lambda_RHS = M11^{-1} lambda with the step's solver
-    FELBM_CUDA(cudaMemcpyAsync(b.rhs, a.lam, sizeof(double) * 18 * m.Np, cudaMemcpyDeviceToDevice, s));
     if (st->mode == FELBM_SOLVER_FP64)
-        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, st->inv_theta);
+        k_cheb_start<false><<<ng, nb, 0, s>>>(m, b, a.lam, st->inv_theta);
     else
-        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, st->tau[0]);
+        k_cheb_start<true><<<ng, nb, 0, s>>>(m, b, a.lam, st->tau[0]);
     a.lamRHS = enqueue_solve(st, m, b, s, false);
-    k_adj_elem_a<<<grid_for(m.T, 128), 128, 0, s>>>(m, st->phys, b, a);
-    k_adj_elem_b<<<grid_for(m.T, kBlock), kBlock, 0, s>>>(m, a);
-    k_adj_node_d<<<grid_for(m.N, 128), 128, 0, s>>>(m, st->phys, a);
-    k_adj_node_e<<<grid_for(m.N, 128), 128, 0, s>>>(m, st->phys, b, a);
+    k_adj_elem_a<<<tg, tb, 0, s>>>(m, st->phys, b, a);
+    k_adj_elem_b<<<tg, tb, 0, s>>>(m, a);
+    k_adj_node_d<<<ng, nb, 0, s>>>(m, st->phys, a);
+    k_adj_node_e<<<ng, nb, 0, s>>>(m, st->phys, b, a);
     FELBM_CUDA(cudaGetLastError());
     return FELBM_OK;
 }
