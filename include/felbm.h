@@ -428,8 +428,8 @@ typedef struct felbm_step_timing {
     float collide_ms;   /* moments and collision */
     float mu_ms;        /* chemical potential with the wetting flux */
     float gradmu_ms;    /* P0 gradient of mu */
-    float element_ms;   /* element Laplacian of mu, forces, element residual */
-    float rhs_ms;       /* streaming right-hand-side gather */
+    float element_ms;   /* element Laplacian of mu, forces, element residual (FP32_DEV on larger meshes: and the gather) */
+    float rhs_ms;       /* streaming right-hand-side gather (near 0 where element_ms covers it) */
     float solve_ms;     /* all sweeps of the mass solve */
     float total_ms;
     int32_t solve_launches;  /* kernel launches inside solve_ms */

@@ -98,6 +98,10 @@ struct DevMesh {
     int32_t n_blocks;         // node blocks (contiguous id ranges, HostMesh::blk_ptr)
     int32_t blk_steps;        // most steps of the blocked solve per launch (layers around the blocks), 0 = not blocked
     const int32_t* blk_ptr;   // [n_blocks + 1]
+    const int32_t* blk_tri_ptr; // [n_blocks + 1] triangles at the nodes of each block
+    const int32_t* blk_tri;
+    int32_t max_blk_tri;
+    const uint16_t* iell_loc; // [iell_w][Np] iell_tri as indices into the block's triangle list (padding: past its end)
     const int32_t* blk_cnt;   // [n_blocks][kBlockSteps + 1] nodes of a block and its first l layers
     const int32_t* blk_halo_ptr; // [n_blocks + 1]
     const int32_t* blk_halo;  // the layers' nodes, layer by layer
@@ -165,7 +169,7 @@ struct Bufs {
     float* e0;       // [18 Np] FP32 iterates
     float* e1;
     // FP32-deviation storage (precision FELBM_FP32_DEV); C above stays FP64
-    float* dpsi;     // deviations from equilibrium: [Np][16] rows (q = 1..8 of g, h), then [2][Np] (q = 0)
+    float* dpsi;     // [18 Np] deviations from equilibrium (layout: vec_at)
     float* p32;      // [Np]
     float* ux32;
     float* uy32;
@@ -217,6 +221,28 @@ __device__ __forceinline__ void store_vec(float* x, int Np, int p, int i, const 
     else
         reinterpret_cast<float2*>(x + (size_t)16 * Np)[i] = make_float2(v[0], v[1]);
 }
+template <int NV>
+__device__ __forceinline__ void load_shared(float (&v)[NV], const float* x) {
+    if constexpr (NV == 4) {
+        const float4 t = *reinterpret_cast<const float4*>(x);
+        v[0] = t.x;
+        v[1] = t.y;
+        v[2] = t.z;
+        v[3] = t.w;
+    } else {
+        const float2 t = *reinterpret_cast<const float2*>(x);
+        v[0] = t.x;
+        v[1] = t.y;
+    }
+}
+template <int NV>
+__device__ __forceinline__ void store_shared(float* x, const float (&v)[NV]) {
+    if constexpr (NV == 4)
+        *reinterpret_cast<float4*>(x) = make_float4(v[0], v[1], v[2], v[3]);
+    else
+        *reinterpret_cast<float2*>(x) = make_float2(v[0], v[1]);
+}
+
 // All 18 values of node i, indexed by q18.
 __device__ __forceinline__ void load_all(float (&d)[18], const float* x, int Np, int i) {
 #pragma unroll
@@ -1122,9 +1148,10 @@ __device__ __forceinline__ void diag_node(const DevMesh& m, const Phys& c, const
         const float uuf = uxf * uxf + uyf * uyf;
         uu = uuf;
         ruu = rhof * uuf;
-        float dsum = 0.0f;
+        float dsum = 0.0f, dev[18];
+        load_all(dev, b.dpsi, Np, i);
 #pragma unroll
-        for (int q = 0; q < 18; ++q) dsum += b.dpsi[dpsi_at(Np, q, i)];
+        for (int q = 0; q < 18; ++q) dsum += dev[q];
         // non-finite deviations are reported too
         finite = finite_bits(C) && isfinite(b.p32[i]) && isfinite(uuf) && isfinite(dsum);
     } else {
@@ -1568,6 +1595,10 @@ static size_t carve(const HostMesh& h, bool dev32, void* base, DevMesh* dm, Bufs
     d.iell_tri = cv.take<int32_t>((size_t)std::max(iw, 1) * Np);
     d.iell_bx32 = cv.take<float>((size_t)std::max(iw, 1) * Np);
     d.iell_by32 = cv.take<float>((size_t)std::max(iw, 1) * Np);
+    d.max_blk_tri = dev32 && iw > 0 && h.max_blk_tri <= kForceTris ? h.max_blk_tri : 0;   // 0: k_force32 unused
+    d.blk_tri_ptr = cv.take<int32_t>(h.blk_tri_ptr.size());
+    d.blk_tri = cv.take<int32_t>(d.max_blk_tri > 0 ? h.blk_tri.size() : 1);
+    d.iell_loc = cv.take<uint16_t>(d.max_blk_tri > 0 ? (size_t)iw * Np : 1);
     d.inv_lumped32 = cv.take<float>(Np);
     d.lumped = cv.take<double>(Np);
     d.inv_vol = cv.take<double>(Np);
@@ -1975,7 +2006,18 @@ static int solve_launches(const felbm_state* st) {
     return refines * (groups(st->sweeps - 1) + 1) + last + 1;
 }
 
-static int step_launches(const felbm_state* st) { return (st->dev32 ? 4 : 5) + solve_launches(st); }
+// FP32 states: residuals and their gather in one kernel (k_force32) from this
+// many blocks per multiprocessor on; below, 384 threads a block leave most of
+// the device idle (11,615 nodes: 45 us a step fused, 43 us not; the figures for
+// large meshes stand at the kernel).
+constexpr int kFuseForcesFrom = 1;
+static bool fused_forces(const felbm_state* st, const DevMesh& m) {
+    return st->dev32 && m.max_blk_tri > 0 && m.n_blocks >= kFuseForcesFrom * st->n_sm;
+}
+
+static int step_launches(const felbm_state* st) {
+    return (st->dev32 ? (fused_forces(st, st->dm) ? 3 : 4) : 5) + solve_launches(st);
+}
 
 int set_schedule(felbm_state* st, int32_t max_nodes);
 
@@ -2023,12 +2065,23 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
             else
                 launch_k(chain, k_gradmu32, dim3(grid_for(mt.T, kBlock)), dim3(kBlock), 0, s, mt, b);
             mark(3);
-            launch_k(chain, k_element32, dim3(grid_for(mt.T, 128)), dim3(128), 0, s, mt, st->phys, b);
-            mark(4);
             const bool from_rhs = first_from_rhs(st, mt);
             const float tau0 = (float)st->tau[0];
+            // residuals and their gather in one kernel where the blocks fill the device
+            const bool fused = fused_forces(st, mt);
+            if (fused) {
+                const size_t smem = force_smem_bytes(mt.max_blk_tri);
+                const auto go = [&](auto kern) {
+                    launch_k(chain, kern, dim3(mt.n_blocks), dim3(kForceThreads), smem, s, mt, st->phys, b, tau0,
+                             from_rhs ? 0 : 1);
+                };
+                mt.iell_w == 6 ? go(k_force32<6>) : mt.iell_w == 8 ? go(k_force32<8>) : go(k_force32<12>);
+            } else {
+                launch_k(chain, k_element32, dim3(grid_for(mt.T, 128)), dim3(128), 0, s, mt, st->phys, b);
+            }
+            mark(4);
             const dim3 gn(grid_for(mt.N, 128)), bn(128);
-            switch (mt.iell_w * 2 + (from_rhs ? 1 : 0)) {
+            if (!fused) switch (mt.iell_w * 2 + (from_rhs ? 1 : 0)) {
                 case 12: launch_k(chain, k_rhs32<6, true>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
                 case 13: launch_k(chain, k_rhs32<6, false>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
                 case 16: launch_k(chain, k_rhs32<8, true>, gn, bn, 0, s, mt, st->phys, b, tau0); break;
@@ -2344,6 +2397,30 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
                 ibx[at] = inc_bx32[k];
                 iby[at] = inc_by32[k];
             }
+        std::vector<uint16_t> iloc;
+        if (st->dm.max_blk_tri > 0) {
+            iloc.resize((size_t)iw * Npi);
+            parallel_for(nblk, 32, []() { return 0; }, [&](int32_t t, int&) {
+                const int32_t* l0 = h.blk_tri.data() + h.blk_tri_ptr[t];
+                const int32_t* l1 = h.blk_tri.data() + h.blk_tri_ptr[t + 1];
+                for (int32_t i = h.blk_ptr[t]; i < h.blk_ptr[t + 1]; ++i)
+                    for (int k = 0; k < iw; ++k) {
+                        const int32_t tri = itri[(size_t)k * Npi + i];
+                        iloc[(size_t)k * Npi + i] = (uint16_t)(tri < h.T ? std::lower_bound(l0, l1, tri) - l0 : l1 - l0);
+                    }
+            });
+            UP(d.blk_tri_ptr, h.blk_tri_ptr);
+            UP(d.blk_tri, h.blk_tri);
+            UP(d.iell_loc, iloc);
+            // (the limit holds for every state of the process: the largest any may ask for)
+            const int bytes = (int)force_smem_bytes(kForceTris);
+            const auto allow = [&](auto kern) {
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            };
+            allow(k_force32<6>);
+            allow(k_force32<8>);
+            allow(k_force32<12>);
+        }
         UP(d.iell_tri, itri);
         UP(d.iell_bx32, ibx);
         UP(d.iell_by32, iby);

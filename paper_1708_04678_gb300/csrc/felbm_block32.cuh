@@ -45,28 +45,6 @@ struct BlockTau {
     float tau[kBlockSteps];
 };
 
-template <int NV>
-__device__ __forceinline__ void load_shared(float (&v)[NV], const float* x) {
-    if constexpr (NV == 4) {
-        const float4 t = *reinterpret_cast<const float4*>(x);
-        v[0] = t.x;
-        v[1] = t.y;
-        v[2] = t.z;
-        v[3] = t.w;
-    } else {
-        const float2 t = *reinterpret_cast<const float2*>(x);
-        v[0] = t.x;
-        v[1] = t.y;
-    }
-}
-template <int NV>
-__device__ __forceinline__ void store_shared(float* x, const float (&v)[NV]) {
-    if constexpr (NV == 4)
-        *reinterpret_cast<float4*>(x) = make_float4(v[0], v[1], v[2], v[3]);
-    else
-        *reinterpret_cast<float2*>(x) = make_float2(v[0], v[1]);
-}
-
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 template <int NV>
 __device__ __forceinline__ void cp_async_vec(float* dst, const float* x, int Np, int p, int i) {

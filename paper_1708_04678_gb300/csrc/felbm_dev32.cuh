@@ -17,15 +17,10 @@
 //    FP64) and the deviations in place.
 #pragma once
 
-// Layout of the deviations (18 Np floats): the moving populations q = 1..8
-// of g and then of h as one 64-byte row per node (dpsi + 16 i), so that a
-// gather of a vertex's 16 values is four 16-byte loads; the rest populations
-// (q = 0) of g and of h after all rows, one value per node each.
-// q18 = q for g, 9 + q for h.
-__device__ __forceinline__ size_t dpsi_at(int Np, int q18, int i) {
-    const int part = q18 >= 9 ? 1 : 0, q = q18 - 9 * part;
-    return q == 0 ? (size_t)(16 + part) * Np + i : (size_t)i * 16 + part * 8 + (q - 1);
-}
+// The deviations are stored in the planes of vec_at: consecutive vertices of
+// consecutive triangles are consecutive 16-byte words, so a warp's gather of a
+// plane touches 3 or 4 lines.  With one 64-byte row per node each 16-byte load
+// of a warp touched 16.
 
 // omega = 1 / (tau + 1/2), 1/tau = C/tau_l + (1-C)/tau_v (Sec. II.A)
 __device__ __forceinline__ float omega32(float C, const Phys& c) {
@@ -134,8 +129,8 @@ __global__ void __launch_bounds__(kBlock) k_gradmu32(DevMesh m, Bufs b) {
 // ------------------------------- forces and element residual (FP32) ------
 // R_a = A (Phi_a - e_a . grad psi_hat_a), psi_hat = psi^eq + (1 - omega) dpsi,
 // gradients formed from differences to vertex 0 (sum of the b_v is zero).
-__device__ __forceinline__ void element32_tri(const DevMesh& m, const Phys& c, const Bufs& b, int t) {
-    const int Tp = m.Tp, Np = m.Np;
+__device__ __forceinline__ void element32_out(const DevMesh& m, const Phys& c, const Bufs& b, int t, float (&out)[18]) {
+    const int Tp = m.Tp;
     int v[3];
     float bx[3], by[3];
 #pragma unroll
@@ -162,8 +157,6 @@ __device__ __forceinline__ void element32_tri(const DevMesh& m, const Phys& c, c
     om1[1] = 1.0f - omega32(C0 + dC1, c);
     om1[2] = 1.0f - omega32(C0 + dC2, c);
     const float third = 1.0f / 3.0f;
-    const float pb = (p[0] + p[1] + p[2]) * third;
-    (void)pb;
     const float ubx = (ux[0] + ux[1] + ux[2]) * third, uby = (uy[0] + uy[1] + uy[2]) * third;
     const float mub = mus * third;
     const float gCx = dC1 * bx[1] + dC2 * bx[2], gCy = dC1 * by[1] + dC2 * by[2];
@@ -182,72 +175,97 @@ __device__ __forceinline__ void element32_tri(const DevMesh& m, const Phys& c, c
     }
     const float drho = c.drho_f;
     const float rhob = c.rho_v_f + Cb * drho;
-    const float rho0 = c.rho_v_f + C0 * drho;
-    const float grx = drho * gCx, gry = drho * gCy;
     const float f = 3.0f * Cb / rhob;
     const float vhx = gCx - f * (gpx - mub * gCx), vhy = gCy - f * (gpy - mub * gCy);
-    const float u_gr = ubx * grx + uby * gry, u_gC = ubx * gCx + uby * gCy, u_vh = ubx * vhx + uby * vhy;
+    // Forces as in k_element: with T = Gamma / w - 1, A Phi_g = w s (P + Q T) and
+    // A Phi_h = w A ((e - u).v + M lap mu)(1 + T), the axis weight folded into the vectors.
     const float uub15 = 1.5f * (ubx * ubx + uby * uby);
-    const float Mlap = c.mobility_f * lapmu;
-    // vertex velocity differences to vertex 0
-    const float du1x = ux[1] - ux[0], du1y = uy[1] - uy[0], su1x = ux[1] + ux[0], su1y = uy[1] + uy[0];
-    const float du2x = ux[2] - ux[0], du2y = uy[2] - uy[0], su2x = ux[2] + ux[0], su2y = uy[2] + uy[0];
+    const float w1 = 1.0f / 9.0f, Aw = A * w1, P = A * mub, Q = fmaf(A * third, drho, P);
+    const float sx = w1 * gCx, sy = w1 * gCy, su = ubx * sx + uby * sy;
+    const float vx = Aw * vhx, vy = Aw * vhy, vu = ubx * vx + uby * vy - Aw * (c.mobility_f * lapmu);
+    // Differences of the equilibria to vertex 0, k = 1, 2:
+    //   h: w ((1 + T_0) dC_k + C_k dT_k),  g: w (dp_k + (drho_k T_0 + rho_k dT_k) / 3),
+    //   dT_k = 3 e.du_k + 4.5 (e.du_k)(e.su_k) - 1.5 du_k.su_k, su_k = u_k + u_0
     const float uu0 = 1.5f * (ux[0] * ux[0] + uy[0] * uy[0]);
-    const float drho1 = drho * dC1, drho2 = drho * dC2;
+    const float dC[2] = {dC1, dC2}, dp[2] = {dp1, dp2};
+    float dux[2], duy[2], sux[2], suy[2], D[2], Ck[2], rk[2], dr[2], abx[2], aby[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        dux[k] = ux[k + 1] - ux[0];
+        duy[k] = uy[k + 1] - uy[0];
+        sux[k] = ux[k + 1] + ux[0];
+        suy[k] = uy[k + 1] + uy[0];
+        D[k] = -1.5f * (dux[k] * sux[k] + duy[k] * suy[k]);
+        Ck[k] = C0 + dC[k];
+        dr[k] = drho * third * dC[k];
+        rk[k] = third * (c.rho_v_f + C0 * drho) + dr[k];
+        abx[k] = A * bx[k + 1];
+        aby[k] = A * by[k + 1];
+    }
     // the post-collision deviations of the three vertices, all loaded first
-    // (each vertex's row: four 16-byte loads)
+    // (the rest populations do not enter)
     float pg[3][9], ph[3][9];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float4* row = reinterpret_cast<const float4*>(b.dpsi + (size_t)v[k] * 16);
-        const float4 a0 = row[0], a1 = row[1], a2 = row[2], a3 = row[3];
-        pg[k][1] = a0.x; pg[k][2] = a0.y; pg[k][3] = a0.z; pg[k][4] = a0.w;
-        pg[k][5] = a1.x; pg[k][6] = a1.y; pg[k][7] = a1.z; pg[k][8] = a1.w;
-        ph[k][1] = a2.x; ph[k][2] = a2.y; ph[k][3] = a2.z; ph[k][4] = a2.w;
-        ph[k][5] = a3.x; ph[k][6] = a3.y; ph[k][7] = a3.z; ph[k][8] = a3.w;
-    }
-    float out[18];
-#define FELBM_ELEM32_Q(q)                                                                          \
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            float g4[4], h4[4];
+            load_vec(g4, b.dpsi, m.Np, j, v[k]);
+            load_vec(h4, b.dpsi, m.Np, 2 + j, v[k]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                pg[k][1 + 4 * j + e] = g4[e];
+                ph[k][1 + 4 * j + e] = h4[e];
+            }
+        }
+    out[0] = -4.0f * su * fmaf(Q, -uub15, P);
+    out[9] = -4.0f * fmaf(vu, -uub15, vu);
+    // a direction and its opposite together: e.u changes sign, the squares do not
+#define FELBM_ELEM32_PAIR(q, fw)                                                                   \
     {                                                                                              \
         const float w = (float)wq(q);                                                              \
-        const float G = gamma32<q>(ubx, uby, uub15);                                               \
-        const float phig = third * (G - w) * (edot<q, float>(grx, gry) - u_gr) + mub * G * (edot<q, float>(gCx, gCy) - u_gC); \
-        const float phih = ((edot<q, float>(vhx, vhy) - u_vh) + Mlap) * G;                               \
-        float dg = 0.0f, dh = 0.0f;                                                                \
-        if (q != 0) {                                                                              \
-            const float G0 = gamma32<q>(ux[0], uy[0], uu0);                                        \
-            const float dG1 = dgamma32<q>(du1x, du1y, su1x, su1y);                                 \
-            const float dG2 = dgamma32<q>(du2x, du2y, su2x, su2y);                                 \
-            /* differences of the equilibria to vertex 0 */                                       \
-            const float dhe1 = (G0 + dG1) * dC1 + C0 * dG1, dhe2 = (G0 + dG2) * dC2 + C0 * dG2;     \
-            const float dge1 = w * dp1 + third * (drho1 * (G0 + dG1 - w) + rho0 * dG1);            \
-            const float dge2 = w * dp2 + third * (drho2 * (G0 + dG2 - w) + rho0 * dG2);            \
-            /* differences of the post-collision deviations */                                     \
-            const float g0 = om1[0] * pg[0][q], h0 = om1[0] * ph[0][q];                            \
-            const float dgd1 = om1[1] * pg[1][q] - g0;                                             \
-            const float dgd2 = om1[2] * pg[2][q] - g0;                                             \
-            const float dhd1 = om1[1] * ph[1][q] - h0;                                             \
-            const float dhd2 = om1[2] * ph[2][q] - h0;                                             \
-            const float eb1 = edot<q, float>(bx[1], by[1]), eb2 = edot<q, float>(bx[2], by[2]);                  \
-            dg = (dge1 + dgd1) * eb1 + (dge2 + dgd2) * eb2;                                        \
-            dh = (dhe1 + dhd1) * eb1 + (dhe2 + dhd2) * eb2;                                        \
+        const float eu = edot<q, float>(ubx, uby), t2 = fmaf(4.5f * eu, eu, -uub15);               \
+        const float tp = fmaf(3.0f, eu, t2), tm = fmaf(-3.0f, eu, t2);                             \
+        const float es = edot<q, float>((fw) * sx, (fw) * sy), ev = edot<q, float>((fw) * vx, (fw) * vy); \
+        const float vp = ev - (fw) * vu, vm = -ev - (fw) * vu;                                     \
+        float gp = (es - (fw) * su) * fmaf(Q, tp, P), gm = (-es - (fw) * su) * fmaf(Q, tm, P);     \
+        float hp = fmaf(vp, tp, vp), hm = fmaf(vm, tm, vm);                                        \
+        const float e0 = edot<q, float>(ux[0], uy[0]), z2 = fmaf(4.5f * e0, e0, -uu0);             \
+        const float zp = fmaf(3.0f, e0, z2), zm = fmaf(-3.0f, e0, z2);                             \
+        const float g0p = om1[0] * pg[0][q], g0m = om1[0] * pg[0][opp(q)];                         \
+        const float h0p = om1[0] * ph[0][q], h0m = om1[0] * ph[0][opp(q)];                         \
+        _Pragma("unroll") for (int k = 0; k < 2; ++k) {                                            \
+            const float ed = edot<q, float>(dux[k], duy[k]), es2 = edot<q, float>(sux[k], suy[k]); \
+            const float d2 = fmaf(4.5f * ed, es2, D[k]);                                           \
+            const float dTp = fmaf(3.0f, ed, d2), dTm = fmaf(-3.0f, ed, d2);                       \
+            const float eb = edot<q, float>(abx[k], aby[k]);                                       \
+            const float gqp = fmaf(dTp, rk[k], fmaf(zp, dr[k], dp[k])), gqm = fmaf(dTm, rk[k], fmaf(zm, dr[k], dp[k])); \
+            const float hqp = fmaf(dTp, Ck[k], fmaf(zp, dC[k], dC[k])), hqm = fmaf(dTm, Ck[k], fmaf(zm, dC[k], dC[k])); \
+            gp = fmaf(-eb, fmaf(w, gqp, fmaf(om1[k + 1], pg[k + 1][q], -g0p)), gp);                \
+            gm = fmaf(eb, fmaf(w, gqm, fmaf(om1[k + 1], pg[k + 1][opp(q)], -g0m)), gm);            \
+            hp = fmaf(-eb, fmaf(w, hqp, fmaf(om1[k + 1], ph[k + 1][q], -h0p)), hp);                \
+            hm = fmaf(eb, fmaf(w, hqm, fmaf(om1[k + 1], ph[k + 1][opp(q)], -h0m)), hm);            \
         }                                                                                          \
-        out[q] = A * (phig - dg);                                                                  \
-        out[9 + q] = A * (phih - dh);                                                              \
+        out[q] = gp;                                                                               \
+        out[opp(q)] = gm;                                                                          \
+        out[9 + (q)] = hp;                                                                         \
+        out[9 + opp(q)] = hm;                                                                      \
     }
-    FELBM_ELEM32_Q(0) FELBM_ELEM32_Q(1) FELBM_ELEM32_Q(2) FELBM_ELEM32_Q(3) FELBM_ELEM32_Q(4)
-    FELBM_ELEM32_Q(5) FELBM_ELEM32_Q(6) FELBM_ELEM32_Q(7) FELBM_ELEM32_Q(8)
-#undef FELBM_ELEM32_Q
+    FELBM_ELEM32_PAIR(1, 1.0f) FELBM_ELEM32_PAIR(2, 1.0f) FELBM_ELEM32_PAIR(5, 0.25f) FELBM_ELEM32_PAIR(6, 0.25f)
+#undef FELBM_ELEM32_PAIR
+}
+
+__device__ __forceinline__ void element32_tri(const DevMesh& m, const Phys& c, const Bufs& b, int t) {
+    float out[18];
+    element32_out(m, c, b, t, out);
     float2* dst = reinterpret_cast<float2*>(b.R32 + (size_t)t * 18);
 #pragma unroll
     for (int k = 0; k < 9; ++k) dst[k] = make_float2(out[2 * k], out[2 * k + 1]);
 }
 
-// The vertices' 48 deviation values are all loaded (as twelve 16-byte row
-// loads) before the per-direction arithmetic, so that they are in flight
-// together; 80 registers (6 blocks of 128 per SM).  On the 2.08M-node rough
-// wall: 0.229 ms, against 0.300 ms with one array per population and 0.324
-// ms with the loads inside the arithmetic at 64 registers.
+// The vertices' 48 deviation values are all loaded (as twelve 16-byte loads)
+// before the per-direction arithmetic, so that they are in flight together; 80
+// registers (6 blocks of 128 per SM).  Runs where k_force32 does not.
 __global__ void __launch_bounds__(128, 6) k_element32(DevMesh m, Phys c, Bufs b) {
     pdl_release();
     pdl_wait();
@@ -259,6 +277,42 @@ __global__ void __launch_bounds__(128, 6) k_element32(DevMesh m, Phys c, Bufs b)
 // As k_rhs; the wall term needs psi_hat_opp - psi_hat at a node, which in the
 // split form is  g: -2 w rho (e.u) + (1-omega)(dg_opp - dg),
 //                h: -6 w C (e.u)   + (1-omega)(dh_opp - dh).
+// What the weak bounce-back of a wall edge reads at one of its ends.
+struct WallEnd {
+    float C, ux, uy, om, rho;
+    float4 d[4];      // deviations (planes of vec_at)
+};
+template <int kP0, int kP1>
+__device__ __forceinline__ WallEnd wall_end(const Phys& c, const Bufs& b, int Np, int v) {
+    WallEnd e;
+    e.C = (float)b.C[v];
+    e.ux = b.ux32[v];
+    e.uy = b.uy32[v];
+#pragma unroll
+    for (int p = kP0; p < kP1; ++p) e.d[p] = reinterpret_cast<const float4*>(b.dpsi)[(size_t)p * Np + v];
+    e.om = 1.0f - omega32(e.C, c);
+    e.rho = c.rho_v_f + e.C * c.drho_f;
+    return e;
+}
+// psi_hat_opp - psi_hat of component k of plane p at one end; a direction's
+// opposite is two components further in the same plane.
+template <int kP, int k>
+__device__ __forceinline__ float wall_diff(const WallEnd& e) {
+    constexpr int q = 1 + 4 * (kP & 1) + k;
+    static_assert(opp(q) == 1 + 4 * (kP & 1) + (k ^ 2), "opposites share a plane");
+    const float w = (float)wq(q), eu = edot<q, float>(e.ux, e.uy);
+    const float4 d = e.d[kP];
+    const float dev = k == 0 ? d.z - d.x : k == 1 ? d.w - d.y : k == 2 ? d.x - d.z : d.y - d.w;
+    return (kP < 2 ? -2.0f * w * e.rho * eu : -6.0f * w * e.C * eu) + e.om * dev;
+}
+// The term of component k of plane p: zero for the outgoing directions.
+template <int kP, int k>
+__device__ __forceinline__ float wall32(const Phys& c, const WallEnd& i, const WallEnd& o, float L, float nx, float ny) {
+    const float en = edot<1 + 4 * (kP & 1) + k, float>(nx, ny);
+    if (!(en < 0.0f)) return 0.0f;
+    return -c.dt_f * en * (L * (1.0f / 3.0f) * wall_diff<kP, k>(i) + L * (1.0f / 6.0f) * wall_diff<kP, k>(o));
+}
+
 // kI > 0: the incident triangles from the incidence ELL (padding: the zero
 // residual row T), their ids and gradients loaded up front; kI = 0: CSR.
 template <int kI = 0, bool kFirst = true>
@@ -311,35 +365,18 @@ __device__ __forceinline__ void rhs32_node(const DevMesh& m, const Phys& c, cons
         FELBM_RHS32_Q(5) FELBM_RHS32_Q(6) FELBM_RHS32_Q(7) FELBM_RHS32_Q(8)
 #undef FELBM_RHS32_Q
     }
-    if (m.winc_ptr[i] < m.winc_ptr[i + 1]) {
-        const float drho = c.drho_f;
-        for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
-            int e = m.winc_edge[k];
-            int o = m.wall_a[e] == i ? m.wall_b[e] : m.wall_a[e];
-            float L = (float)m.wall_len[e], nx = (float)m.wall_nx[e], ny = (float)m.wall_ny[e];
-            float Ci = (float)b.C[i], Co = (float)b.C[o];
-            float rhoi = c.rho_v_f + Ci * drho, rhoo = c.rho_v_f + Co * drho;
-            float omi = 1.0f - omega32(Ci, c), omo = 1.0f - omega32(Co, c);
-            float uxi = b.ux32[i], uyi = b.uy32[i], uxo = b.ux32[o], uyo = b.uy32[o];
-#define FELBM_WALL32_Q(q)                                                                           \
-            {                                                                                       \
-                float en = edot<q, float>(nx, ny);                                                         \
-                if (en < 0.0f) {                                                                    \
-                    const float w = (float)wq(q);                                                   \
-                    float f = -c.dt_f * en;                                                         \
-                    float eui = edot<q, float>(uxi, uyi), euo = edot<q, float>(uxo, uyo);                         \
-                    float dgi = -2.0f * w * rhoi * eui + omi * (b.dpsi[dpsi_at(Np, opp(q), i)] - b.dpsi[dpsi_at(Np, q, i)]); \
-                    float dgo = -2.0f * w * rhoo * euo + omo * (b.dpsi[dpsi_at(Np, opp(q), o)] - b.dpsi[dpsi_at(Np, q, o)]); \
-                    float dhi = -6.0f * w * Ci * eui + omi * (b.dpsi[dpsi_at(Np, (9 + opp(q)), i)] - b.dpsi[dpsi_at(Np, (9 + q), i)]); \
-                    float dho = -6.0f * w * Co * euo + omo * (b.dpsi[dpsi_at(Np, (9 + opp(q)), o)] - b.dpsi[dpsi_at(Np, (9 + q), o)]); \
-                    acc[q] += f * (L * (1.0f / 3.0f) * dgi + L * (1.0f / 6.0f) * dgo);              \
-                    acc[9 + q] += f * (L * (1.0f / 3.0f) * dhi + L * (1.0f / 6.0f) * dho);          \
-                }                                                                                   \
-            }
-            FELBM_WALL32_Q(1) FELBM_WALL32_Q(2) FELBM_WALL32_Q(3) FELBM_WALL32_Q(4)
-            FELBM_WALL32_Q(5) FELBM_WALL32_Q(6) FELBM_WALL32_Q(7) FELBM_WALL32_Q(8)
-#undef FELBM_WALL32_Q
-        }
+    for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
+        const int e = m.winc_edge[k];
+        const int o = m.wall_a[e] == i ? m.wall_b[e] : m.wall_a[e];
+        const float L = (float)m.wall_len[e], nx = (float)m.wall_nx[e], ny = (float)m.wall_ny[e];
+        const WallEnd ei = wall_end<0, 4>(c, b, Np, i), eo = wall_end<0, 4>(c, b, Np, o);
+#define FELBM_WALL32_P(p)                                                \
+        acc[vec_row(p, 0)] += wall32<p, 0>(c, ei, eo, L, nx, ny);        \
+        acc[vec_row(p, 1)] += wall32<p, 1>(c, ei, eo, L, nx, ny);        \
+        acc[vec_row(p, 2)] += wall32<p, 2>(c, ei, eo, L, nx, ny);        \
+        acc[vec_row(p, 3)] += wall32<p, 3>(c, ei, eo, L, nx, ny);
+        FELBM_WALL32_P(0) FELBM_WALL32_P(1) FELBM_WALL32_P(2) FELBM_WALL32_P(3)
+#undef FELBM_WALL32_P
     }
     float s = m.inv_lumped32[i] * tau0;
     store_all(b.r32, Np, i, acc);
@@ -357,6 +394,120 @@ __global__ void __launch_bounds__(128, 8) k_rhs32(DevMesh m, Phys c, Bufs b, flo
     pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m.N) rhs32_node<kI, kFirst>(m, c, b, i, tau0);
+}
+
+// -------------------- element residuals and their gather in one kernel ----
+// One node block (HostMesh::blk_ptr) per thread block: the residuals of the
+// triangles at its nodes go to shared memory, then two threads a node (one per
+// class of directions) gather them.  The same arithmetic as k_element32 and
+// k_rhs32 in the same order; the residuals, 72 bytes a triangle written and
+// gathered back through DRAM by those two, never leave the multiprocessor, for
+// about 10 % of the triangles formed twice.  Bound by load latency and L1 (48 %
+// of its wavefronts, 34 % of the issue slots, 24 warps at 80 registers): 337 us
+// on 2,082,816 nodes against 237 + 144 us for the two kernels, 31 against 22 +
+// 19 us on 131,072 nodes.  Two threads a triangle at 80 or 64 registers: 352
+// and 381 us; 256 threads a block: 416 us.  Residual rows hold the planes of
+// vec_at one after another, 20 floats apart (16-byte words of consecutive
+// triangles in different banks); the row after the last is zero (padding).
+constexpr int kForceThreads = 384;
+constexpr int kForceRow = 20;
+constexpr int kForceTris = 1400;       // two thread blocks' rows fit a multiprocessor's shared memory
+
+__host__ __device__ constexpr size_t force_smem_bytes(int max_tri) { return (size_t)(max_tri + 1) * kForceRow * 4; }
+
+// The gather of the planes kC and kC + 2 (one class of directions of g and of
+// h, which share the weights), with the rest populations in class 0.
+template <int kC, int kI>
+__device__ __forceinline__ void force32_gather(const DevMesh& m, const Phys& c, const Bufs& b, const float* R, int i,
+                                               float tau0, int first) {
+    const int Np = m.Np;
+    const float c1 = c.dt3_f, c2 = c.dt2h_f;
+    int tt[kI];
+    float bxx[kI], byy[kI];
+#pragma unroll
+    for (int k = 0; k < kI; ++k) {
+        tt[k] = m.iell_loc[k * Np + i];
+        bxx[k] = m.iell_bx32[k * Np + i];
+        byy[k] = m.iell_by32[k * Np + i];
+    }
+    const int w0 = m.winc_ptr[i], w1 = m.winc_ptr[i + 1];
+    float ag[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ah[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ar[2] = {0.0f, 0.0f};
+    constexpr int q0 = 1 + 4 * kC;
+#pragma unroll
+    for (int k = 0; k < kI; ++k) {
+        const float* row = R + tt[k] * kForceRow;
+        float rg[4], rh[4];
+        load_shared(rg, row + 4 * kC);
+        load_shared(rh, row + 8 + 4 * kC);
+        const float w[4] = {c1 + c2 * edot<q0, float>(bxx[k], byy[k]), c1 + c2 * edot<q0 + 1, float>(bxx[k], byy[k]),
+                            c1 + c2 * edot<q0 + 2, float>(bxx[k], byy[k]), c1 + c2 * edot<q0 + 3, float>(bxx[k], byy[k])};
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            ag[v] = fmaf(rg[v], w[v], ag[v]);
+            ah[v] = fmaf(rh[v], w[v], ah[v]);
+        }
+        if constexpr (kC == 0) {
+            float r0[2];
+            load_shared(r0, row + 16);
+            ar[0] = fmaf(r0[0], c1, ar[0]);
+            ar[1] = fmaf(r0[1], c1, ar[1]);
+        }
+    }
+    for (int k = w0; k < w1; ++k) {
+        const int e = m.winc_edge[k];
+        const int o = m.wall_a[e] == i ? m.wall_b[e] : m.wall_a[e];
+        const float L = (float)m.wall_len[e], nx = (float)m.wall_nx[e], ny = (float)m.wall_ny[e];
+        const WallEnd ei = wall_end<0, 4>(c, b, Np, i), eo = wall_end<0, 4>(c, b, Np, o);
+#define FELBM_FORCE_WALL(v)                                              \
+        ag[v] += wall32<kC, v>(c, ei, eo, L, nx, ny);                    \
+        ah[v] += wall32<kC + 2, v>(c, ei, eo, L, nx, ny);
+        FELBM_FORCE_WALL(0) FELBM_FORCE_WALL(1) FELBM_FORCE_WALL(2) FELBM_FORCE_WALL(3)
+#undef FELBM_FORCE_WALL
+    }
+    store_vec(b.r32, Np, kC, i, ag);
+    store_vec(b.r32, Np, kC + 2, i, ah);
+    if (kC == 0) store_vec(b.r32, Np, 4, i, ar);
+    if (first) {
+        const float s = m.inv_lumped32[i] * tau0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            ag[v] *= s;
+            ah[v] *= s;
+            if (v < 2) ar[v] *= s;
+        }
+        store_vec(b.e1, Np, kC, i, ag);
+        store_vec(b.e1, Np, kC + 2, i, ah);
+        if (kC == 0) store_vec(b.e1, Np, 4, i, ar);
+    }
+}
+
+template <int kI>
+__global__ void __launch_bounds__(kForceThreads, 2) k_force32(DevMesh m, Phys c, Bufs b, float tau0, int first) {
+    extern __shared__ __align__(16) float force_rows[];
+    float* R = force_rows;
+    pdl_release();
+    const int blk = (int)blockIdx.x, tid = (int)threadIdx.x;
+    const int t0 = m.blk_tri_ptr[blk], nt = m.blk_tri_ptr[blk + 1] - t0;
+    const int s0 = m.blk_ptr[blk], ni = m.blk_ptr[blk + 1] - s0;
+    if (tid < kForceRow) R[nt * kForceRow + tid] = 0.0f;
+    pdl_wait();
+    for (int r = tid; r < nt; r += kForceThreads) {
+        float out[18];
+        element32_out(m, c, b, m.blk_tri[t0 + r], out);
+        float* row = R + r * kForceRow;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            *reinterpret_cast<float4*>(row + 4 * p) =
+                make_float4(out[vec_row(p, 0)], out[vec_row(p, 1)], out[vec_row(p, 2)], out[vec_row(p, 3)]);
+        *reinterpret_cast<float2*>(row + 16) = make_float2(out[0], out[9]);
+    }
+    __syncthreads();
+    for (int w = tid; w < 2 * ni; w += kForceThreads) {
+        if (w < ni)
+            force32_gather<0, kI>(m, c, b, R, s0 + w, tau0, first);
+        else
+            force32_gather<1, kI>(m, c, b, R, s0 + w - ni, tau0, first);
+    }
 }
 
 // ---------------------------- update of fields and deviations (node) ------
@@ -390,28 +541,20 @@ __device__ __forceinline__ void dev32_update(const DevMesh& m, const Phys& c, co
     const float dux = uxn - ux, duy = uyn - uy, sux = uxn + ux, suy = uyn + uy;
     const float uun15 = 1.5f * (uxn * uxn + uyn * uyn);
     const float third = 1.0f / 3.0f;
-    // the node's deviations: its 64-byte row (q = 1..8) and the rest populations
-    float4* row = reinterpret_cast<float4*>(b.dpsi + (size_t)i * 16);
-    const float4 r0 = row[0], r1 = row[1], r2 = row[2], r3 = row[3];
-    float dg[9] = {b.dpsi[dpsi_at(Np, 0, i)], r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-    float dh[9] = {b.dpsi[dpsi_at(Np, 9, i)], r2.x, r2.y, r2.z, r2.w, r3.x, r3.y, r3.z, r3.w};
+    float dev[18];
+    load_all(dev, b.dpsi, Np, i);
 #define FELBM_UPD32_Q(q)                                                                         \
     {                                                                                            \
         const float w = (float)wq(q);                                                            \
         const float Gn = gamma32<q>(uxn, uyn, uun15);                                            \
         const float dG = dgamma32<q>(dux, duy, sux, suy);                                        \
-        dg[q] = om1 * dg[q] + d[q] - (w * dp + third * (drho * (Gn - w) + rho * dG));            \
-        dh[q] = om1 * dh[q] + d[9 + q] - (Gn * dC + C * dG);                                     \
+        dev[q] = om1 * dev[q] + d[q] - (w * dp + third * (drho * (Gn - w) + rho * dG));            \
+        dev[9 + q] = om1 * dev[9 + q] + d[9 + q] - (Gn * dC + C * dG);                                     \
     }
     FELBM_UPD32_Q(0) FELBM_UPD32_Q(1) FELBM_UPD32_Q(2) FELBM_UPD32_Q(3) FELBM_UPD32_Q(4)
     FELBM_UPD32_Q(5) FELBM_UPD32_Q(6) FELBM_UPD32_Q(7) FELBM_UPD32_Q(8)
 #undef FELBM_UPD32_Q
-    b.dpsi[dpsi_at(Np, 0, i)] = dg[0];
-    b.dpsi[dpsi_at(Np, 9, i)] = dh[0];
-    row[0] = make_float4(dg[1], dg[2], dg[3], dg[4]);
-    row[1] = make_float4(dg[5], dg[6], dg[7], dg[8]);
-    row[2] = make_float4(dh[1], dh[2], dh[3], dh[4]);
-    row[3] = make_float4(dh[5], dh[6], dh[7], dh[8]);
+    store_all(b.dpsi, Np, i, dev);
     b.C[i] = Cnd;
     b.p32[i] = p + dp;
     b.ux32[i] = uxn;
@@ -429,12 +572,14 @@ __global__ void k_dev32_to_full(DevMesh m, Phys c, Bufs b, double* stage) {
     double C = b.C[i], p = b.p32[i], ux = b.ux32[i], uy = b.uy32[i];
     double rho = c.rho_v + C * (c.rho_l - c.rho_v);
     double uu15 = 1.5 * (ux * ux + uy * uy);
+    float dev[18];
+    load_all(dev, b.dpsi, Np, i);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         double eu = ex(q) * ux + ey(q) * uy;
         double G = wq(q) * (1.0 + 3.0 * eu + 4.5 * eu * eu - uu15);
-        stage[(size_t)q * N + o] = wq(q) * p + rho * (1.0 / 3.0) * (G - wq(q)) + (double)b.dpsi[dpsi_at(Np, q, i)];
-        stage[(size_t)(9 + q) * N + o] = G * C + (double)b.dpsi[dpsi_at(Np, (9 + q), i)];
+        stage[(size_t)q * N + o] = wq(q) * p + rho * (1.0 / 3.0) * (G - wq(q)) + (double)dev[q];
+        stage[(size_t)(9 + q) * N + o] = G * C + (double)dev[9 + q];
     }
 }
 
@@ -466,15 +611,17 @@ __global__ void k_full_to_dev32(DevMesh m, Phys c, Bufs b, const double* __restr
     // g_q - g_q^eq = (g_q - w p) - (rho/3) w T_q and h_q - h_q^eq = (h_q - w C) - w T_q C,
     // T_q = Gamma_q / w_q - 1 = 3 e.u + 4.5 (e.u)^2 - 1.5 u.u: the large differences in
     // FP64, rounded once to FP32; the velocity terms (O(|u|) of the state) in FP32
+    float dev[18];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const float wf = (float)wq(q);
         const float eu = (float)ex(q) * uxf + (float)ey(q) * uyf;
         const float T = 3.0f * eu + 4.5f * eu * eu - uu15;
         const float dg0 = (float)(g[q] - wq(q) * ps), dh0 = (float)(h[q] - wq(q) * C);
-        b.dpsi[dpsi_at(Np, q, i)] = dg0 - r3 * (wf * T);
-        b.dpsi[dpsi_at(Np, (9 + q), i)] = dh0 - (wf * T) * Cf;
+        dev[q] = dg0 - r3 * (wf * T);
+        dev[9 + q] = dh0 - (wf * T) * Cf;
     }
+    store_all(b.dpsi, Np, i, dev);
     b.C[i] = C;
     b.p32[i] = pf;
     b.ux32[i] = uxf;
@@ -493,7 +640,7 @@ __global__ void k_init_dev32(DevMesh m, Bufs b, const double* __restrict__ stage
     b.ux32[i] = has_u ? (float)u[o] : 0.0f;
     b.uy32[i] = has_u ? (float)u[N + o] : 0.0f;
 #pragma unroll
-    for (int q = 0; q < 18; ++q) b.dpsi[dpsi_at(m.Np, q, i)] = 0.0f;
+    for (int q = 0; q < 18; ++q) b.dpsi[vec_at(m.Np, q, i)] = 0.0f;
 }
 
 __global__ void k_gather_out_f(DevMesh m, const float* __restrict__ src, double* stage) {

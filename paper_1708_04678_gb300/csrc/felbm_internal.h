@@ -102,6 +102,9 @@ struct HostMesh {
     std::vector<int32_t> halo_ptr, halo;
     std::vector<int32_t> layer_cnt;           // [blocks][kBlockSteps + 1]
     int32_t n_layers = 0;
+    // triangles at the nodes of block k: blk_tri[blk_tri_ptr[k] ...], sorted
+    std::vector<int32_t> blk_tri_ptr, blk_tri;
+    int32_t max_blk_tri = 0;
     // connected components ("groups"), numbered by their lowest caller node
     // id; each occupies a contiguous range of internal nodes and triangles
     int32_t G = 0;

@@ -519,6 +519,26 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
                       m.halo.begin() + m.halo_ptr[k]);
     }
 
+    // ---- triangles of every block ---------------------------------------------
+    {
+        const int32_t nblk = (int32_t)m.blk_ptr.size() - 1;
+        std::vector<std::vector<int32_t>> list(nblk);
+        parallel_for(nblk, 32, []() { return 0; }, [&](int32_t k, int&) {
+            std::vector<int32_t>& l = list[k];
+            l.assign(m.inc_tri.begin() + m.inc_ptr[m.blk_ptr[k]], m.inc_tri.begin() + m.inc_ptr[m.blk_ptr[k + 1]]);
+            std::sort(l.begin(), l.end());
+            l.erase(std::unique(l.begin(), l.end()), l.end());
+        });
+        m.blk_tri_ptr.assign(nblk + 1, 0);
+        m.max_blk_tri = 0;
+        for (int32_t k = 0; k < nblk; ++k) {
+            m.blk_tri_ptr[k + 1] = m.blk_tri_ptr[k] + (int32_t)list[k].size();
+            m.max_blk_tri = std::max(m.max_blk_tri, (int32_t)list[k].size());
+        }
+        m.blk_tri.resize(m.blk_tri_ptr[nblk]);
+        for (int32_t k = 0; k < nblk; ++k) std::copy(list[k].begin(), list[k].end(), m.blk_tri.begin() + m.blk_tri_ptr[k]);
+    }
+
     // ---- wall edges: new ids, length and unit normal out of the fluid ----
     m.wall_a.assign(E, 0);
     m.wall_b.assign(E, 0);

@@ -78,3 +78,23 @@ def test_blocked_solve_gives_the_gathered_bits(case, precision, iters):
     for x, y in zip(a.get_state(), b.get_state()):
         np.testing.assert_array_equal(x, y)
     assert np.isfinite(x).all() and np.abs(x).max() > 0
+
+
+@pytest.mark.parametrize("case", ["all planes per block", "free 208", "rows of 13, large"])
+def test_fused_forces_match_the_fp64_step(case):
+    """Large FP32 states form the residuals and gather them in one kernel (rows of
+    7, 9 and 13 entries): the step agrees with the FP64 state's to the FP32 level
+    that the separate kernels are held to."""
+    w = {"all planes per block": CASES["all planes per block"],
+         "free 208": lambda: I.small_free_droplet(n=208, R=50.0),
+         "rows of 13, large": lambda: _refined(220, 180, True)}[case]()
+    mesh = F.Mesh.from_dict(w["mesh"])
+    st = F.State(mesh, F.params_derive(w["phys"], precision=F.FP32_DEV), w["C0"])
+    st.timing_enable(True)
+    st.step(3)
+    assert st.timing_get()["rhs_ms"] < 0.3 * st.timing_get()["element_ms"]     # the gather ran in the element kernel
+    ref = F.State(mesh, F.params_derive(w["phys"]), w["C0"])
+    ref.step(3)
+    (g, h), (gr, hr) = st.get_state(), ref.get_state()
+    assert np.abs(h - hr).max() < 1e-6 * np.abs(hr).max()
+    assert np.abs(g - gr).max() < 1e-4 * np.abs(gr).max()
