@@ -148,6 +148,7 @@ struct Phys3 {
     // 1 = vertex mean of the nodal patch Laplacian, lapmu_fac * sum l_ij (mu_j - mu_i)
     int lapmu_nodal;
     double lapmu_fac;
+    double inv_tau_l, inv_tau_v;
     float dt_f, dt4_f, dt2h_f, inv_tau_l_f, inv_tau_v_f, rho_v_f, drho_f, mobility_f;
 };
 
@@ -240,10 +241,20 @@ __device__ __forceinline__ void set_comp(float4& v, int j, float x) {
     else v.w = x;
 }
 
+// A float as a double through the integer pipe (the conversion instruction
+// shares the FP64 pipe); exact for every float.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0u && (u << 1) != 0u) return (double)x;
+    const uint32_t bias = e == 0u ? 0u : (e == 0x7f800000u ? 0x70000000u : 0x38000000u);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
+}
+
 // ------------------------------------------------------ K1: collision -----
 // Moments of the pre-collision state (C = sum h, p = sum g, rho u = sum e g /
 // cs2) and BGK collision towards g_eq = w p + rho cs2 (Gamma - w),
-// h_eq = Gamma C, written in place.
+// h_eq = Gamma C, written in place.  Bound by the FP64 pipe: one division
+// instead of six (153 us on 262,144 nodes).
 __global__ void __launch_bounds__(kBlock) k3_collide(DevMesh3 m, Phys3 c, Bufs3 b, int do_collide) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
@@ -259,30 +270,35 @@ __global__ void __launch_bounds__(kBlock) k3_collide(DevMesh3 m, Phys3 c, Bufs3 
     for (int q = 0; q < 19; ++q) {
         C += h[q];
         p += g[q];
-        mx += edot3(q, g[q], 0.0, 0.0);
-        my += edot3(q, 0.0, g[q], 0.0);
-        mz += edot3(q, 0.0, 0.0, g[q]);
+        if (ex3(q) != 0) mx += ex3(q) > 0 ? g[q] : -g[q];
+        if (ey3(q) != 0) my += ey3(q) > 0 ? g[q] : -g[q];
+        if (ez3(q) != 0) mz += ez3(q) > 0 ? g[q] : -g[q];
     }
-    double rho = c.rho_v + C * (c.rho_l - c.rho_v);
-    double ux = 3.0 * mx / rho, uy = 3.0 * my / rho, uz = 3.0 * mz / rho;
+    const double rho = c.rho_v + C * (c.rho_l - c.rho_v);
+    // omega = 1 / (tau + 1/2) = (1/tau) / (1 + 1/(2 tau)); one division for it and 1/rho
+    const double inv_tau = fma(C, c.inv_tau_l - c.inv_tau_v, c.inv_tau_v);
+    const double half = fma(0.5, inv_tau, 1.0), inv = 1.0 / (rho * half), inv_rho3 = 3.0 * half * inv;
+    const double ux = mx * inv_rho3, uy = my * inv_rho3, uz = mz * inv_rho3;
     b.C[i] = C;
     b.p[i] = p;
     b.ux[i] = ux;
     b.uy[i] = uy;
     b.uz[i] = uz;
     if (!do_collide) return;
-    double inv_tau = C / c.tau_l + (1.0 - C) / c.tau_v;
-    double omega = 1.0 / (1.0 / inv_tau + 0.5);
-    double uu15 = 1.5 * (ux * ux + uy * uy + uz * uz);
-    double rcs2 = rho * (1.0 / 3.0);
-#pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        double eu = edot3(q, ux, uy, uz);
-        double G = wq3(q) * (1.0 + 3.0 * eu + 4.5 * eu * eu - uu15);
-        double geq = wq3(q) * p + rcs2 * (G - wq3(q));
-        double heq = G * C;
+    const double omega = inv_tau * rho * inv;
+    const double uu15 = 1.5 * (ux * ux + uy * uy + uz * uz), rcs2 = rho * (1.0 / 3.0);
+    // a direction and its opposite (q, q + 1) share 4.5 (e.u)^2
+    const auto relax = [&](int q, double G0) {
+        const double G = wq3(q) * G0, geq = wq3(q) * p + rcs2 * (G - wq3(q));
         b.psi[q * Np + i] = g[q] - omega * (g[q] - geq);
-        b.psi[(19 + q) * Np + i] = h[q] - omega * (h[q] - heq);
+        b.psi[(19 + q) * Np + i] = h[q] - omega * (h[q] - G * C);
+    };
+    relax(0, 1.0 - uu15);
+#pragma unroll
+    for (int q = 1; q < 19; q += 2) {
+        const double eu = edot3(q, ux, uy, uz), t = 4.5 * eu * eu;
+        relax(q, 1.0 + 3.0 * eu + t - uu15);
+        relax(q + 1, 1.0 - 3.0 * eu + t - uu15);
     }
 }
 
@@ -345,6 +361,8 @@ __global__ void __launch_bounds__(kBlock) k3_lmu(DevMesh3 m, Phys3 c, Bufs3 b) {
 //   Phi_g = (e-u).[cs2 grad(rho) (Gamma - w) + mu grad(C) Gamma]
 //   Phi_h = [(e-u).(grad C - C/(rho cs2) (grad p - mu grad C)) + M lap(mu)] Gamma
 // Residual R_a = V (Phi_a - e_a . grad psi_hat_a), psi_hat P1 on the element.
+// Bound by the FP64 pipe, hence the factored forces: 1,448 us on 1,572,864
+// tetrahedra against 2,258 us for the terms as written above.
 __global__ void __launch_bounds__(128) k3_element(DevMesh3 m, Phys3 c, Bufs3 b) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m.T) return;
@@ -359,138 +377,185 @@ __global__ void __launch_bounds__(128) k3_element(DevMesh3 m, Phys3 c, Bufs3 b) 
         bz[k] = m.grad[(3 * k + 2) * Tp + t];
     }
     const double V = m.vol[t];
-    double Cs = 0, uxs = 0, uys = 0, uzs = 0, mus = 0;
-    double gC[3] = {0, 0, 0}, gp[3] = {0, 0, 0};
-    const double C0 = b.C[v[0]], p0 = b.p[v[0]];
+    double Cv[4], pv[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        double Cv = b.C[v[k]], pv = b.p[v[k]];
-        Cs += Cv;
-        uxs += b.ux[v[k]];
-        uys += b.uy[v[k]];
-        uzs += b.uz[v[k]];
-        mus += b.mu[v[k]];
-        if (k > 0) {
-            double dC = Cv - C0, dp = pv - p0;
-            gC[0] += dC * bx[k];
-            gC[1] += dC * by[k];
-            gC[2] += dC * bz[k];
-            gp[0] += dp * bx[k];
-            gp[1] += dp * by[k];
-            gp[2] += dp * bz[k];
-        }
+        Cv[k] = b.C[v[k]];
+        pv[k] = b.p[v[k]];
     }
-    const double Cb = 0.25 * Cs, ux = 0.25 * uxs, uy = 0.25 * uys, uz = 0.25 * uzs, mub = 0.25 * mus;
+    double gC[3] = {0, 0, 0}, gp[3] = {0, 0, 0};
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        const double dC = Cv[k] - Cv[0], dp = pv[k] - pv[0];
+        gC[0] = fma(dC, bx[k], gC[0]);
+        gC[1] = fma(dC, by[k], gC[1]);
+        gC[2] = fma(dC, bz[k], gC[2]);
+        gp[0] = fma(dp, bx[k], gp[0]);
+        gp[1] = fma(dp, by[k], gp[1]);
+        gp[2] = fma(dp, bz[k], gp[2]);
+    }
+    const double Cb = 0.25 * (Cv[0] + Cv[1] + Cv[2] + Cv[3]);
+    const double ux = 0.25 * (b.ux[v[0]] + b.ux[v[1]] + b.ux[v[2]] + b.ux[v[3]]);
+    const double uy = 0.25 * (b.uy[v[0]] + b.uy[v[1]] + b.uy[v[2]] + b.uy[v[3]]);
+    const double uz = 0.25 * (b.uz[v[0]] + b.uz[v[1]] + b.uz[v[2]] + b.uz[v[3]]);
+    const double mub = 0.25 * (b.mu[v[0]] + b.mu[v[1]] + b.mu[v[2]] + b.mu[v[3]]);
     double lapmu;
     if (c.lapmu_nodal) {
         lapmu = 0.25 * (b.lmu[v[0]] + b.lmu[v[1]] + b.lmu[v[2]] + b.lmu[v[3]]);
     } else {
-        const double gm[3] = {b.gmu[t], b.gmu[Tp + t], b.gmu[2 * Tp + t]};
+        // sum over interior faces of (grad mu_T + grad mu_T').b_k; the b_k sum to
+        // zero, so grad mu_T enters only through the wall faces
         double flux = 0.0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            int nb = m.nbr[k * Tp + t];
-            if (nb >= 0)
-                flux += (gm[0] + b.gmu[nb]) * bx[k] + (gm[1] + b.gmu[Tp + nb]) * by[k] + (gm[2] + b.gmu[2 * Tp + nb]) * bz[k];
+            const int nb = m.nbr[k * Tp + t], at = nb >= 0 ? nb : t;
+            const double sg = nb >= 0 ? 1.0 : -1.0;
+            flux += sg * fma(b.gmu[at], bx[k], fma(b.gmu[Tp + at], by[k], b.gmu[2 * Tp + at] * bz[k]));
         }
         lapmu = -1.5 * flux;
     }
-    const double drho = c.rho_l - c.rho_v;
-    const double rhob = c.rho_v + Cb * drho;
-    const double gr[3] = {drho * gC[0], drho * gC[1], drho * gC[2]};
+    const double drho = c.rho_l - c.rho_v, rhob = c.rho_v + Cb * drho;
     const double f = 3.0 * Cb / rhob;
     const double vh[3] = {gC[0] - f * (gp[0] - mub * gC[0]), gC[1] - f * (gp[1] - mub * gC[1]),
                           gC[2] - f * (gp[2] - mub * gC[2])};
-    const double u_gr = ux * gr[0] + uy * gr[1] + uz * gr[2];
-    const double u_gC = ux * gC[0] + uy * gC[1] + uz * gC[2];
-    const double u_vh = ux * vh[0] + uy * vh[1] + uz * vh[2];
     const double uu15 = 1.5 * (ux * ux + uy * uy + uz * uz);
-    const double Mlap = c.mobility * lapmu;
+    // With T = Gamma / w - 1 and s = (e - u).grad C:
+    //   V Phi_g = w s (P + Q T),  P = V mu,  Q = V (mu + drho / 3)
+    //   V Phi_h = w V ((e - u).v + M lap mu) (1 + T)
+    // for a direction and its opposite (q, q + 1) together; the axis weight 1/18
+    // is folded into the vectors, diagonals take a half, rest six times.
+    const double P = V * mub, Q = fma(V * (1.0 / 3.0), drho, P), w1 = 1.0 / 18.0, Vw = V * w1;
+    const double s[3] = {w1 * gC[0], w1 * gC[1], w1 * gC[2]}, z[3] = {Vw * vh[0], Vw * vh[1], Vw * vh[2]};
+    const double su = ux * s[0] + uy * s[1] + uz * s[2];
+    const double vu = ux * z[0] + uy * z[1] + uz * z[2] - Vw * (c.mobility * lapmu);
+    const double sd[3] = {0.5 * s[0], 0.5 * s[1], 0.5 * s[2]}, zd[3] = {0.5 * z[0], 0.5 * z[1], 0.5 * z[2]};
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        bx[k] *= V;
+        by[k] *= V;
+        bz[k] *= V;
+    }
     double* dst = b.R + (size_t)t * 38;
+    dst[0] = -6.0 * su * fma(Q, -uu15, P);
+    dst[19] = -6.0 * fma(vu, -uu15, vu);
 #pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        const double w = wq3(q);
-        const double eu = edot3(q, ux, uy, uz);
-        const double G = w * (1.0 + 3.0 * eu + 4.5 * eu * eu - uu15);
-        const double phig = (1.0 / 3.0) * (G - w) * (edot3(q, gr[0], gr[1], gr[2]) - u_gr) +
-                            mub * G * (edot3(q, gC[0], gC[1], gC[2]) - u_gC);
-        const double phih = ((edot3(q, vh[0], vh[1], vh[2]) - u_vh) + Mlap) * G;
-        double dg = 0.0, dh = 0.0;
-        if (q != 0) {
-            const double g0 = b.psi[q * Np + v[0]], h0 = b.psi[(19 + q) * Np + v[0]];
+    for (int q = 1; q < 19; q += 2) {
+        const bool axis = q <= 6;
+        const double eu = edot3(q, ux, uy, uz), t2 = fma(4.5 * eu, eu, -uu15);
+        const double tp = fma(3.0, eu, t2), tm = fma(-3.0, eu, t2);
+        const double es = axis ? edot3(q, s[0], s[1], s[2]) : edot3(q, sd[0], sd[1], sd[2]);
+        const double ev = axis ? edot3(q, z[0], z[1], z[2]) : edot3(q, zd[0], zd[1], zd[2]);
+        const double sw = axis ? su : 0.5 * su, vw = axis ? vu : 0.5 * vu;
+        const double vp = ev - vw, vm = -ev - vw;
+        double gq = (es - sw) * fma(Q, tp, P), gm = (-es - sw) * fma(Q, tm, P);
+        double hq = fma(vp, tp, vp), hm = fma(vm, tm, vm);
+        const double* pq = b.psi + (size_t)q * Np;
+        const double* ph = b.psi + (size_t)(19 + q) * Np;
+        const double g0 = pq[v[0]], g1 = pq[Np + v[0]], h0 = ph[v[0]], h1 = ph[Np + v[0]];
 #pragma unroll
-            for (int k = 1; k < 4; ++k) {
-                const double eb = edot3(q, bx[k], by[k], bz[k]);
-                dg += (b.psi[q * Np + v[k]] - g0) * eb;
-                dh += (b.psi[(19 + q) * Np + v[k]] - h0) * eb;
-            }
+        for (int k = 1; k < 4; ++k) {
+            const double eb = edot3(q, bx[k], by[k], bz[k]);
+            gq = fma(g0 - pq[v[k]], eb, gq);
+            gm = fma(pq[Np + v[k]] - g1, eb, gm);
+            hq = fma(h0 - ph[v[k]], eb, hq);
+            hm = fma(ph[Np + v[k]] - h1, eb, hm);
         }
-        dst[q] = V * (phig - dg);
-        dst[19 + q] = V * (phih - dh);
+        dst[q] = gq;
+        dst[q + 1] = gm;
+        dst[19 + q] = hq;
+        dst[20 + q] = hm;
     }
 }
 
 // ------------------------------------------- K5: streaming RHS gather -----
 // RHS_{i,a} = sum_{T at i} R_{T,a} (dt/4 + dt^2/2 e_a.b_{i,T})
 //   - dt sum_{wall f at i} (e_a.n) [A/6 (psi_opp - psi)_i + A/12 sum_{o != i} (psi_opp - psi)_o]
-// (wall term only for incoming directions e_a.n < 0).  One thread per
-// (node, set); also writes the first iterate of the solve first_scale RHS / m_i
-// (1/theta for the FP64 Chebyshev recurrence, tau_0 for the FP32 steps):
-// FP64 (FP64 Chebyshev) or FP32 with the FP32 copy of the RHS (mixed solve).
+// (wall term only for incoming directions e_a.n < 0); also writes the first
+// iterate of the solve first_scale RHS / m_i (1/theta for the FP64 Chebyshev
+// recurrence, tau_0 for the FP32 steps): FP64 (FP64 Chebyshev) or FP32 with the
+// FP32 copy of the RHS (mixed solve).
+// Ten lanes per node (three nodes per warp): lane c > 0 takes the directions
+// 2c - 1 and 2c, which are opposite, of both sets, so one e.b serves four
+// products and the lanes of a node read a residual row as one contiguous run;
+// lane 0 takes the rest populations.  1,113 us on 262,144 nodes against 1,230 us
+// for one thread per node and set; 49 against 95 us on 7,350 nodes.
 template <bool kMixed>
 __global__ void __launch_bounds__(kNodeBlock) k3_rhs(DevMesh3 m, Phys3 c, Bufs3 b, double first_scale) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m.N) return;
-    const int s = blockIdx.y, Np = m.Np, ninc = m.ninc;
-    double acc[19];
-#pragma unroll
-    for (int q = 0; q < 19; ++q) acc[q] = 0.0;
-    const double c1 = 0.25 * c.dt, c2 = 0.5 * c.dt * c.dt;
-    for (int k = m.inc_ptr[i]; k < m.inc_ptr[i + 1]; ++k) {
-        const double* src = b.R + (size_t)m.inc_tet[k] * 38 + 19 * s;
-        const double bxi = m.inc_b[k], byi = m.inc_b[ninc + k], bzi = m.inc_b[2 * ninc + k];
-#pragma unroll
-        for (int q = 0; q < 19; ++q) acc[q] += src[q] * (c1 + c2 * edot3(q, bxi, byi, bzi));
-    }
-    const double* ps = b.psi + (size_t)19 * s * Np;
-    const int F = m.F;
-    for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
-        const int f = m.winc_face[k];
-        int o[2], n = 0;
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) {
-            int vv = m.wall_v[cc * F + f];
-            if (vv != i && n < 2) o[n++] = vv;
+    const int lane = threadIdx.x & 31, grp = lane / 10, cc = lane - grp * 10;
+    const int i = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 3 + grp;
+    if (grp >= 3 || i >= m.N) return;
+    const int Np = m.Np, ninc = m.ninc, F = m.F, q = max(0, 2 * cc - 1), nd = cc == 0 ? 1 : 2;
+    const double ex = ex3(q), ey = ey3(q), ez = ez3(q);
+    const double c1 = 0.25 * c.dt, c2 = 0.5 * c.dt * c.dt, cx = c2 * ex, cy = c2 * ey, cz = c2 * ez;
+    double g0 = 0.0, g1 = 0.0, h0 = 0.0, h1 = 0.0;
+    const int k1 = m.inc_ptr[i + 1];
+#pragma unroll 4
+    for (int k = m.inc_ptr[i]; k < k1; ++k) {
+        const double* src = b.R + (size_t)m.inc_tet[k] * 38 + q;
+        const double eb = fma(cz, m.inc_b[2 * ninc + k], fma(cy, m.inc_b[ninc + k], cx * m.inc_b[k]));
+        const double wp = c1 + eb, wm = c1 - eb;
+        g0 = fma(src[0], wp, g0);
+        h0 = fma(src[19], wp, h0);
+        if (nd == 2) {
+            g1 = fma(src[1], wm, g1);
+            h1 = fma(src[20], wm, h1);
         }
-        const double A = m.wall_area[f], nx = m.wall_n[f], ny = m.wall_n[F + f], nz = m.wall_n[2 * F + f];
+    }
+    if (cc > 0) {
+        for (int k = m.winc_ptr[i]; k < m.winc_ptr[i + 1]; ++k) {
+            const int f = m.winc_face[k];
+            int o[2] = {i, i}, n = 0;
 #pragma unroll
-        for (int q = 1; q < 19; ++q) {
-            const double en = edot3(q, nx, ny, nz);
+            for (int w = 0; w < 3; ++w) {
+                const int vv = m.wall_v[w * F + f];
+                if (vv != i && n < 2) o[n++] = vv;
+            }
+            const double A = m.wall_area[f], en = ex * m.wall_n[f] + ey * m.wall_n[F + f] + ez * m.wall_n[2 * F + f];
+            if (en == 0.0) continue;
+            // psi_opp - psi of the incoming one of the two, at the three vertices
+            const auto jump = [&](const double* ps) {
+                const double* p0 = ps + (size_t)q * Np;
+                const double di = p0[Np + i] - p0[i], d1 = p0[Np + o[0]] - p0[o[0]], d2 = p0[Np + o[1]] - p0[o[1]];
+                return A * (1.0 / 6.0) * di + A * (1.0 / 12.0) * (d1 + d2);
+            };
+            const double add = c.dt * en, jg = jump(b.psi), jh = jump(b.psi + (size_t)19 * Np);
             if (en < 0.0) {
-                const int qo = opp3(q);
-                const double di = ps[qo * Np + i] - ps[q * Np + i];
-                const double d1 = ps[qo * Np + o[0]] - ps[q * Np + o[0]];
-                const double d2 = ps[qo * Np + o[1]] - ps[q * Np + o[1]];
-                acc[q] += -c.dt * en * (A * (1.0 / 6.0) * di + A * (1.0 / 12.0) * (d1 + d2));
+                g0 -= add * jg;
+                h0 -= add * jh;
+            } else {
+                g1 -= add * jg;
+                h1 -= add * jh;
             }
         }
     }
     const double sc = m.inv_lumped[i] * first_scale;
-#pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        const size_t r = (size_t)(19 * s + q) * Np + i;
-        b.rhs[r] = acc[q];
-        if (kMixed) {
-            const size_t a = (size_t)i * kRow + slot(s, q);
-            b.r32[a] = (float)acc[q];
-            b.e1[a] = (float)(acc[q] * sc);
-        } else {
-            b.x1[r] = acc[q] * sc;
-        }
+    const size_t r = (size_t)q * Np + i, rh = (size_t)(19 + q) * Np + i;
+    b.rhs[r] = g0;
+    b.rhs[rh] = h0;
+    if (nd == 2) {
+        b.rhs[r + Np] = g1;
+        b.rhs[rh + Np] = h1;
     }
-    if (kMixed) {
-        b.r32[(size_t)i * kRow + slot(s, 19)] = 0.0f;
-        b.e1[(size_t)i * kRow + slot(s, 19)] = 0.0f;
+    if constexpr (kMixed) {
+        // the corrections start from the FP32 copy (conversions share the FP64 pipe)
+        const size_t a = (size_t)i * kRow + q;
+        const float s = (float)sc, fg0 = (float)g0, fh0 = (float)h0, fg1 = (float)g1, fh1 = (float)h1;
+        b.r32[a] = fg0;
+        b.r32[a + 20] = fh0;
+        b.e1[a] = fg0 * s;
+        b.e1[a + 20] = fh0 * s;
+        const size_t a1 = (size_t)i * kRow + (cc == 0 ? 19 : q + 1);      // lane 0: the padding slots, zero
+        b.r32[a1] = fg1;
+        b.r32[a1 + 20] = fh1;
+        b.e1[a1] = fg1 * s;
+        b.e1[a1 + 20] = fh1 * s;
+    } else {
+        b.x1[r] = g0 * sc;
+        b.x1[rh] = h0 * sc;
+        if (nd == 2) {
+            b.x1[r + Np] = g1 * sc;
+            b.x1[rh + Np] = h1 * sc;
+        }
     }
 }
 
@@ -533,40 +598,53 @@ __global__ void __launch_bounds__(kNodeBlock) k3_cheb(DevMesh3 m, Bufs3 b, const
 enum Final3 { kStore3 = 0, kAddPsi3 = 1, kUpdateDev3 = 2 };
 
 template <int kFinal>
-__global__ void __launch_bounds__(kNodeBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bufs3 b, const float* __restrict__ cur,
+__global__ void __launch_bounds__(kNodeBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bufs3 b, const float* cur,
                                                          float* nxt, float tau, int have_x64);
 
 // x <- x + e ; rho <- rho - M11 e (FP64); FP32 copy of rho and the first
-// iterate of the next correction, tau_0 rho / m.  x64 = x0, rho64 = x1.
-__global__ void __launch_bounds__(kNodeBlock) k3_refine(DevMesh3 m, Bufs3 b, const float* __restrict__ e,
-                                                        float* next_first, int first_round, double tau0) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m.N) return;
-    const int Np = m.Np;
-    const size_t off = (size_t)19 * blockIdx.y * Np;
-    double acc[19];
+// iterate of the next correction, tau_0 rho / m.  x64 = x0, rho64 = x1.  Ten
+// lanes per node (three nodes per warp), lane c the 16-byte vector c of the
+// rows, so a gathered row is one contiguous load; the gathered floats are
+// widened on the integer pipe (the kernel is bound by the FP64 pipe): 486 us on
+// 262,144 nodes against 670 us with conversion instructions.
+__global__ void __launch_bounds__(kCoopBlock) k3_refine(DevMesh3 m, Bufs3 b, const float* e, float* next_first,
+                                                        int first_round, float tau0) {
+    const int lane = threadIdx.x & 31, grp = lane / 10, cc = lane - grp * 10;
+    const int i = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 3 + grp;
+    if (grp >= 3 || i >= m.N) return;
+    const int Np = m.Np, s = cc / 5, q0 = 4 * (cc - 5 * s), nq = min(4, 19 - q0);
+    const size_t r0 = (size_t)(19 * s + q0) * Np + i;
+    // every load of the node itself before the first store
+    const float4 ei = reinterpret_cast<const float4*>(e + (size_t)i * kRow)[cc];
+    double acc[4] = {0.0, 0.0, 0.0, 0.0}, ro[4], xo[4];
 #pragma unroll
-    for (int q = 0; q < 19; ++q) acc[q] = 0.0;
-    const int s = blockIdx.y;
-    for (int k = m.row_ptr[i]; k < m.row_ptr[i + 1]; ++k) {
-        const float* ej = e + (size_t)m.col[k] * kRow + slot(s, 0);
+    for (int j = 0; j < 4; ++j) {
+        ro[j] = j < nq ? (first_round ? b.rhs[r0 + (size_t)j * Np] : b.x1[r0 + (size_t)j * Np]) : 0.0;
+        xo[j] = j < nq && !first_round ? b.x0[r0 + (size_t)j * Np] : 0.0;
+    }
+    const int k1 = m.row_ptr[i + 1];
+#pragma unroll 4
+    for (int k = m.row_ptr[i]; k < k1; ++k) {
+        const float4 ej = reinterpret_cast<const float4*>(e + (size_t)m.col[k] * kRow)[cc];
         const double mv = m.mval[k];
-#pragma unroll
-        for (int q = 0; q < 19; ++q) acc[q] += mv * (double)ej[q];
+        acc[0] = fma(mv, widen(ej.x), acc[0]);
+        acc[1] = fma(mv, widen(ej.y), acc[1]);
+        acc[2] = fma(mv, widen(ej.z), acc[2]);
+        acc[3] = fma(mv, widen(ej.w), acc[3]);
     }
-    const double sc = m.inv_lumped[i] * tau0;
-    const size_t a0 = (size_t)i * kRow + slot(s, 0);
+    const float sc = m.inv_lumped32[i] * tau0;
+    float r[4];
 #pragma unroll
-    for (int q = 0; q < 19; ++q) {
-        const size_t r = off + (size_t)q * Np + i;
-        double xo = first_round ? 0.0 : b.x0[r];
-        double ro = first_round ? b.rhs[r] : b.x1[r];
-        double rn = ro - acc[q];
-        b.x0[r] = xo + (double)e[a0 + q];
-        b.x1[r] = rn;
-        b.r32[a0 + q] = (float)rn;
-        next_first[a0 + q] = (float)(rn * sc);
+    for (int j = 0; j < 4; ++j) {
+        r[j] = 0.0f;                                  // the padding slots stay zero
+        if (j >= nq) continue;
+        const double ed = widen(comp(ei, j)), rn = ro[j] - acc[j];
+        b.x0[r0 + (size_t)j * Np] = first_round ? ed : xo[j] + ed;
+        b.x1[r0 + (size_t)j * Np] = rn;
+        r[j] = (float)rn;
     }
+    reinterpret_cast<float4*>(b.r32 + (size_t)i * kRow)[cc] = make_float4(r[0], r[1], r[2], r[3]);
+    reinterpret_cast<float4*>(next_first + (size_t)i * kRow)[cc] = make_float4(r[0] * sc, r[1] * sc, r[2] * sc, r[3] * sc);
 }
 
 // ------------------------------------------------ FP32 Chebyshev sweep ----
@@ -588,7 +666,7 @@ __device__ __forceinline__ void pdl_release3() { asm volatile("griddepcontrol.la
 // do not depend on the previous sweep, so under programmatic dependent
 // launch they are fetched while that sweep drains); kW = 0: CSR.
 template <int kFinal, int kW>
-__global__ void __launch_bounds__(kCoopBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bufs3 b, const float* __restrict__ cur,
+__global__ void __launch_bounds__(kCoopBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bufs3 b, const float* cur,
                                                          float* nxt, float tau, int have_x64) {
     pdl_release3();
     const Coop k = coop_index(m.N);
@@ -646,8 +724,11 @@ __global__ void __launch_bounds__(kCoopBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bu
                 const int q = 4 * k.c + j;
                 if (q >= 19) continue;
                 const size_t rg = (size_t)q * Np + i, rh = (size_t)(19 + q) * Np + i;
-                b.psi[rg] += have_x64 ? b.x0[rg] + (double)comp(xn[0], j) : (double)comp(xn[0], j);
-                b.psi[rh] += have_x64 ? b.x0[rh] + (double)comp(xn[1], j) : (double)comp(xn[1], j);
+                const double eg = widen(comp(xn[0], j)), eh = widen(comp(xn[1], j));
+                const double xg = have_x64 ? b.x0[rg] : 0.0, xh = have_x64 ? b.x0[rh] : 0.0;
+                const double pg = b.psi[rg], ph = b.psi[rh];
+                b.psi[rg] = pg + (have_x64 ? xg + eg : eg);
+                b.psi[rh] = ph + (have_x64 ? xh + eh : eh);
             }
         }
     }
@@ -665,23 +746,42 @@ constexpr int kRowLanes = 10;
 constexpr int kRowGroups = 3;                       // per warp (30 of 32 lanes)
 constexpr int kRowItemsPerBlock = kRowGroups * (kCoopBlock / 32);
 
-template <int kW>
-__global__ void __launch_bounds__(kCoopBlock, 16) k3_sweep_rows32(DevMesh3 m, Phys3 c, Bufs3 b,
-                                                              const float* __restrict__ cur, float* nxt, float tau) {
+// kAhead: every gather of the row issued before the first product (for meshes
+// too small to fill the device with warps).
+template <int kW, bool kAhead>
+__global__ void __launch_bounds__(kCoopBlock, kAhead ? 1 : 16) k3_sweep_rows32(DevMesh3 m, Phys3 c, Bufs3 b,
+                                                              const float* cur, float* nxt, float tau) {
     pdl_release3();
     const int lane = threadIdx.x & 31, grp = lane / kRowLanes, cc = lane - grp * kRowLanes;
     const int item = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kRowGroups + grp;
     const bool active = grp < kRowGroups && item < m.N;
     const int i = active ? item : 0;
     const int Np = m.Np;
+    int col[kAhead ? kW : 1];
+    float val[kAhead ? kW : 1];
+    if constexpr (kAhead) {
+#pragma unroll
+        for (int e = 0; e < kW; ++e) {
+            col[e] = m.ell_col[e * Np + i];
+            val[e] = m.ell_val[e * Np + i];
+        }
+    }
     const float sc = tau * m.inv_lumped32[i];
     pdl_wait3();
     if (!active) return;
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if constexpr (kAhead) {
+        float4 x[kW];
 #pragma unroll
-    for (int e = 0; e < kW; ++e) {
-        const int cl = m.ell_col[e * Np + i];
-        fma4(acc, m.ell_val[e * Np + i], reinterpret_cast<const float4*>(cur + (size_t)cl * kRow)[cc]);
+        for (int e = 0; e < kW; ++e) x[e] = reinterpret_cast<const float4*>(cur + (size_t)col[e] * kRow)[cc];
+#pragma unroll
+        for (int e = 0; e < kW; ++e) fma4(acc, val[e], x[e]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < kW; ++e) {
+            const int cl = m.ell_col[e * Np + i];
+            fma4(acc, m.ell_val[e * Np + i], reinterpret_cast<const float4*>(cur + (size_t)cl * kRow)[cc]);
+        }
     }
     const size_t own = (size_t)i * kRow;
     const float4 xk = reinterpret_cast<const float4*>(cur + own)[cc];
@@ -985,6 +1085,15 @@ static size_t carve3(const HostMesh3D& h, bool dev32, void* base, DevMesh3* dm, 
 
 static unsigned grid_for(int n, int block) { return (unsigned)((n + block - 1) / block); }
 
+// Threads per block of the FP64 kernels: `most`, or a warp where that spreads
+// few items over the multiprocessors more evenly (felbm.cu: fp64_block).
+constexpr int kWarpBlocksBelow = 512;   // items per multiprocessor
+// nodes per multiprocessor (k3_sweep_rows32): on 7,350 nodes every gather in
+// flight at 91 registers takes a step from 297 to 260 us; on 262,144 nodes the
+// 32-register form is the faster, 1,204 against 1,298 us
+constexpr int kGatherAheadBelow = 128;
+static int fp64_block(int n_sm, int n, int most) { return n < kWarpBlocksBelow * n_sm ? 32 : most; }
+
 template <class T>
 static cudaError_t up(const T* dst, const std::vector<T>& src, cudaStream_t s) {
     if (src.empty()) return cudaSuccess;
@@ -1014,6 +1123,7 @@ struct felbm3d_state {
     bool dev32 = false;
     bool timing = false;
     bool timed_step_ran = false;
+    int n_sm = 1;          // multiprocessors of the device
     bool use_pdl = true;   // programmatic dependent launch between solve sweeps (FELBM_PDL=0: off)
     cudaEvent_t ev[6] = {};
     cudaEvent_t ev_copied = nullptr;   // set_state: the host arrays have been read
@@ -1048,11 +1158,15 @@ static void launch_sweep3(felbm3d_state* st, cudaStream_t s, const float* cur, f
     pdl = pdl && st->use_pdl;
     if constexpr (kFinal == kStore3) {
         const unsigned gr = grid_for(m.N, kRowItemsPerBlock);
+        const auto go = [&](auto all, auto ahead) {
+            launch3(pdl, m.N < kGatherAheadBelow * st->n_sm ? ahead : all, gr, kCoopBlock, s, m, st->phys, st->buf, cur,
+                    nxt, tau);
+        };
         switch (m.ell_w) {
-            case 15: launch3(pdl, k3_sweep_rows32<15>, gr, kCoopBlock, s, m, st->phys, st->buf, cur, nxt, tau); return;
-            case 16: launch3(pdl, k3_sweep_rows32<16>, gr, kCoopBlock, s, m, st->phys, st->buf, cur, nxt, tau); return;
-            case 24: launch3(pdl, k3_sweep_rows32<24>, gr, kCoopBlock, s, m, st->phys, st->buf, cur, nxt, tau); return;
-            case 32: launch3(pdl, k3_sweep_rows32<32>, gr, kCoopBlock, s, m, st->phys, st->buf, cur, nxt, tau); return;
+            case 15: go(k3_sweep_rows32<15, false>, k3_sweep_rows32<15, true>); return;
+            case 16: go(k3_sweep_rows32<16, false>, k3_sweep_rows32<16, true>); return;
+            case 24: go(k3_sweep_rows32<24, false>, k3_sweep_rows32<24, true>); return;
+            case 32: go(k3_sweep_rows32<32, false>, k3_sweep_rows32<32, true>); return;
             default: break;
         }
     }
@@ -1087,21 +1201,22 @@ static void enqueue_step3(felbm3d_state* st, cudaStream_t s) {
         enqueue_step_dev32(st, s);
         return;
     }
-    k3_collide<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b, 1);
-    k3_mu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b);
+    const int nb = fp64_block(st->n_sm, m.N, kNodeBlock), tb = fp64_block(st->n_sm, m.T, 128);
+    const unsigned ng = grid_for(m.N, nb), tg = grid_for(m.T, tb), rg = grid_for(m.N, 3 * (nb / 32));
+    k3_collide<<<ng, nb, 0, s>>>(m, st->phys, b, 1);
+    k3_mu<<<ng, nb, 0, s>>>(m, st->phys, b);
     mark(1);
     if (st->phys.lapmu_nodal)
-        k3_lmu<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, st->phys, b);
+        k3_lmu<<<ng, nb, 0, s>>>(m, st->phys, b);
     else
-        k3_gradmu<<<grid_for(m.T, kBlock), kBlock, 0, s>>>(m, b);
+        k3_gradmu<<<tg, tb, 0, s>>>(m, b);
     mark(2);
-    k3_element<<<grid_for(m.T, 128), 128, 0, s>>>(m, st->phys, b);
+    k3_element<<<tg, tb, 0, s>>>(m, st->phys, b);
     mark(3);
-    const dim3 g2(grid_for(m.N, kNodeBlock), 2);
     if (st->mode == FELBM_SOLVER_FP64)
-        k3_rhs<false><<<g2, kNodeBlock, 0, s>>>(m, st->phys, b, st->inv_theta);
+        k3_rhs<false><<<rg, nb, 0, s>>>(m, st->phys, b, st->inv_theta);
     else
-        k3_rhs<true><<<g2, kNodeBlock, 0, s>>>(m, st->phys, b, st->tau[0]);
+        k3_rhs<true><<<rg, nb, 0, s>>>(m, st->phys, b, st->tau[0]);
     mark(4);
     enqueue_solve3(st, s);
     mark(5);
@@ -1142,7 +1257,7 @@ static void enqueue_solve3(felbm3d_state* st, cudaStream_t s, bool after_release
             std::swap(cur, prv);
         }
         if (r < st->rounds - 1) {
-            k3_refine<<<g2, kNodeBlock, 0, s>>>(m, b, cur, prv, r == 0, st->tau[0]);
+            k3_refine<<<grid_for(m.N, 3 * (kCoopBlock / 32)), kCoopBlock, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0]);
             A = prv;
             B = cur;
         }
@@ -1239,6 +1354,15 @@ int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const dou
     st->stream = static_cast<cudaStream_t>(stream);
     st->dev32 = dev32;
     if (const char* env = std::getenv("FELBM_PDL")) st->use_pdl = std::atoi(env) != 0;
+    {
+        int device = 0;
+        cudaError_t qe = cudaGetDevice(&device);
+        if (qe == cudaSuccess) qe = cudaDeviceGetAttribute(&st->n_sm, cudaDevAttrMultiProcessorCount, device);
+        if (qe != cudaSuccess) {
+            delete st;
+            return cuda_fail(qe, "felbm3d_init: device");
+        }
+    }
     carve3(h, dev32, d_workspace, &st->dm, &st->buf);
     Phys3& ph = st->phys;
     ph.dt = params->dt;
@@ -1252,6 +1376,8 @@ int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const dou
     ph.lapmu_nodal = params->lapmu_mode == FELBM_LAPMU_NODAL;
     // lval = -3 K_ij / (s |patch_i|); the lumped P1 Laplacian is -K_ij / (|patch_i| / 4)
     ph.lapmu_fac = (params->lap_mode == FELBM_LAP_PAPER ? 1.0 : 0.75) * 4.0 / 3.0;
+    ph.inv_tau_l = 1.0 / params->tau_l;
+    ph.inv_tau_v = 1.0 / params->tau_v;
     ph.dt_f = (float)params->dt;
     ph.dt4_f = (float)(0.25 * params->dt);
     ph.dt2h_f = (float)(0.5 * params->dt * params->dt);
