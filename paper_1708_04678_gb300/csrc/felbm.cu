@@ -267,6 +267,16 @@ __device__ __forceinline__ void store_all(float* x, int Np, int i, const float (
     store_vec(x, Np, 4, i, v);
 }
 
+// A float as a double through the integer pipe: the conversion instruction
+// shares the FP64 pipe, whose rate is 1/64 of it.  Exact for every float
+// (the rare denormals take the instruction).
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0u && (u << 1) != 0u) return (double)x;
+    const uint32_t bias = e == 0u ? 0u : (e == 0x7f800000u ? 0x70000000u : 0x38000000u);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
+}
+
 constexpr int kBlock = 256;
 constexpr int kWarpBlocksBelow = 512;   // items per multiprocessor (fp64_block)
 constexpr int kDiagBlocks = 608;   // fixed grid (4 x 152 SMs): the reduction order never changes
@@ -640,6 +650,61 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
     }
 }
 
+// Start of felbm_mass_solve: rows [0, k) from B ([k][N], caller order), the
+// other rows of the planes in use (n4, see k_block32) zero; right-hand side and
+// first iterate as k_cheb_start writes them.
+template <bool kMixed>
+__global__ void __launch_bounds__(kBlock) k_solve_in(DevMesh m, Bufs b, const double* __restrict__ B, int k, int n4,
+                                                     double first_scale) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m.N) return;
+    const int Np = m.Np, o = m.perm[i];
+    const double s = m.inv_lumped[i] * first_scale;
+    double v[18];
+#pragma unroll
+    for (int q = 0; q < 18; ++q) v[q] = q < k ? B[(size_t)q * m.N + o] : 0.0;
+#pragma unroll
+    for (int p = 0; p < kPlanes; ++p) {
+        if (p >= n4 && p != 4) continue;
+        float r[4], e[4];
+#pragma unroll
+        for (int c = 0; c < (p < 4 ? 4 : 2); ++c) {
+            const int q = vec_row(p, c);
+            b.rhs[q * Np + i] = v[q];
+            if (!kMixed) b.x1[q * Np + i] = v[q] * s;
+            r[c] = (float)v[q];
+            e[c] = r[c] * (float)s;
+        }
+        if (kMixed && p < 4) {
+            store_vec(b.r32, Np, p, i, r);
+            store_vec(b.e1, Np, p, i, e);
+        } else if (kMixed) {
+            const float r2[2] = {r[0], r[1]}, e2[2] = {e[0], e[1]};
+            store_vec(b.r32, Np, 4, i, r2);
+            store_vec(b.e1, Np, 4, i, e2);
+        }
+    }
+}
+
+// End of felbm_mass_solve: rows [0, k) of x64 plus (where given) the last
+// correction e, to X ([k][N], caller order).
+__global__ void __launch_bounds__(kBlock) k_solve_out(DevMesh m, const double* __restrict__ x64,
+                                                      const float* __restrict__ e, double* X, int k, int have_x64) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m.N) return;
+    const int o = m.perm[i];
+#pragma unroll
+    for (int q = 0; q < 18; ++q) {
+        if (q >= k) continue;
+        double x = have_x64 ? x64[(size_t)q * m.Np + i] : 0.0;
+        if (e) {
+            const double ed = widen(e[vec_at(m.Np, q, i)]);
+            x = have_x64 ? x + ed : ed;
+        }
+        X[(size_t)q * m.N + o] = x;
+    }
+}
+
 // Start of a standalone solve for the right-hand sides src ([18][Np], copied
 // to rhs): x1 = first_scale * B / m_i (1/theta for the FP64 recurrence, tau_0
 // for the FP32 steps).
@@ -703,16 +768,6 @@ __global__ void __launch_bounds__(128) k_cheb(DevMesh m, Bufs b, const double* _
 // recurrence rho <- rho - M11 e with M11 in FP64.  GB300 runs FP32 FMA at
 // ~70x the FP64 rate, so only the refinement kernels pay FP64 matvecs.
 enum Final { kStore = 0, kAddPsi = 1, kAddX64 = 2, kUpdateDev = 3 };
-
-// A float as a double through the integer pipe: the conversion instruction
-// shares the FP64 pipe, whose rate is 1/64 of it.  Exact for every float
-// (the rare denormals take the instruction).
-__device__ __forceinline__ double widen(float x) {
-    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
-    if (e == 0u && (u << 1) != 0u) return (double)x;
-    const uint32_t bias = e == 0u ? 0u : (e == 0x7f800000u ? 0x70000000u : 0x38000000u);
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
-}
 
 #include "felbm_dev32.cuh"
 #include "felbm_adjoint.cuh"
@@ -929,8 +984,8 @@ __device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, co
 }
 
 __global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* e,
-                                                float* next_first, int first_round, float tau0) {
-    const int nb = (int)blockIdx.x / kPlanes, p = (int)blockIdx.x - kPlanes * nb;
+                                                float* next_first, int first_round, float tau0, int n4) {
+    const int nb = (int)blockIdx.x / (n4 + 1), l = (int)blockIdx.x - (n4 + 1) * nb, p = l < n4 ? l : 4;
     const int i = nb * (int)blockDim.x + (int)threadIdx.x;
     if (i >= m.N) return;
     if (p < 4)
@@ -1032,11 +1087,6 @@ __global__ void k_gather_out(DevMesh m, const double* __restrict__ src, double* 
     if (i >= m.N) return;
     int o = m.perm[i];
     for (int q = 0; q < rows; ++q) stage[(size_t)q * m.N + o] = src[q * m.Np + i];
-}
-__global__ void k_zero_rows(DevMesh m, double* dst, int row0, int row1) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m.N) return;
-    for (int q = row0; q < row1; ++q) dst[q * m.Np + i] = 0.0;
 }
 // Initial state at equilibrium with the fields C0, p0, u0 (caller order in
 // stage: C0 [N], then p0 [N] if has_p, then u0 [2N] as x, y if has_u; the
@@ -1757,14 +1807,14 @@ static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, si
 // where that would leave multiprocessors idle.
 template <bool kFromRhs>
 static void launch_block(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                         float* nxt, const BlockTau& bt, int K, float tau0, bool pdl) {
+                         float* nxt, const BlockTau& bt, int K, float tau0, int n4, bool pdl) {
     const bool full = m.n_blocks >= kSplitPlanesBelow * st->n_sm;
-    const dim3 grid((unsigned)m.n_blocks, full ? 1 : kPlanes);
+    const dim3 grid((unsigned)m.n_blocks, full ? 1 : n4 + 1);
     const auto go = [&](auto kern) {
         // dependent launch places the blocks of a small grid on whatever
         // multiprocessors the previous kernel has left, two on one while
         // others idle: 82 against 74 us a step on 2,112 nodes (FP64)
-        launch_k(pdl && full && st->use_pdl, kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur, nxt, bt, K, tau0);
+        launch_k(pdl && full && st->use_pdl, kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur, nxt, bt, K, tau0, n4);
     };
     switch (m.ell_w) {
         case 7: go(k_block32<7, kFromRhs>); break;
@@ -1873,7 +1923,7 @@ static bool blocked(const felbm_state* st, const DevMesh& m) { return st->sweep_
 // layers allow, of about equal length.  Returns the buffer with the last
 // iterate.
 static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, float* cur, float* prv,
-                              int k, int end, bool from_rhs, bool pdl) {
+                              int k, int end, bool from_rhs, int n4, bool pdl) {
     int left = (end - k + m.blk_steps - 1) / m.blk_steps;
     for (; left > 0; --left) {
         const int K = (end - k + left - 1) / left;
@@ -1881,9 +1931,9 @@ static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, 
         for (int j = 0; j < K; ++j) bt.tau[j] = (float)st->tau[k + j];
         const float tau0 = (float)st->tau[0];
         if (from_rhs)
-            launch_block<true>(st, m, b, s, nullptr, prv, bt, K, tau0, pdl);
+            launch_block<true>(st, m, b, s, nullptr, prv, bt, K, tau0, n4, pdl);
         else
-            launch_block<false>(st, m, b, s, cur, prv, bt, K, tau0, pdl);
+            launch_block<false>(st, m, b, s, cur, prv, bt, K, tau0, n4, pdl);
         from_rhs = false;
         pdl = true;
         k += K;
@@ -1921,10 +1971,13 @@ static void launch_mu(const DevMesh& m, const Phys& c, const Bufs& b, unsigned g
 // Enqueue the mass solve for the right-hand side in b.rhs (first iterate
 // already written, unless from_rhs).  into_psi: add the increment to psi (time step); else
 // leave the solution in x1/x0 (FP64 mode, returned) or x64 (mixed mode).
-// bufs: the buffers the solve reads and writes (the state's own, or another
-// set of scratch buffers with the same layout).
+// b: the buffers the solve reads and writes (the state's own, or another set of
+// scratch buffers with the same layout).  n4: planes in use (k_block32; blocked
+// solves only).  last: where given (blocked, not into_psi), the last correction
+// is not added to x64 but returned through it.
 static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s,
-                                   bool into_psi, bool after_release = false, bool from_rhs = false) {
+                                   bool into_psi, bool after_release = false, bool from_rhs = false, int n4 = 4,
+                                   const float** last = nullptr) {
     const int nb = fp64_block(st, m.N, 128);
     const unsigned grid = grid_for(m.N, nb);
     if (st->mode == FELBM_SOLVER_FP64) {
@@ -1949,19 +2002,21 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
             bool pdl = r == 0 && after_release;
             int k = 1;
             if (last_round && st->check) {
-                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, false, pdl);
+                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, false, n4, pdl);
                 prv = x == cur ? prv : cur;
                 cur = x;
                 enqueue_resid(st, m, b, s, cur);
                 k = st->sweeps - 1;
                 pdl = false;
             }
-            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, from_rhs && r == 0, pdl);
+            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, from_rhs && r == 0, n4, pdl);
             prv = x == cur ? prv : cur;
             cur = x;
             if (last_round && into_psi && st->dev32)
                 launch_k(st->use_pdl, k_update32, dim3(grid_for(m.N, 128)), dim3(128), 0, s, m, st->phys, b,
                          (const float*)cur);
+            else if (last_round && last)
+                *last = cur;
             else if (last_round)
                 launch_k(st->use_pdl, into_psi ? k_add64<true> : k_add64<false>, dim3(grid), dim3(nb), 0, s, m, b,
                          (const float*)cur, have_x64);
@@ -1988,12 +2043,29 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
             std::swap(cur, prv);
         }
         if (!last_round) {
-            k_refine<<<grid * kPlanes, nb, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0]);
+            k_refine<<<grid * (n4 + 1), nb, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0], n4);
             A = prv;
             B = cur;
         }
     }
     return b.x64;
+}
+
+// X = M11^{-1} B for rows [0, k) (device, caller order), with scratch b.  A
+// blocked solve takes only the planes that hold those rows: 5 of 18 rows on
+// 80,000 nodes take 168 us instead of 378.
+static void enqueue_mass_solve(felbm_state* st, const Bufs& b, const double* B, double* X, int k, cudaStream_t s) {
+    const DevMesh& m = st->dm;
+    const unsigned grid = grid_for(m.N, kBlock);
+    const bool part = blocked(st, m) && !st->check;   // the checked residual covers all rows
+    const int n4 = !part ? 4 : (k <= 1 ? 0 : k <= 5 ? 1 : k <= 10 ? 2 : k <= 14 ? 3 : 4);
+    if (st->mode == FELBM_SOLVER_FP64)
+        k_solve_in<false><<<grid, kBlock, 0, s>>>(m, b, B, k, n4, st->inv_theta);
+    else
+        k_solve_in<true><<<grid, kBlock, 0, s>>>(m, b, B, k, n4, st->tau[0]);
+    const float* last = nullptr;
+    const double* x = enqueue_solve(st, m, b, s, false, false, false, n4, part ? &last : nullptr);
+    k_solve_out<<<grid, kBlock, 0, s>>>(m, x, last, X, k, !last || st->rounds > 1);
 }
 
 static int solve_launches(const felbm_state* st) {
@@ -2937,14 +3009,7 @@ int felbm_mass_solve(felbm_state* st, const double* B, double* X, int32_t k) {
     const DevMesh& m = st->dm;
     const Bufs& b = st->buf;
     FELBM_CUDA(cudaMemcpyAsync(b.stage, B, sizeof(double) * k * m.N, cudaMemcpyHostToDevice, s));
-    k_scatter_in<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b.stage, b.rhs, k);
-    if (k < 18) k_zero_rows<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b.rhs, k, 18);
-    if (st->mode == FELBM_SOLVER_FP64)
-        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, b.rhs, st->inv_theta);
-    else
-        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, b, b.rhs, st->tau[0]);
-    const double* result = enqueue_solve(st, st->dm, b, s, false);
-    k_gather_out<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, result, b.stage, k);
+    enqueue_mass_solve(st, b, b.stage, b.stage, k, s);
     FELBM_CUDA(cudaGetLastError());
     FELBM_CUDA(cudaMemcpyAsync(X, b.stage, sizeof(double) * k * m.N, cudaMemcpyDeviceToHost, s));
     FELBM_CUDA(cudaStreamSynchronize(s));
@@ -3025,14 +3090,7 @@ int felbm_mass_solve_static(felbm_state* st, const double* d_B, double* d_X, int
     sb.e0 = sc.take<float>(rows);
     sb.e1 = sc.take<float>(rows);
     cudaStream_t s = st->stream;
-    k_scatter_in<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, d_B, sb.rhs, k);
-    if (k < 18) k_zero_rows<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb.rhs, k, 18);
-    if (st->mode == FELBM_SOLVER_FP64)
-        k_cheb_start<false><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, sb.rhs, st->inv_theta);
-    else
-        k_cheb_start<true><<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, sb, sb.rhs, st->tau[0]);
-    const double* result = enqueue_solve(st, st->dm, sb, s, false);
-    k_gather_out<<<grid_for(m.N, kBlock), kBlock, 0, s>>>(m, result, d_X, k);
+    enqueue_mass_solve(st, sb, d_B, d_X, k, s);
     FELBM_CUDA(cudaGetLastError());
     return FELBM_OK;
 }

@@ -152,12 +152,13 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
     return free;
 }
 
-// kW: ELL width; kFromRhs: x_0 = tau_0 b / m formed here.  Grid: blocks x (1 or kPlanes): all planes of
-// a block in turn, or one.
+// kW: ELL width; kFromRhs: x_0 = tau_0 b / m formed here.  n4: float4 planes in
+// use (the first n4 of them, and always the rest plane).  Grid: blocks x (1 or
+// n4 + 1): all planes in use of a block in turn, or one.
 template <int kW, bool kFromRhs>
 __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
     k_block32(DevMesh m, Bufs b, const float* cur, float* nxt, const __grid_constant__ BlockTau bt, int K,
-              float tau0) {
+              float tau0, int n4) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BlockSmem& sm = *reinterpret_cast<BlockSmem*>(smem_raw);
     pdl_release();
@@ -179,12 +180,14 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
         node[n] = r < ni ? s0 + r : (r < nreg ? halo[r] : s0);
         im[n] = m.inv_lumped32[node[n]];
     }
-    const int p0 = (int)blockIdx.y, p1 = gridDim.y > 1 ? p0 + 1 : kPlanes;
+    const bool one = gridDim.y > 1;
+    const int p0 = one ? (int)blockIdx.y : 0, p1 = one ? min(p0 + 1, n4) : n4;   // float4 planes [p0, p1)
+    const bool rest = !one || p0 == n4;
     pdl_wait();
-    if (p0 < 4)
+    if (p0 < p1)
         block_fetch<4, kFromRhs>(sm, m, b, cur, K, p0, 0, node);
     else
-        block_fetch<2, kFromRhs>(sm, m, b, cur, K, p0, 0, node);
+        block_fetch<2, kFromRhs>(sm, m, b, cur, K, 4, 0, node);
 #pragma unroll
     for (int n = 0; n < kBlockNpt; ++n) {
         const int r = tid + n * kBlockThreads;
@@ -196,10 +199,10 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
         }
     }
     int buf = 0;
-    for (int p = p0; p < min(p1, 4); ++p)
+    for (int p = p0; p < p1; ++p)
         buf = block_plane<4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, p,
-                                                   p + 1 < p1 ? p + 1 : kPlanes, buf, node, val, col, im);
-    if (p1 == kPlanes)
+                                           p + 1 < p1 ? p + 1 : (rest ? 4 : kPlanes), buf, node, val, col, im);
+    if (rest)
         block_plane<2, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, 4, kPlanes, buf, node, val, col, im);
 }
 

@@ -98,3 +98,18 @@ def test_fused_forces_match_the_fp64_step(case):
     (g, h), (gr, hr) = st.get_state(), ref.get_state()
     assert np.abs(h - hr).max() < 1e-6 * np.abs(hr).max()
     assert np.abs(g - gr).max() < 1e-4 * np.abs(gr).max()
+
+
+@pytest.mark.parametrize("precision", [F.FP64, F.FP32_DEV])
+@pytest.mark.parametrize("case", ["two blocks", "all planes per block"])
+def test_mass_solve_of_some_rows(case, precision):
+    """The blocked solve takes only the planes that hold the requested rows: at
+    every boundary of the planes the rows are those of the gathered solve of all."""
+    w = CASES[case]()
+    mesh, params = F.Mesh.from_dict(w["mesh"]), F.params_derive(w["phys"], precision=precision)
+    a, b = (F.State(mesh, params, w["C0"]) for _ in range(2))
+    a.sweep_tiled(False)
+    B = np.random.default_rng(4).standard_normal((18, len(w["C0"])))
+    X = a.mass_solve(B)
+    for k in (18, 1, 2, 5, 6, 9, 10, 11, 14, 15):
+        np.testing.assert_array_equal(b.mass_solve(B[:k]), X[:k])
