@@ -1803,23 +1803,25 @@ static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, si
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// One blocked launch: K steps from cur (or from b) to nxt.  All planes of a block in one thread block; one plane each
-// where that would leave multiprocessors idle.
+// One blocked launch: K steps from cur (or from b) to nxt.  All planes of a
+// block in one thread block; one plane or pair of right-hand sides each where
+// that would leave multiprocessors idle.
 template <bool kFromRhs>
 static void launch_block(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
                          float* nxt, const BlockTau& bt, int K, float tau0, int n4, bool pdl) {
-    const bool full = m.n_blocks >= kSplitPlanesBelow * st->n_sm;
-    const dim3 grid((unsigned)m.n_blocks, full ? 1 : n4 + 1);
-    const auto go = [&](auto kern) {
+    const bool full = m.n_blocks >= kSplitPlanesBelow * st->n_sm, pairs = split_pairs(m.n_blocks, st->n_sm);
+    const dim3 grid((unsigned)m.n_blocks, full ? 1 : (pairs ? 2 * n4 + 1 : n4 + 1));
+    const auto go = [&](auto kern, auto pair_kern) {
         // dependent launch places the blocks of a small grid on whatever
         // multiprocessors the previous kernel has left, two on one while
         // others idle: 82 against 74 us a step on 2,112 nodes (FP64)
-        launch_k(pdl && full && st->use_pdl, kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m, b, cur, nxt, bt, K, tau0, n4);
+        launch_k(pdl && full && st->use_pdl, pairs ? pair_kern : kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m,
+                 b, cur, nxt, bt, K, tau0, n4);
     };
     switch (m.ell_w) {
-        case 7: go(k_block32<7, kFromRhs>); break;
-        case 9: go(k_block32<9, kFromRhs>); break;
-        default: go(k_block32<12, kFromRhs>);
+        case 7: go(k_block32<7, kFromRhs, false>, k_block32<7, kFromRhs, true>); break;
+        case 9: go(k_block32<9, kFromRhs, false>, k_block32<9, kFromRhs, true>); break;
+        default: go(k_block32<12, kFromRhs, false>, k_block32<12, kFromRhs, true>);
     }
 }
 
@@ -1831,8 +1833,10 @@ static cudaError_t allow_block_smem() {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSmem));
     };
-    set(k_block32<kW, false>);
-    set(k_block32<kW, true>);
+    set(k_block32<kW, false, false>);
+    set(k_block32<kW, true, false>);
+    set(k_block32<kW, false, true>);
+    set(k_block32<kW, true, true>);
     return e;
 }
 

@@ -34,28 +34,32 @@
 constexpr int kHaloMax = 504;          // largest first layer of a tile (felbm_sweep_tiled's limit)
 constexpr int kBlockThreads = 512;
 constexpr int kBlockNpt = kBlockNodes / kBlockThreads;      // nodes per thread
-// Fewer blocks than this per multiprocessor run one plane per thread block (a
-// plane at a time leaves the chip idle): 2,048 nodes spread over 20 thread
-// blocks instead of 4.  From one block per multiprocessor on, five planes on
-// the same rows are the faster form: 84 us against 88 us for the solve on
-// 131,072 nodes (256 blocks), 1,618 against 1,771 us on 520,704 (FP64).
+// Fewer blocks than this per multiprocessor run one plane per thread block (all
+// planes in one leave the chip idle); from one block per multiprocessor on, five
+// planes on the same rows are the faster form: 84 us against 88 us for the solve
+// on 131,072 nodes (256 blocks), 1,618 against 1,771 us on 520,704 (FP64).
+// Where even nine thread blocks per block fit the chip one to a multiprocessor,
+// one pair of right-hand sides each: 72 us a step against 78 on 2,112 nodes (8
+// blocks, FP64); on 18,432 nodes (64 blocks) 160 against 148.
 constexpr int kSplitPlanesBelow = 1;
+static bool split_pairs(int n_blocks, int n_sm) { return 9 * n_blocks <= n_sm; }
 
 struct BlockTau {
     float tau[kBlockSteps];
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-template <int NV>
-__device__ __forceinline__ void cp_async_vec(float* dst, const float* x, int Np, int p, int i) {
+// A piece of the FP32 vectors: NV consecutive values of node i at x + off +
+// kStride i -- a plane of vec_at (NV 4, stride 4; rest plane NV 2, stride 2) or
+// half of a float4 plane (NV 2, stride 4).
+__device__ __forceinline__ uint32_t plane_off(int Np, int p) { return (p < 4 ? 4u * p : 16u) * (uint32_t)Np; }
+template <int NV, int kStride>
+__device__ __forceinline__ void cp_async_piece(float* dst, const float* x, uint32_t off, int i) {
+    const float* src = x + off + (size_t)kStride * i;
     if constexpr (NV == 4)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)),
-                     "l"(x + ((size_t)p * Np + i) * 4)
-                     : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
     else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)),
-                     "l"(x + (size_t)16 * Np + 2 * (size_t)i)
-                     : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 
 // Shared memory of a block: three copies of x (two for the steps, one that
@@ -66,29 +70,29 @@ struct BlockSmem {
     int cnt[kBlockSteps + 1];          // nodes up to each layer
 };
 
-// Queue the copies of plane p: x_k on the region into x[buf], b on the nodes
+// Queue the copies of the piece at off: x_k on the region into x[buf], b on the nodes
 // that are stepped (kFromRhs: b on the whole region and no x).
-template <int NV, bool kFromRhs>
-__device__ __forceinline__ void block_fetch(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* cur, int K, int p,
+template <int NV, int kStride, bool kFromRhs>
+__device__ __forceinline__ void block_fetch(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* cur, int K, uint32_t off,
                                             int buf, const int (&node)[kBlockNpt]) {
 #pragma unroll
     for (int n = 0; n < kBlockNpt; ++n) {
         const int r = (int)threadIdx.x + n * kBlockThreads;
-        if (r < sm.cnt[kFromRhs ? K : K - 1]) cp_async_vec<NV>(sm.b + r * NV, b.r32, m.Np, p, node[n]);
-        if (!kFromRhs && r < sm.cnt[K]) cp_async_vec<NV>(sm.x[buf] + r * NV, cur, m.Np, p, node[n]);
+        if (r < sm.cnt[kFromRhs ? K : K - 1]) cp_async_piece<NV, kStride>(sm.b + r * NV, b.r32, off, node[n]);
+        if (!kFromRhs && r < sm.cnt[K]) cp_async_piece<NV, kStride>(sm.x[buf] + r * NV, cur, off, node[n]);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// The K steps of plane p, whose copies into x[buf] and b were queued by this
+// The K steps of the piece at off, whose copies into x[buf] and b were queued by this
 // thread; queues those of plane `next` (kPlanes: none) into the third buffer,
 // which it returns.
-template <int NV, int kW, bool kFromRhs>
+template <int NV, int kStride, int kW, bool kFromRhs>
 __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* cur,
-                                           float* nxt, const BlockTau& bt, int K, float tau0, int p, int next, int buf, const int (&node)[kBlockNpt],
+                                           float* nxt, const BlockTau& bt, int K, float tau0, uint32_t off, int next, int buf, const int (&node)[kBlockNpt],
                                            const float (&val)[kBlockNpt][kW], const uint32_t (&col)[kBlockNpt][kW / 2],
                                            const float (&im)[kBlockNpt]) {
-    const int Np = m.Np, tid = (int)threadIdx.x;
+    const int tid = (int)threadIdx.x;
     float x[kBlockNpt][NV], rr[kBlockNpt][NV];
     int ia = buf, ib = buf == 2 ? 0 : buf + 1;
     const int free = ib == 2 ? 0 : ib + 1;
@@ -112,9 +116,9 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
     }
     __syncthreads();
     if (next < 4)
-        block_fetch<4, kFromRhs>(sm, m, b, cur, K, next, free, node);
+        block_fetch<4, 4, kFromRhs>(sm, m, b, cur, K, plane_off(m.Np, next), free, node);
     else if (next == 4)
-        block_fetch<2, kFromRhs>(sm, m, b, cur, K, next, free, node);
+        block_fetch<2, 2, kFromRhs>(sm, m, b, cur, K, plane_off(m.Np, 4), free, node);
     for (int step = 1; step <= K; ++step) {
         const int nc = sm.cnt[K - step];
         const float tau = bt.tau[step - 1];
@@ -141,7 +145,7 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
                 if (step < K)
                     store_shared(xb + r * NV, x[n]);
                 else
-                    store_vec(nxt, Np, p, node[n], x[n]);
+                    store_shared(nxt + off + (size_t)kStride * node[n], x[n]);
             }
         }
         if (step < K) __syncthreads();
@@ -153,9 +157,10 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
 }
 
 // kW: ELL width; kFromRhs: x_0 = tau_0 b / m formed here.  n4: float4 planes in
-// use (the first n4 of them, and always the rest plane).  Grid: blocks x (1 or
-// n4 + 1): all planes in use of a block in turn, or one.
-template <int kW, bool kFromRhs>
+// use (the first n4 of them, and always the rest plane).  Grid: blocks x 1 (all
+// planes in use of a block in turn), blocks x (n4 + 1) (a plane each) or, kPair,
+// blocks x (2 n4 + 1) (a pair of right-hand sides each).
+template <int kW, bool kFromRhs, bool kPair>
 __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
     k_block32(DevMesh m, Bufs b, const float* cur, float* nxt, const __grid_constant__ BlockTau bt, int K,
               float tau0, int n4) {
@@ -180,14 +185,18 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
         node[n] = r < ni ? s0 + r : (r < nreg ? halo[r] : s0);
         im[n] = m.inv_lumped32[node[n]];
     }
+    const int y = (int)blockIdx.y;
     const bool one = gridDim.y > 1;
-    const int p0 = one ? (int)blockIdx.y : 0, p1 = one ? min(p0 + 1, n4) : n4;   // float4 planes [p0, p1)
-    const bool rest = !one || p0 == n4;
+    const int p0 = one ? y : 0, p1 = one ? min(y + 1, n4) : n4;      // float4 planes [p0, p1)
+    const bool rest = kPair ? y == 2 * n4 : (!one || y == n4);
+    const uint32_t half = plane_off(m.Np, y >> 1) + 2 * (y & 1);
     pdl_wait();
-    if (p0 < p1)
-        block_fetch<4, kFromRhs>(sm, m, b, cur, K, p0, 0, node);
+    if (kPair && !rest)
+        block_fetch<2, 4, kFromRhs>(sm, m, b, cur, K, half, 0, node);
+    else if (!kPair && p0 < p1)
+        block_fetch<4, 4, kFromRhs>(sm, m, b, cur, K, plane_off(m.Np, p0), 0, node);
     else
-        block_fetch<2, kFromRhs>(sm, m, b, cur, K, 4, 0, node);
+        block_fetch<2, 2, kFromRhs>(sm, m, b, cur, K, plane_off(m.Np, 4), 0, node);
 #pragma unroll
     for (int n = 0; n < kBlockNpt; ++n) {
         const int r = tid + n * kBlockThreads;
@@ -199,11 +208,17 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
         }
     }
     int buf = 0;
-    for (int p = p0; p < p1; ++p)
-        buf = block_plane<4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, p,
-                                           p + 1 < p1 ? p + 1 : (rest ? 4 : kPlanes), buf, node, val, col, im);
+    if constexpr (kPair) {
+        if (!rest)
+            block_plane<2, 4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, half, kPlanes, 0, node, val, col, im);
+    } else {
+        for (int p = p0; p < p1; ++p)
+            buf = block_plane<4, 4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, p),
+                                                  p + 1 < p1 ? p + 1 : (rest ? 4 : kPlanes), buf, node, val, col, im);
+    }
     if (rest)
-        block_plane<2, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, 4, kPlanes, buf, node, val, col, im);
+        block_plane<2, 2, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, 4), kPlanes, buf, node, val, col,
+                                        im);
 }
 
 // The field and deviation update from the solve's last iterate (FP32-deviation
