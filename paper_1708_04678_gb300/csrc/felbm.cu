@@ -1808,20 +1808,20 @@ static void launch_k(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, si
 // that would leave multiprocessors idle.
 template <bool kFromRhs>
 static void launch_block(const felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, const float* cur,
-                         float* nxt, const BlockTau& bt, int K, float tau0, int n4, bool pdl) {
+                         float* nxt, const BlockTau& bt, int K, float tau0, int n4, bool update, bool pdl) {
     const bool full = m.n_blocks >= kSplitPlanesBelow * st->n_sm, pairs = split_pairs(m.n_blocks, st->n_sm);
     const dim3 grid((unsigned)m.n_blocks, full ? 1 : (pairs ? 2 * n4 + 1 : n4 + 1));
-    const auto go = [&](auto kern, auto pair_kern) {
+    const auto go = [&](auto kern, auto pair_kern, auto update_kern) {
         // dependent launch places the blocks of a small grid on whatever
         // multiprocessors the previous kernel has left, two on one while
         // others idle: 82 against 74 us a step on 2,112 nodes (FP64)
-        launch_k(pdl && full && st->use_pdl, pairs ? pair_kern : kern, grid, dim3(kBlockThreads), sizeof(BlockSmem), s, m,
-                 b, cur, nxt, bt, K, tau0, n4);
+        launch_k(pdl && full && st->use_pdl, update ? update_kern : (pairs ? pair_kern : kern), grid, dim3(kBlockThreads),
+                 update ? sizeof(BlockUpdateSmem) : sizeof(BlockSmem), s, m, st->phys, b, cur, nxt, bt, K, tau0, n4);
     };
     switch (m.ell_w) {
-        case 7: go(k_block32<7, kFromRhs, false>, k_block32<7, kFromRhs, true>); break;
-        case 9: go(k_block32<9, kFromRhs, false>, k_block32<9, kFromRhs, true>); break;
-        default: go(k_block32<12, kFromRhs, false>, k_block32<12, kFromRhs, true>);
+        case 7: go(k_block32<7, kFromRhs, false>, k_block32<7, kFromRhs, true>, k_block32<7, false, false, true>); break;
+        case 9: go(k_block32<9, kFromRhs, false>, k_block32<9, kFromRhs, true>, k_block32<9, false, false, true>); break;
+        default: go(k_block32<12, kFromRhs, false>, k_block32<12, kFromRhs, true>, k_block32<12, false, false, true>);
     }
 }
 
@@ -1831,12 +1831,13 @@ static cudaError_t allow_block_smem() {
     cudaError_t e = cudaSuccess;
     const auto set = [&](auto kern) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockSmem));
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockUpdateSmem));
     };
     set(k_block32<kW, false, false>);
     set(k_block32<kW, true, false>);
     set(k_block32<kW, false, true>);
     set(k_block32<kW, true, true>);
+    set(k_block32<kW, false, false, true>);
     return e;
 }
 
@@ -1923,11 +1924,21 @@ static void launch_first(felbm_state* st, const DevMesh& m, const Bufs& b, cudaS
 // Whether the solve on m runs blocked.
 static bool blocked(const felbm_state* st, const DevMesh& m) { return st->sweep_tiled && m.blk_steps > 0; }
 
+static bool first_from_rhs(const felbm_state* st, const DevMesh& m);
+
+// Whether the last launch of an FP32-deviation state's solve, whose first step
+// is `first`, updates fields and deviations: all planes in one thread block, and
+// not the launch that forms x_0.
+static bool fused_update(const felbm_state* st, const DevMesh& m, int first) {
+    return st->dev32 && m.n_blocks >= kSplitPlanesBelow * st->n_sm &&
+           (first > 1 || st->sweeps - 1 > m.blk_steps || !first_from_rhs(st, m));
+}
+
 // The steps [k, end) of one correction in as few blocked launches as the
-// layers allow, of about equal length.  Returns the buffer with the last
-// iterate.
+// layers allow, of about equal length.  update: the last launch also updates
+// fields and deviations (fused_update).  Returns the buffer with the last iterate.
 static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s, float* cur, float* prv,
-                              int k, int end, bool from_rhs, int n4, bool pdl) {
+                              int k, int end, bool from_rhs, int n4, bool update, bool pdl) {
     int left = (end - k + m.blk_steps - 1) / m.blk_steps;
     for (; left > 0; --left) {
         const int K = (end - k + left - 1) / left;
@@ -1935,9 +1946,9 @@ static float* enqueue_blocked(felbm_state* st, const DevMesh& m, const Bufs& b, 
         for (int j = 0; j < K; ++j) bt.tau[j] = (float)st->tau[k + j];
         const float tau0 = (float)st->tau[0];
         if (from_rhs)
-            launch_block<true>(st, m, b, s, nullptr, prv, bt, K, tau0, n4, pdl);
+            launch_block<true>(st, m, b, s, nullptr, prv, bt, K, tau0, n4, false, pdl);
         else
-            launch_block<false>(st, m, b, s, cur, prv, bt, K, tau0, n4, pdl);
+            launch_block<false>(st, m, b, s, cur, prv, bt, K, tau0, n4, update && left == 1, pdl);
         from_rhs = false;
         pdl = true;
         k += K;
@@ -2006,19 +2017,22 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
             bool pdl = r == 0 && after_release;
             int k = 1;
             if (last_round && st->check) {
-                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, false, n4, pdl);
+                float* const x = enqueue_blocked(st, m, b, s, cur, prv, 1, st->sweeps - 1, false, n4, false, pdl);
                 prv = x == cur ? prv : cur;
                 cur = x;
                 enqueue_resid(st, m, b, s, cur);
                 k = st->sweeps - 1;
                 pdl = false;
             }
-            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, from_rhs && r == 0, n4, pdl);
+            const bool update = last_round && into_psi && fused_update(st, m, k);
+            float* const x = enqueue_blocked(st, m, b, s, cur, prv, k, st->sweeps, from_rhs && r == 0, n4, update, pdl);
             prv = x == cur ? prv : cur;
             cur = x;
-            if (last_round && into_psi && st->dev32)
+            if (last_round && into_psi && st->dev32 && !update)
                 launch_k(st->use_pdl, k_update32, dim3(grid_for(m.N, 128)), dim3(128), 0, s, m, st->phys, b,
                          (const float*)cur);
+            else if (last_round && into_psi && st->dev32)
+                ;   // updated in the last launch
             else if (last_round && last)
                 *last = cur;
             else if (last_round)
@@ -2079,7 +2093,8 @@ static int solve_launches(const felbm_state* st) {
     const int most = st->dm.blk_steps;
     const auto groups = [&](int steps) { return (steps + most - 1) / most; };
     const int last = st->check ? groups(st->sweeps - 2) + 1 : groups(st->sweeps - 1);
-    return refines * (groups(st->sweeps - 1) + 1) + last + 1;
+    const bool update = fused_update(st, st->dm, st->check ? st->sweeps - 1 : 1);
+    return refines * (groups(st->sweeps - 1) + 1) + last + (update ? 0 : 1);
 }
 
 // FP32 states: residuals and their gather in one kernel (k_force32) from this

@@ -22,15 +22,15 @@
 // step and about 1.4 times the conflict-free count; DRAM is 20 % busy.  Solve
 // phase of the time step, field update included (GB300):
 //                                    step at a time   blocked
-//   2,082,816 nodes, FP32, 10 steps      1,098 us      792 us
-//     131,072 nodes, FP32, 10 steps        109 us       84 us (rows of 9)
-//     520,704 nodes, FP64, 3 x 14        2,019 us    1,618 us (FP64 refinement included)
-//       2,112 nodes, FP64, 3 x 14          164 us       71 us
+//   2,082,816 nodes, FP32, 10 steps      1,098 us      758 us
+//     131,072 nodes, FP32, 10 steps        109 us       82 us (rows of 9)
+//     520,704 nodes, FP64, 3 x 14        2,019 us    1,303 us (FP64 refinement included)
+//       2,112 nodes, FP64, 3 x 14          164 us       43 us
 // Blocks of 512 nodes at 64 registers put two thread blocks on a
 // multiprocessor, one computing while the other loads.  With blocks of 1,024
 // nodes, 128 registers and one thread block the 2.08M-node phase took 1,157 us,
-// without the cp.async prefetch 942 us.
-
+// without the cp.async prefetch 942 us, with two steps a launch 889 us (blocked
+// phase then 792 us).
 constexpr int kHaloMax = 504;          // largest first layer of a tile (felbm_sweep_tiled's limit)
 constexpr int kBlockThreads = 512;
 constexpr int kBlockNpt = kBlockNodes / kBlockThreads;      // nodes per thread
@@ -69,6 +69,11 @@ struct BlockSmem {
     float b[kBlockNodes * 4];
     int cnt[kBlockSteps + 1];          // nodes up to each layer
 };
+// With the field update in the last launch: the increments of the block's own
+// nodes, piece by piece ([18][kBlockCore] floats).
+struct BlockUpdateSmem : BlockSmem {
+    alignas(16) float d[18 * kBlockCore];
+};
 
 // Queue the copies of the piece at off: x_k on the region into x[buf], b on the nodes
 // that are stepped (kFromRhs: b on the whole region and no x).
@@ -87,7 +92,7 @@ __device__ __forceinline__ void block_fetch(BlockSmem& sm, const DevMesh& m, con
 // The K steps of the piece at off, whose copies into x[buf] and b were queued by this
 // thread; queues those of plane `next` (kPlanes: none) into the third buffer,
 // which it returns.
-template <int NV, int kStride, int kW, bool kFromRhs>
+template <int NV, int kStride, int kW, bool kFromRhs, bool kUpdate>
 __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, const Bufs& b, const float* cur,
                                            float* nxt, const BlockTau& bt, int K, float tau0, uint32_t off, int next, int buf, const int (&node)[kBlockNpt],
                                            const float (&val)[kBlockNpt][kW], const uint32_t (&col)[kBlockNpt][kW / 2],
@@ -145,7 +150,9 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
                 if (step < K)
                     store_shared(xb + r * NV, x[n]);
                 else
-                    store_shared(nxt + off + (size_t)kStride * node[n], x[n]);
+                    store_shared(kUpdate ? nxt + (size_t)(off / (uint32_t)m.Np) * kBlockCore + kStride * r
+                                         : nxt + off + (size_t)kStride * node[n],
+                                 x[n]);
             }
         }
         if (step < K) __syncthreads();
@@ -159,11 +166,15 @@ __device__ __forceinline__ int block_plane(BlockSmem& sm, const DevMesh& m, cons
 // kW: ELL width; kFromRhs: x_0 = tau_0 b / m formed here.  n4: float4 planes in
 // use (the first n4 of them, and always the rest plane).  Grid: blocks x 1 (all
 // planes in use of a block in turn), blocks x (n4 + 1) (a plane each) or, kPair,
-// blocks x (2 n4 + 1) (a pair of right-hand sides each).
-template <int kW, bool kFromRhs, bool kPair>
+// blocks x (2 n4 + 1) (a pair of right-hand sides each).  kUpdate (first form,
+// all planes): the last iterate is the increment of the time step; it stays in
+// shared memory and the fields and deviations are updated here, which saves
+// writing and reading it: solve phase 788 -> 758 us on 2,082,816 nodes.
+template <int kW, bool kFromRhs, bool kPair, bool kUpdate = false>
 __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
-    k_block32(DevMesh m, Bufs b, const float* cur, float* nxt, const __grid_constant__ BlockTau bt, int K,
+    k_block32(DevMesh m, Phys c, Bufs b, const float* cur, float* nxt, const __grid_constant__ BlockTau bt, int K,
               float tau0, int n4) {
+    static_assert(!(kPair && kUpdate), "the update needs all planes");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BlockSmem& sm = *reinterpret_cast<BlockSmem*>(smem_raw);
     pdl_release();
@@ -208,17 +219,30 @@ __global__ void __launch_bounds__(kBlockThreads, kW <= 9 ? 2 : 1)
         }
     }
     int buf = 0;
+    if constexpr (kUpdate) nxt = static_cast<BlockUpdateSmem&>(sm).d;
     if constexpr (kPair) {
         if (!rest)
-            block_plane<2, 4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, half, kPlanes, 0, node, val, col, im);
+            block_plane<2, 4, kW, kFromRhs, false>(sm, m, b, cur, nxt, bt, K, tau0, half, kPlanes, 0, node, val, col, im);
     } else {
         for (int p = p0; p < p1; ++p)
-            buf = block_plane<4, 4, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, p),
+            buf = block_plane<4, 4, kW, kFromRhs, kUpdate>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, p),
                                                   p + 1 < p1 ? p + 1 : (rest ? 4 : kPlanes), buf, node, val, col, im);
     }
     if (rest)
-        block_plane<2, 2, kW, kFromRhs>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, 4), kPlanes, buf, node, val, col,
+        block_plane<2, 2, kW, kFromRhs, kUpdate>(sm, m, b, cur, nxt, bt, K, tau0, plane_off(m.Np, 4), kPlanes, buf, node, val, col,
                                         im);
+    if constexpr (kUpdate) {
+        __syncthreads();
+        if (tid < ni) {
+            float d[18];
+#pragma unroll
+            for (int p = 0; p < kPlanes; ++p)
+#pragma unroll
+                for (int v = 0; v < (p < 4 ? 4 : 2); ++v)
+                    d[vec_row(p, v)] = nxt[(4 * p) * kBlockCore + (p < 4 ? 4 : 2) * tid + v];
+            dev32_update(m, c, b, s0 + tid, d);
+        }
+    }
 }
 
 // The field and deviation update from the solve's last iterate (FP32-deviation
