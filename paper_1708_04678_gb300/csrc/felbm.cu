@@ -2374,7 +2374,7 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
             std::vector<int32_t> blk, at;      // a node's index in the list of the block that saw it last
         };
         const auto make = [&]() { return Index{std::vector<int32_t>(h.N, -1), std::vector<int32_t>(h.N)}; };
-        parallel_for(nblk, 32, make, [&](int32_t t, Index& ix) {
+        parallel_for(nblk, 4, make, [&](int32_t t, Index& ix) {
             const int32_t s0 = h.blk_ptr[t], ni = h.blk_ptr[t + 1] - s0;
             const int32_t* cnt = h.layer_cnt.data() + (size_t)t * (kBlockSteps + 1);
             const int32_t* halo = h.halo.data() + h.halo_ptr[t];
@@ -2491,7 +2491,7 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
         std::vector<uint16_t> iloc;
         if (st->dm.max_blk_tri > 0) {
             iloc.resize((size_t)iw * Npi);
-            parallel_for(nblk, 32, []() { return 0; }, [&](int32_t t, int&) {
+            parallel_for(nblk, 4, []() { return 0; }, [&](int32_t t, int&) {
                 const int32_t* l0 = h.blk_tri.data() + h.blk_tri_ptr[t];
                 const int32_t* l1 = h.blk_tri.data() + h.blk_tri_ptr[t + 1];
                 for (int32_t i = h.blk_ptr[t]; i < h.blk_ptr[t + 1]; ++i)
