@@ -100,19 +100,35 @@ __device__ __forceinline__ Dir4 lane_dirs(int c) {
 // only FP64 work: C differences) into shared memory; (B) five-lane groups
 // take one tetrahedron at a time, lane c its directions 4c..4c+3 of both
 // sets, reading the vertices' deviation rows as whole contiguous rows.
+//
+// The equilibrium part of e.grad psi_hat is linear in dC_n, dp_n and
+// dG_n = Gamma_n - Gamma_0, so per vertex only sum (e.b_n) dG_n and
+// sum (e.b_n) dC_n dG_n are formed; the rest is e.grad C and e.grad p, which
+// the forces need as well.  With the per-vertex differences of the equilibria
+// themselves and one 4-byte load per element quantity the kernel was bound by
+// instructions (66 % of the issue slots) and shared-memory wavefronts (41 % of
+// the L1's 68 %): 1,572,864 tetrahedra took 235 us, now 200 us.  95 registers
+// (5 blocks per SM); 80 and 72 spill: 215 and 292 us.
 constexpr int kElemTets = kCoopBlock;
-enum ElemField {
-    EF_V, EF_C0, EF_DC1, EF_DC2, EF_DC3, EF_DP1, EF_DP2, EF_DP3, EF_U0X, EF_U0Y, EF_U0Z,
-    EF_DU1X, EF_DU1Y, EF_DU1Z, EF_DU2X, EF_DU2Y, EF_DU2Z, EF_DU3X, EF_DU3Y, EF_DU3Z,
-    EF_OM0, EF_OM1, EF_OM2, EF_OM3, EF_DSU1, EF_DSU2, EF_DSU3,
-    EF_B1X, EF_B1Y, EF_B1Z, EF_B2X, EF_B2Y, EF_B2Z, EF_B3X, EF_B3Y, EF_B3Z,
-    EF_UBX, EF_UBY, EF_UBZ, EF_MUB, EF_UUB, EF_UU0, EF_RHO0, EF_GRX, EF_GRY, EF_GRZ, EF_GCX, EF_GCY, EF_GCZ,
-    EF_VHX, EF_VHY, EF_VHZ, EF_UGR, EF_UGC, EF_UVH, EF_MLAP, EF_COUNT
+// Element quantities of one tetrahedron, 13 16-byte words (an odd number, so
+// that neither the threads' rows of phase A nor the groups' of phase B share
+// banks); every word is one load of a group.
+enum ElemWord {
+    EW_S,              // V, C_0, rho_0 / 3, mean mu
+    EW_U0,             // u_0, 1.5 u_0^2
+    EW_UB,             // mean u, 1.5 of its square
+    EW_GC,             // grad C, (mean u).grad C
+    EW_GP,             // grad p, f
+    EW_OM,             // 1 - omega of the vertices
+    EW_H,              // 1 + f mu, M lap mu - (mean u).v_h
+    EW_B1, EW_B2, EW_B3,   // shape gradient, dC
+    EW_D1, EW_D2, EW_D3,   // du, 1.5 (u_n^2 - u_0^2)
+    EW_COUNT
 };
 
 __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, Bufs3 b) {
-    __shared__ float rec[EF_COUNT][kElemTets];
-    __shared__ int vid[4][kElemTets];
+    __shared__ float4 rec[kElemTets][EW_COUNT];
+    __shared__ int4 vid[kElemTets];
     pdl_release3();
     pdl_wait3();
     const int t0 = blockIdx.x * kElemTets, Tp = m.Tp;
@@ -128,11 +144,11 @@ __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, 
             bx[n] = m.grad32[(3 * n) * Tp + t];
             by[n] = m.grad32[(3 * n + 1) * Tp + t];
             bz[n] = m.grad32[(3 * n + 2) * Tp + t];
-            vid[n][r] = v[n];
         }
+        vid[r] = make_int4(v[0], v[1], v[2], v[3]);
         const double C0d = b.C[v[0]];
         const float C0 = (float)C0d;
-        float dC[4], p[4], ux[4], uy[4], uz[4];
+        float dC[4], p[4], ux[4], uy[4], uz[4], om[4];
         float mus = 0.0f;
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
@@ -142,7 +158,7 @@ __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, 
             uy[n] = b.uy32[v[n]];
             uz[n] = b.uz32[v[n]];
             mus += b.mu32[v[n]];
-            rec[EF_OM0 + n][r] = 1.0f - omega32_3(C0 + dC[n], c);
+            om[n] = 1.0f - omega32_3(C0 + dC[n], c);
         }
         const float Cb = C0 + 0.25f * (dC[1] + dC[2] + dC[3]);
         const float ubx = 0.25f * (ux[0] + ux[1] + ux[2] + ux[3]);
@@ -160,15 +176,9 @@ __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, 
             gp[1] = fmaf(dp, by[n], gp[1]);
             gp[2] = fmaf(dp, bz[n], gp[2]);
             const float dx = ux[n] - ux[0], dy = uy[n] - uy[0], dz = uz[n] - uz[0];
-            rec[EF_DC1 + n - 1][r] = dC[n];
-            rec[EF_DP1 + n - 1][r] = dp;
-            rec[EF_DU1X + 3 * (n - 1)][r] = dx;
-            rec[EF_DU1X + 3 * (n - 1) + 1][r] = dy;
-            rec[EF_DU1X + 3 * (n - 1) + 2][r] = dz;
-            rec[EF_DSU1 + n - 1][r] = dx * (ux[n] + ux[0]) + dy * (uy[n] + uy[0]) + dz * (uz[n] + uz[0]);
-            rec[EF_B1X + 3 * (n - 1)][r] = bx[n];
-            rec[EF_B1X + 3 * (n - 1) + 1][r] = by[n];
-            rec[EF_B1X + 3 * (n - 1) + 2][r] = bz[n];
+            rec[r][EW_B1 + n - 1] = make_float4(bx[n], by[n], bz[n], dC[n]);
+            rec[r][EW_D1 + n - 1] =
+                make_float4(dx, dy, dz, 1.5f * (dx * (ux[n] + ux[0]) + dy * (uy[n] + uy[0]) + dz * (uz[n] + uz[0])));
         }
         float lapmu;
         if (c.lapmu_nodal) {
@@ -184,34 +194,17 @@ __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, 
             }
             lapmu = -1.5f * flux;
         }
-        const float drho = c.drho_f;
-        const float rhob = c.rho_v_f + Cb * drho;
-        const float f = 3.0f * Cb / rhob;
-        const float gr[3] = {drho * gC[0], drho * gC[1], drho * gC[2]};
-        const float vh[3] = {gC[0] - f * (gp[0] - mub * gC[0]), gC[1] - f * (gp[1] - mub * gC[1]),
-                             gC[2] - f * (gp[2] - mub * gC[2])};
-        rec[EF_V][r] = m.vol32[t];
-        rec[EF_C0][r] = C0;
-        rec[EF_U0X][r] = ux[0];
-        rec[EF_U0Y][r] = uy[0];
-        rec[EF_U0Z][r] = uz[0];
-        rec[EF_UBX][r] = ubx;
-        rec[EF_UBY][r] = uby;
-        rec[EF_UBZ][r] = ubz;
-        rec[EF_MUB][r] = mub;
-        rec[EF_UUB][r] = 1.5f * (ubx * ubx + uby * uby + ubz * ubz);
-        rec[EF_UU0][r] = 1.5f * (ux[0] * ux[0] + uy[0] * uy[0] + uz[0] * uz[0]);
-        rec[EF_RHO0][r] = c.rho_v_f + C0 * drho;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            rec[EF_GRX + a][r] = gr[a];
-            rec[EF_GCX + a][r] = gC[a];
-            rec[EF_VHX + a][r] = vh[a];
-        }
-        rec[EF_UGR][r] = ubx * gr[0] + uby * gr[1] + ubz * gr[2];
-        rec[EF_UGC][r] = ubx * gC[0] + uby * gC[1] + ubz * gC[2];
-        rec[EF_UVH][r] = ubx * vh[0] + uby * vh[1] + ubz * vh[2];
-        rec[EF_MLAP][r] = c.mobility_f * lapmu;
+        const float rhob = c.rho_v_f + Cb * c.drho_f;
+        const float f = 3.0f * Cb / rhob, f1 = 1.0f + f * mub;      // v_h = f1 grad C - f grad p
+        const float u_gC = ubx * gC[0] + uby * gC[1] + ubz * gC[2];
+        const float u_gp = ubx * gp[0] + uby * gp[1] + ubz * gp[2];
+        rec[r][EW_S] = make_float4(m.vol32[t], C0, (1.0f / 3.0f) * (c.rho_v_f + C0 * c.drho_f), mub);
+        rec[r][EW_U0] = make_float4(ux[0], uy[0], uz[0], 1.5f * (ux[0] * ux[0] + uy[0] * uy[0] + uz[0] * uz[0]));
+        rec[r][EW_UB] = make_float4(ubx, uby, ubz, 1.5f * (ubx * ubx + uby * uby + ubz * ubz));
+        rec[r][EW_GC] = make_float4(gC[0], gC[1], gC[2], u_gC);
+        rec[r][EW_GP] = make_float4(gp[0], gp[1], gp[2], f);
+        rec[r][EW_OM] = make_float4(om[0], om[1], om[2], om[3]);
+        rec[r][EW_H] = make_float4(f1, c.mobility_f * lapmu - (f1 * u_gC - f * u_gp), 0.0f, 0.0f);
     }
     __syncthreads();
     // ---- phase B: directions, five lanes per tetrahedron
@@ -220,55 +213,59 @@ __global__ void __launch_bounds__(kCoopBlock) k3_element32(DevMesh3 m, Phys3 c, 
     const int g = (threadIdx.x >> 5) * kGroupsPerWarp + grp;          // 0..23
     constexpr int kGroups = kGroupsPerWarp * (kCoopBlock / 32);
     const Dir4 d = lane_dirs(cl);
-    const float drho = c.drho_f;
+    const float drho3 = (1.0f / 3.0f) * c.drho_f;
     for (int r = g; r < nt; r += kGroups) {
-        const float V = rec[EF_V][r], C0 = rec[EF_C0][r];
-        const float u0x = rec[EF_U0X][r], u0y = rec[EF_U0Y][r], u0z = rec[EF_U0Z][r];
-        const float ubx = rec[EF_UBX][r], uby = rec[EF_UBY][r], ubz = rec[EF_UBZ][r];
-        const float mub = rec[EF_MUB][r], uub15 = rec[EF_UUB][r], uu0 = rec[EF_UU0][r], rho0 = rec[EF_RHO0][r];
-        const float u_gr = rec[EF_UGR][r], u_gC = rec[EF_UGC][r], u_vh = rec[EF_UVH][r], Mlap = rec[EF_MLAP][r];
         float4 gk[4], hk[4];
+        const int4 v = vid[r];
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-            const float4* row = reinterpret_cast<const float4*>(b.dpsi + (size_t)vid[n][r] * kRow);
+            const int vn = n == 0 ? v.x : n == 1 ? v.y : n == 2 ? v.z : v.w;
+            const float4* row = reinterpret_cast<const float4*>(b.dpsi + (size_t)vn * kRow);
             gk[n] = row[cl];
             hk[n] = row[5 + cl];
         }
-        float4 og = make_float4(0.0f, 0.0f, 0.0f, 0.0f), oh = og;
+        const float4 S = rec[r][EW_S], U0 = rec[r][EW_U0], UB = rec[r][EW_UB], GC = rec[r][EW_GC], GP = rec[r][EW_GP];
+        const float4 OM = rec[r][EW_OM], H = rec[r][EW_H];
+        const float V = S.x, C0 = S.y, rho3 = S.z, mub = S.w;
+        // sums over the vertices: (e.b) dG / w, (e.b) dC dG / w, (e.b) of the damped deviations' differences
+        float P1[4], P2[4], Qg[4], Qh[4], e0[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            e0[j] = d.ex[j] * U0.x + d.ey[j] * U0.y + d.ez[j] * U0.z;
+            set_comp(gk[0], j, OM.x * comp(gk[0], j));
+            set_comp(hk[0], j, OM.x * comp(hk[0], j));
+            P1[j] = P2[j] = Qg[j] = Qh[j] = 0.0f;
+        }
+#pragma unroll
+        for (int n = 1; n < 4; ++n) {
+            const float4 B = rec[r][EW_B1 + n - 1], D = rec[r][EW_D1 + n - 1];
+            const float om = comp(OM, n);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float ex = d.ex[j], ey = d.ey[j], ez = d.ez[j];
+                const float edu = ex * D.x + ey * D.y + ez * D.z;
+                // dG / w = 3 e.du + 4.5 (e.du) e.(u_n + u_0) - 1.5 (u_n^2 - u_0^2)
+                const float dG = fmaf(edu, fmaf(4.5f, edu, fmaf(9.0f, e0[j], 3.0f)), -D.w);
+                const float eb = ex * B.x + ey * B.y + ez * B.z;
+                P1[j] = fmaf(eb, dG, P1[j]);
+                P2[j] = fmaf(eb * B.w, dG, P2[j]);
+                Qg[j] = fmaf(eb, fmaf(om, comp(gk[n], j), -comp(gk[0], j)), Qg[j]);
+                Qh[j] = fmaf(eb, fmaf(om, comp(hk[n], j), -comp(hk[0], j)), Qh[j]);
+            }
+        }
+        float4 og, oh;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float ex = d.ex[j], ey = d.ey[j], ez = d.ez[j], w = d.w[j];
-            const float eu = ex * ubx + ey * uby + ez * ubz;
-            const float G = w * (1.0f + 3.0f * eu + 4.5f * eu * eu - uub15);
-            const float egr = ex * rec[EF_GRX][r] + ey * rec[EF_GRY][r] + ez * rec[EF_GRZ][r];
-            const float egc = ex * rec[EF_GCX][r] + ey * rec[EF_GCY][r] + ez * rec[EF_GCZ][r];
-            const float evh = ex * rec[EF_VHX][r] + ey * rec[EF_VHY][r] + ez * rec[EF_VHZ][r];
-            const float phig = (1.0f / 3.0f) * (G - w) * (egr - u_gr) + mub * G * (egc - u_gC);
-            const float phih = ((evh - u_vh) + Mlap) * G;
-            const float e0 = ex * u0x + ey * u0y + ez * u0z;
-            const float G0 = w * (1.0f + 3.0f * e0 + 4.5f * e0 * e0 - uu0);
-            const float om0 = rec[EF_OM0][r];
-            const float g0 = om0 * comp(gk[0], j), h0 = om0 * comp(hk[0], j);
-            float dg = 0.0f, dh = 0.0f;
-#pragma unroll
-            for (int n = 1; n < 4; ++n) {
-                const float dx = rec[EF_DU1X + 3 * (n - 1)][r], dy = rec[EF_DU1X + 3 * (n - 1) + 1][r],
-                            dz = rec[EF_DU1X + 3 * (n - 1) + 2][r];
-                const float edu = ex * dx + ey * dy + ez * dz;
-                const float esu = edu + 2.0f * e0;                    // e.(u_n + u_0)
-                const float dG = w * (3.0f * edu + 4.5f * edu * esu - 1.5f * rec[EF_DSU1 + n - 1][r]);
-                const float dCn = rec[EF_DC1 + n - 1][r];
-                // differences of the equilibria and of the post-collision deviations to vertex 0
-                const float dhe = (G0 + dG) * dCn + C0 * dG;
-                const float dge = w * rec[EF_DP1 + n - 1][r] + (1.0f / 3.0f) * (drho * dCn * (G0 + dG - w) + rho0 * dG);
-                const float omn = rec[EF_OM0 + n][r];
-                const float dgd = omn * comp(gk[n], j) - g0;
-                const float dhd = omn * comp(hk[n], j) - h0;
-                const float eb = ex * rec[EF_B1X + 3 * (n - 1)][r] + ey * rec[EF_B1X + 3 * (n - 1) + 1][r] +
-                                 ez * rec[EF_B1X + 3 * (n - 1) + 2][r];
-                dg = fmaf(dge + dgd, eb, dg);
-                dh = fmaf(dhe + dhd, eb, dh);
-            }
+            const float eu = ex * UB.x + ey * UB.y + ez * UB.z;
+            const float Gw = w * fmaf(eu, fmaf(4.5f, eu, 3.0f), -UB.w), G = w + Gw;      // Gamma - w, Gamma
+            const float egc = ex * GC.x + ey * GC.y + ez * GC.z;
+            const float egp = ex * GP.x + ey * GP.y + ez * GP.z;
+            const float phig = (egc - GC.w) * fmaf(drho3, Gw, mub * G);
+            const float phih = (fmaf(H.x, egc, -GP.w * egp) + H.y) * G;
+            const float s0 = fmaf(e0[j], fmaf(4.5f, e0[j], 3.0f), -U0.w);                // Gamma_0 / w - 1
+            const float dg = fmaf(w, egp + fmaf(drho3, fmaf(s0, egc, P2[j]), rho3 * P1[j]), Qg[j]);
+            const float dh = fmaf(w, fmaf(s0, egc, egc) + fmaf(C0, P1[j], P2[j]), Qh[j]);
             // the padding direction has w = 0 and e = 0: its residual is 0
             set_comp(og, j, V * (phig - dg));
             set_comp(oh, j, V * (phih - dh));
