@@ -308,8 +308,9 @@ def fp32_step_bytes(solve_launches):
     """Minimum bytes per node-update of the FP32 form's launches:
     distributions read and written (2 x 18 x 4), right-hand side written and
     read (2 x 18 x 4), per solve launch an iterate, the right-hand side and
-    the new iterate (3 x 18 x 4; the update's: increment and deviations in,
-    deviations out), about 200 B of nodal and element fields."""
+    the new iterate (3 x 18 x 4; the first reads no iterate, the last reads
+    and writes the deviations instead of an iterate), about 200 B of nodal and
+    element fields."""
     return 2 * 18 * 4 + 2 * 18 * 4 + solve_launches * 3 * 18 * 4 + 200
 
 
@@ -687,13 +688,13 @@ def run_gpu(args):
     if rank == 0:
         nnz = r32["info"]["nnz"]
         # the solve phase of the FP32-deviation step: blocked launches (several
-        # steps of the 18 right-hand sides each), then the field update.
-        # Algorithmic bytes of a blocked launch: x in, b, x out (3 x 18 floats
-        # per node), the mass row (column index + FP32 value per entry), the
-        # inverse lumped mass; of the update: the increment and the
-        # deviations in, the deviations out, the fields in and out
+        # steps of the 18 right-hand sides each), the last of which also
+        # updates fields and deviations.  Algorithmic bytes of a launch: 18
+        # floats per node three times (b, x out; b, x in, x out; b, x in and
+        # deviations in and out), the mass row (FP32 value and 16-bit local
+        # index per entry), the inverse lumped mass; once the fields in and out
         n_launch = r32["solve_launches"]
-        alg_bytes = (n_launch - 1) * (N * (3 * 18 * 4 + 4) + nnz * (4 + 4)) + N * (3 * 18 * 4 + 2 * 20)
+        alg_bytes = n_launch * (N * (3 * 18 * 4 + 4) + nnz * (4 + 2)) + N * 2 * 20
         hbm_peak, peak_src = peaks()
         solve_ms = r32["phase_ms"]["solve_ms"]
         achieved = alg_bytes / (solve_ms * 1e-3) / 1e9
@@ -744,7 +745,7 @@ def run_gpu(args):
                               "frac_of_nominal_8TBps": s32["value"] * step_bytes / 1e9 / nominal},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": recorded_traffic("solve_phase"),
-                         "kernel": "solve phase: k_block32 launches of the FP32 solve, then k_update32",
+                         "kernel": "solve phase: k_block32 launches of the FP32 solve, the last with the field update",
                          "source_hash": source_hash(),
                          "alg_bytes": alg_bytes, "phase_ms": solve_ms,
                          "peak_source": peak_src, "frac_of_nominal_8TBps": achieved / nominal},

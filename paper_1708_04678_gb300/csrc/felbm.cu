@@ -8,10 +8,17 @@
 //    double [6][Tp], edge neighbours int [3][Tp] (structure of arrays);
 //  * element residual R: double [T][18] (array of structures: the node gather
 //    reads one triangle's 18 values as 9 contiguous 16-byte loads);
-//  * node-node pattern (CSR) with the consistent mass and Laplacian
-//    coefficients; node -> triangle and node -> wall-edge incidence (CSR).
-// Nodes are in reverse Cuthill-McKee order and triangles sorted by their
-// lowest node, so every gather reads a narrow window of the arrays.
+//  * the 18 FP32 values a node has in the solve (iterates, right-hand side)
+//    and in the deviations of FP32 storage: four planes float4 [Np] and one
+//    float2 [Np] (vec_at);
+//  * node-node pattern (CSR, and ELL with the diagonal first) with the
+//    consistent mass and Laplacian coefficients; node -> triangle and node ->
+//    wall-edge incidence (CSR);
+//  * per block of at most 512 nodes: the layers of nodes around it, its rows of
+//    the mass matrix with 16-bit block-local columns, its triangles.
+// Nodes are in compact tiles and blocks (recursive bisection), in reverse
+// Cuthill-McKee order inside a block, and triangles are sorted by their lowest
+// node, so every gather reads a narrow window of the arrays.
 //
 // One time step (Sec. II.C of arXiv:1708.04678, D2Q9 form) is six kinds of
 // kernels, captured once into a CUDA graph:
@@ -23,7 +30,9 @@
 //               barycentre (eq:G, eq:H, eq:intF) and the element residual
 //               A_T (Phi - e.grad psi_hat) of eq:galerkin_lbm
 //   k_rhs       node-centric gather of the streaming right-hand side with
-//               weak bounce-back on walls; first Chebyshev iterate
+//               weak bounce-back on walls; first Chebyshev iterate (FP32
+//               storage on large meshes: k_force32 does k_element's and k_rhs's
+//               work on one block, residuals in shared memory)
 //   k_block32   sweeps of the consistent-mass solve with the lumped-mass
 //               preconditioner, several per launch (FP32 corrections; k_sweep32
 //               and k_cheb32 one at a time, k_cheb in FP64); the last adds the
