@@ -104,11 +104,12 @@ __device__ __forceinline__ Dir4 lane_dirs(int c) {
 // The equilibrium part of e.grad psi_hat is linear in dC_n, dp_n and
 // dG_n = Gamma_n - Gamma_0, so per vertex only sum (e.b_n) dG_n and
 // sum (e.b_n) dC_n dG_n are formed; the rest is e.grad C and e.grad p, which
-// the forces need as well.  With the per-vertex differences of the equilibria
-// themselves and one 4-byte load per element quantity the kernel was bound by
-// instructions (66 % of the issue slots) and shared-memory wavefronts (41 % of
-// the L1's 68 %): 1,572,864 tetrahedra took 235 us, now 200 us.  95 registers
-// (5 blocks per SM); 80 and 72 spill: 215 and 292 us.
+// the forces need as well.  Bound by L1 wavefronts (78 % busy: a vertex row is
+// five 16-byte loads of a group, a 16-byte shared word of six groups up to four
+// wavefronts) and by instructions: 138 M for 1,572,864 tetrahedra in 200 us.  With
+// the differences of both equilibria formed at every vertex and one 4-byte load
+// per element quantity it was 188 M in 235 us.  95 registers (5 blocks per SM);
+// 80 and 72 spill: 215 and 292 us.
 constexpr int kElemTets = kCoopBlock;
 // Element quantities of one tetrahedron, 13 16-byte words (an odd number, so
 // that neither the threads' rows of phase A nor the groups' of phase B share
