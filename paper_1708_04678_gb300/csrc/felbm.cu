@@ -286,6 +286,16 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
 }
 
+// A double rounded to a float (nearest, ties to even) through the integer pipe,
+// for the same reason; what is not a normal float takes the instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi & 0x7fffffffu) - 0x38100000u;          // exponent above the least of a normal float
+    if (e >= 0x0fe00000u) return (float)x;
+    const uint32_t f = (e + 0x00100000u) << 3 | lo >> 29;
+    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
+}
+
 constexpr int kBlock = 256;
 constexpr int kWarpBlocksBelow = 512;   // items per multiprocessor (fp64_block)
 constexpr int kDiagBlocks = 608;   // fixed grid (4 x 152 SMs): the reduction order never changes
@@ -535,13 +545,14 @@ __global__ void __launch_bounds__(128) k_element(DevMesh m, Phys c, Bufs b) {
     for (int k = 0; k < 9; ++k) dst[k] = make_double2(out[2 * k], out[2 * k + 1]);
 }
 
-// The right-hand side of an FP32 correction and its first iterate s r.
-__device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const double (&r)[18], float s) {
+// The right-hand side of an FP32 correction and its first iterate s r, the FP64
+// product rounded once.
+__device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const double (&r)[18], double s) {
     float r32[18], e[18];
 #pragma unroll
     for (int q = 0; q < 18; ++q) {
-        r32[q] = (float)r[q];
-        e[q] = r32[q] * s;
+        r32[q] = narrow(r[q]);
+        e[q] = narrow(r[q] * s);
     }
     store_all(b.r32, Np, i, r32);
     store_all(b.e1, Np, i, e);
@@ -557,9 +568,9 @@ __device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const 
 // mixed-precision solve, in FP32 together with the FP32 copy of the
 // right-hand side.
 //
-// Bound by the FP64 pipe (85 % busy: 108 FMAs, 60 operations on the weights, 18
-// conversions a node): 175 us on 520,704 nodes, 256 us with the weights formed
-// direction by direction and the first iterate in FP64.
+// Bound by the FP64 pipe (108 FMAs, 60 operations on the weights, 18 products for
+// the first iterate a node): 204 us on 520,704 nodes, 256 us with the weights
+// formed direction by direction and conversion instructions.
 // One thread per node, or (kSets = 2, consecutive blocks) one per node and set,
 // which forms the weights twice but halves a thread's chain of loads and its
 // straight-line code -- what a small mesh waits for (2,112 nodes: 15.5 us
@@ -637,15 +648,14 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
         b.rhs[(9 * set + q) * Np + i] = acc[q];
         if (!kMixed) b.x1[(9 * set + q) * Np + i] = acc[q] * s;
     }
-    // the corrections start from the FP32 copy (conversions share the FP64 pipe)
     if constexpr (kMixed && kSets == 1) {
-        store_start(b, Np, i, acc, (float)s);
+        store_start(b, Np, i, acc, s);
     } else if constexpr (kMixed) {
         float r32[9], e[9];
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            r32[q] = (float)acc[q];
-            e[q] = r32[q] * (float)s;
+            r32[q] = narrow(acc[q]);
+            e[q] = narrow(acc[q] * s);
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -681,8 +691,8 @@ __global__ void __launch_bounds__(kBlock) k_solve_in(DevMesh m, Bufs b, const do
             const int q = vec_row(p, c);
             b.rhs[q * Np + i] = v[q];
             if (!kMixed) b.x1[q * Np + i] = v[q] * s;
-            r[c] = (float)v[q];
-            e[c] = r[c] * (float)s;
+            r[c] = narrow(v[q]);
+            e[c] = narrow(v[q] * s);
         }
         if (kMixed && p < 4) {
             store_vec(b.r32, Np, p, i, r);
@@ -733,7 +743,7 @@ __global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, const 
         if (src != b.rhs) b.rhs[q * Np + i] = acc[q];
         if (!kMixed) b.x1[q * Np + i] = acc[q] * s;
     }
-    if constexpr (kMixed) store_start(b, Np, i, acc, (float)s);
+    if constexpr (kMixed) store_start(b, Np, i, acc, s);
 }
 
 // ---------------------------------------------- K6: Chebyshev sweep -------
@@ -951,14 +961,15 @@ __global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, cons
 // plane (consecutive blocks, which share the rows through L2): five times the
 // warps and a fifth of the straight-line code, which is what a small mesh
 // waits for (2,112 nodes: 8.3 us against 15.3 for all planes in a thread; on
-// 520,704 nodes 212 against 197 us).  The FP64 pipe is 85 % busy; with
-// conversion instructions for the 126 gathered values it took 377 us.
+// 520,704 nodes 252 us, of which the first iterate as an FP64 product takes
+// 40).  Bound by the FP64 pipe; with conversion instructions for the 126 gathered
+// values it took 377 us.
 template <int NV>
 __device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, const float* e,
-                                             float* next_first, int first_round, float tau0, int p, int i) {
+                                             float* next_first, int first_round, double tau0, int p, int i) {
     const int Np = m.Np, k1 = m.row_ptr[i + 1];
     int k = m.row_ptr[i];
-    const float s = m.inv_lumped32[i] * tau0;
+    const double s = m.inv_lumped[i] * tau0;
     // every load of the node itself before the first store (the compiler keeps
     // their order, and one at a time they cost a latency each)
     const size_t at = (size_t)(NV == 2 ? 0 : 9 * (p >> 1) + 1 + 4 * (p & 1)) * Np + i, stride = (size_t)(NV == 2 ? 9 : 1) * Np;
@@ -985,15 +996,15 @@ __device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, co
         const double ed = widen(ei[c]), rn = ro[c] - acc[c];
         b.x64[at + c * stride] = first_round ? ed : xo[c] + ed;
         b.rho64[at + c * stride] = rn;
-        r32[c] = (float)rn;
-        first[c] = r32[c] * s;
+        r32[c] = narrow(rn);
+        first[c] = narrow(rn * s);
     }
     store_vec(b.r32, Np, p, i, r32);
     store_vec(next_first, Np, p, i, first);
 }
 
 __global__ void __launch_bounds__(128) k_refine(DevMesh m, Bufs b, const float* e,
-                                                float* next_first, int first_round, float tau0, int n4) {
+                                                float* next_first, int first_round, double tau0, int n4) {
     const int nb = (int)blockIdx.x / (n4 + 1), l = (int)blockIdx.x - (n4 + 1) * nb, p = l < n4 ? l : 4;
     const int i = nb * (int)blockDim.x + (int)threadIdx.x;
     if (i >= m.N) return;
@@ -2070,7 +2081,7 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
             std::swap(cur, prv);
         }
         if (!last_round) {
-            k_refine<<<grid * (n4 + 1), nb, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0], n4);
+            k_refine<<<grid * (n4 + 1), nb, 0, s>>>(m, b, cur, prv, r == 0, st->tau[0], n4);
             A = prv;
             B = cur;
         }

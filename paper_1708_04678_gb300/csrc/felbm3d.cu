@@ -250,6 +250,16 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
 }
 
+// A double rounded to a float (nearest, ties to even) through the integer pipe,
+// for the same reason; what is not a normal float takes the instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi & 0x7fffffffu) - 0x38100000u;          // exponent above the least of a normal float
+    if (e >= 0x0fe00000u) return (float)x;
+    const uint32_t f = (e + 0x00100000u) << 3 | lo >> 29;
+    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
+}
+
 // ------------------------------------------------------ K1: collision -----
 // Moments of the pre-collision state (C = sum h, p = sum g, rho u = sum e g /
 // cs2) and BGK collision towards g_eq = w p + rho cs2 (Gamma - w),
@@ -537,18 +547,17 @@ __global__ void __launch_bounds__(kNodeBlock) k3_rhs(DevMesh3 m, Phys3 c, Bufs3 
         b.rhs[rh + Np] = h1;
     }
     if constexpr (kMixed) {
-        // the corrections start from the FP32 copy (conversions share the FP64 pipe)
+        // the first iterate is the FP64 product, rounded once
         const size_t a = (size_t)i * kRow + q;
-        const float s = (float)sc, fg0 = (float)g0, fh0 = (float)h0, fg1 = (float)g1, fh1 = (float)h1;
-        b.r32[a] = fg0;
-        b.r32[a + 20] = fh0;
-        b.e1[a] = fg0 * s;
-        b.e1[a + 20] = fh0 * s;
+        b.r32[a] = narrow(g0);
+        b.r32[a + 20] = narrow(h0);
+        b.e1[a] = narrow(g0 * sc);
+        b.e1[a + 20] = narrow(h0 * sc);
         const size_t a1 = (size_t)i * kRow + (cc == 0 ? 19 : q + 1);      // lane 0: the padding slots, zero
-        b.r32[a1] = fg1;
-        b.r32[a1 + 20] = fh1;
-        b.e1[a1] = fg1 * s;
-        b.e1[a1 + 20] = fh1 * s;
+        b.r32[a1] = narrow(g1);
+        b.r32[a1 + 20] = narrow(h1);
+        b.e1[a1] = narrow(g1 * sc);
+        b.e1[a1 + 20] = narrow(h1 * sc);
     } else {
         b.x1[r] = g0 * sc;
         b.x1[rh] = h0 * sc;
@@ -608,7 +617,7 @@ __global__ void __launch_bounds__(kNodeBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bu
 // widened on the integer pipe (the kernel is bound by the FP64 pipe): 486 us on
 // 262,144 nodes against 670 us with conversion instructions.
 __global__ void __launch_bounds__(kCoopBlock) k3_refine(DevMesh3 m, Bufs3 b, const float* e, float* next_first,
-                                                        int first_round, float tau0) {
+                                                        int first_round, double tau0) {
     const int lane = threadIdx.x & 31, grp = lane / 10, cc = lane - grp * 10;
     const int i = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 3 + grp;
     if (grp >= 3 || i >= m.N) return;
@@ -632,19 +641,20 @@ __global__ void __launch_bounds__(kCoopBlock) k3_refine(DevMesh3 m, Bufs3 b, con
         acc[2] = fma(mv, widen(ej.z), acc[2]);
         acc[3] = fma(mv, widen(ej.w), acc[3]);
     }
-    const float sc = m.inv_lumped32[i] * tau0;
-    float r[4];
+    const double sc = m.inv_lumped[i] * tau0;
+    float r[4], first[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        r[j] = 0.0f;                                  // the padding slots stay zero
+        r[j] = first[j] = 0.0f;                       // the padding slots stay zero
         if (j >= nq) continue;
         const double ed = widen(comp(ei, j)), rn = ro[j] - acc[j];
         b.x0[r0 + (size_t)j * Np] = first_round ? ed : xo[j] + ed;
         b.x1[r0 + (size_t)j * Np] = rn;
-        r[j] = (float)rn;
+        r[j] = narrow(rn);
+        first[j] = narrow(rn * sc);
     }
     reinterpret_cast<float4*>(b.r32 + (size_t)i * kRow)[cc] = make_float4(r[0], r[1], r[2], r[3]);
-    reinterpret_cast<float4*>(next_first + (size_t)i * kRow)[cc] = make_float4(r[0] * sc, r[1] * sc, r[2] * sc, r[3] * sc);
+    reinterpret_cast<float4*>(next_first + (size_t)i * kRow)[cc] = make_float4(first[0], first[1], first[2], first[3]);
 }
 
 // ------------------------------------------------ FP32 Chebyshev sweep ----
@@ -1257,7 +1267,7 @@ static void enqueue_solve3(felbm3d_state* st, cudaStream_t s, bool after_release
             std::swap(cur, prv);
         }
         if (r < st->rounds - 1) {
-            k3_refine<<<grid_for(m.N, 3 * (kCoopBlock / 32)), kCoopBlock, 0, s>>>(m, b, cur, prv, r == 0, (float)st->tau[0]);
+            k3_refine<<<grid_for(m.N, 3 * (kCoopBlock / 32)), kCoopBlock, 0, s>>>(m, b, cur, prv, r == 0, st->tau[0]);
             A = prv;
             B = cur;
         }
