@@ -305,9 +305,12 @@ int felbm_sweep_parts(felbm_state* state, int32_t parts);
  * advances several sweeps per launch.  Same arithmetic per row in the same
  * order: the trajectory does not depend on it.  FELBM_ERR_UNSUPPORTED if the
  * mesh has no ELL copy, rows of more than 12 entries, or a node tile that
- * references more than 504 nodes outside it (then 0 is used).  The step graph
- * is rebuilt at the next felbm_step.  Default: 1 where it is supported;
- * felbm_autotune picks one by timing. */
+ * references more than 504 nodes outside it (then 0 is used).  On a mesh whose
+ * node order leaves no room for a layer of nodes around some block, 1 is
+ * accepted and the sweeps stay gathered.  The step graph is rebuilt at the next
+ * felbm_step.  Default: by the mesh and the number of sweeps the form that
+ * measured faster, for felbm_mass_solve of up to 14 rows blocked where it is
+ * supported; felbm_autotune picks one by timing. */
 int felbm_sweep_tiled(felbm_state* state, int32_t on);
 
 typedef struct felbm_tune_result {

@@ -1557,7 +1557,7 @@ struct felbm_state {
     bool dev32 = false;   // FELBM_FP32_DEV storage
     bool use_pdl = true;  // programmatic dependent launch between solve sweeps
     int sweep_parts = 2;  // threads per node of the FP32 store sweeps (1, 2, 3, 6)
-    bool sweep_tiled = false;  // the solve runs several steps of a node block per launch (k_block32)
+    int sweep_tiled = -1;      // several steps of a node block per launch (k_block32): 1, never: 0, where faster: -1
     bool check = false;        // felbm_solver_check: residual of every solve before its last step
     double check_tol = 0.0;
     int n_sm = 1;              // multiprocessors of the device
@@ -1937,8 +1937,42 @@ static void launch_first(felbm_state* st, const DevMesh& m, const Bufs& b, cudaS
     }
 }
 
-// Whether the solve on m runs blocked.
-static bool blocked(const felbm_state* st, const DevMesh& m) { return st->sweep_tiled && m.blk_steps > 0; }
+// One wave of thread blocks, two to a multiprocessor, at least four fifths full.
+static bool full_wave(int n_blocks, int n_sm) { return n_blocks <= 2 * n_sm && 5 * n_blocks >= 8 * n_sm; }
+
+// Where the blocked solve of all rows is the faster form (GB300, solve phase of
+// an FP32 step of 10 steps, blocked against one launch per step; rows of 7
+// unless stated).
+//  * Up to kL2Nodes nodes the three vectors of a step (216 bytes a node) stay in
+//    L2 and a step per launch costs 48 ps a node, beyond it 56 to 70.  There the
+//    blocked form wins: 168 against 205 us on 405,900 nodes, 670 against 1,004
+//    on 2,082,816, and with two steps a launch 889 against 1,018.
+//  * With all planes in a thread block and the vectors in L2 it wins in one full
+//    wave (80,400 nodes in 256 blocks: 44 against 45; 128,000: 42 against 55) and
+//    ties where blocks are nearly full (261,726 nodes, 512 of 511: 101 against
+//    103).  Smaller blocks compute too many rows of their layers and a partial
+//    wave leaves multiprocessors idle: 131,584 nodes in 512 blocks of 257: 74
+//    against 61; a batch of 145,852 nodes in 392 blocks: 77 against 63.
+//  * With a plane per thread block it wins or ties: 19 against 31 on 20,200
+//    nodes, 35 against 34 on 65,341.  Rows of more than 9 entries leave one
+//    thread block to a multiprocessor: 33 against 35 on 26,180 nodes (64
+//    blocks), 52 against 37 on 43,380 (128 blocks), 175 against 150 on 235,620.
+//  * It needs steps to share a load: one step a solve takes 60 against 30 us on
+//    525,312 nodes, nine launches of one step (one layer) 48 against 35 on 36,120.
+constexpr int kL2Nodes = 340000;
+static bool blocked_is_faster(const felbm_state* st, const DevMesh& m) {
+    const bool in_l2 = m.N <= kL2Nodes;
+    if (st->sweeps < 3 || m.blk_steps < (in_l2 ? 3 : 2)) return false;
+    if (!in_l2) return true;
+    if (m.n_blocks < kSplitPlanesBelow * st->n_sm) return m.ell_w <= 9 || kPlanes * m.n_blocks <= 3 * st->n_sm;
+    return m.ell_w <= 9 && (full_wave(m.n_blocks, st->n_sm) || m.N >= 480 * m.n_blocks);
+}
+
+// Whether the solve of all rows on m runs blocked.
+static bool blocked(const felbm_state* st, const DevMesh& m) {
+    if (m.blk_steps == 0 || st->mode == FELBM_SOLVER_FP64) return false;
+    return st->sweep_tiled < 0 ? blocked_is_faster(st, m) : st->sweep_tiled != 0;
+}
 
 static bool first_from_rhs(const felbm_state* st, const DevMesh& m);
 
@@ -2003,12 +2037,12 @@ static void launch_mu(const DevMesh& m, const Phys& c, const Bufs& b, unsigned g
 // already written, unless from_rhs).  into_psi: add the increment to psi (time step); else
 // leave the solution in x1/x0 (FP64 mode, returned) or x64 (mixed mode).
 // b: the buffers the solve reads and writes (the state's own, or another set of
-// scratch buffers with the same layout).  n4: planes in use (k_block32; blocked
+// scratch buffers with the same layout).  tiled: blocked.  n4: planes in use (k_block32; blocked
 // solves only).  last: where given (blocked, not into_psi), the last correction
 // is not added to x64 but returned through it.
 static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs& b, cudaStream_t s,
-                                   bool into_psi, bool after_release = false, bool from_rhs = false, int n4 = 4,
-                                   const float** last = nullptr) {
+                                   bool into_psi, bool tiled, bool after_release = false, bool from_rhs = false,
+                                   int n4 = 4, const float** last = nullptr) {
     const int nb = fp64_block(st, m.N, 128);
     const unsigned grid = grid_for(m.N, nb);
     if (st->mode == FELBM_SOLVER_FP64) {
@@ -2029,7 +2063,7 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
         float* cur = A;
         float* prv = B;
         const bool last_round = r == st->rounds - 1;
-        if (blocked(st, m)) {
+        if (tiled) {
             bool pdl = r == 0 && after_release;
             int k = 1;
             if (last_round && st->check) {
@@ -2055,7 +2089,7 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
                 launch_k(st->use_pdl, into_psi ? k_add64<true> : k_add64<false>, dim3(grid), dim3(nb), 0, s, m, b,
                          (const float*)cur, have_x64);
         }
-        for (int k = 1; k < st->sweeps && !blocked(st, m); ++k) {
+        for (int k = 1; k < st->sweeps && !tiled; ++k) {
             const float tau = (float)st->tau[k];
             const bool last = last_round && k == st->sweeps - 1;
             // the previous launch is a sweep of this round, or a kernel that released its dependents
@@ -2086,19 +2120,21 @@ static const double* enqueue_solve(felbm_state* st, const DevMesh& m, const Bufs
 }
 
 // X = M11^{-1} B for rows [0, k) (device, caller order), with scratch b.  A
-// blocked solve takes only the planes that hold those rows: 5 of 18 rows on
-// 80,000 nodes take 168 us instead of 378.
+// blocked solve takes only the planes that hold those rows (5 of 18 rows on
+// 80,000 nodes take 168 us instead of 378), so it is the default for them.
 static void enqueue_mass_solve(felbm_state* st, const Bufs& b, const double* B, double* X, int k, cudaStream_t s) {
     const DevMesh& m = st->dm;
     const unsigned grid = grid_for(m.N, kBlock);
-    const bool part = blocked(st, m) && !st->check;   // the checked residual covers all rows
-    const int n4 = !part ? 4 : (k <= 1 ? 0 : k <= 5 ? 1 : k <= 10 ? 2 : k <= 14 ? 3 : 4);
+    const int planes = st->check ? 4 : k <= 1 ? 0 : k <= 5 ? 1 : k <= 10 ? 2 : k <= 14 ? 3 : 4;   // the checked residual covers all rows
+    const bool some = planes < 4 && st->sweep_tiled < 0 && m.blk_steps > 0 && st->mode != FELBM_SOLVER_FP64;
+    const bool tiled = some || blocked(st, m), part = tiled && !st->check;
+    const int n4 = part ? planes : 4;
     if (st->mode == FELBM_SOLVER_FP64)
         k_solve_in<false><<<grid, kBlock, 0, s>>>(m, b, B, k, n4, st->inv_theta);
     else
         k_solve_in<true><<<grid, kBlock, 0, s>>>(m, b, B, k, n4, st->tau[0]);
     const float* last = nullptr;
-    const double* x = enqueue_solve(st, m, b, s, false, false, false, n4, part ? &last : nullptr);
+    const double* x = enqueue_solve(st, m, b, s, false, tiled, false, false, n4, part ? &last : nullptr);
     k_solve_out<<<grid, kBlock, 0, s>>>(m, x, last, X, k, !last || st->rounds > 1);
 }
 
@@ -2202,7 +2238,7 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
                         launch_k(chain, k_rhs32<0, true>, gn, bn, 0, s, mt, st->phys, b, tau0);
             }
             mark(5);
-            enqueue_solve(st, mt, st->buf, s, true, chain, from_rhs);
+            enqueue_solve(st, mt, st->buf, s, true, blocked(st, mt), chain, from_rhs);
         } else {
             mark(2);
             mark(3);
@@ -2233,7 +2269,7 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
     else
         nb == 32 ? rhs(k_rhs<true, 2>, 2, st->tau[0]) : rhs(k_rhs<true, 1>, 1, st->tau[0]);
     mark(5);
-    enqueue_solve(st, st->dm, st->buf, s, true);
+    enqueue_solve(st, m, st->buf, s, true, blocked(st, m));
     mark(6);
 }
 
@@ -2420,7 +2456,6 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
             delete st;
             return FELBM_ERR_BAD_MESH;
         }
-        st->sweep_tiled = st->mode != FELBM_SOLVER_FP64;
     }
     auto pad_tri = [&](const std::vector<int32_t>& src, int rows) {
         std::vector<int32_t> outv((size_t)rows * st->dm.Tp, 0);
@@ -3229,7 +3264,7 @@ int felbm_autotune(felbm_state* st, int32_t trials, felbm_tune_result* out) {
     //    and where the iterate comes from (gathered, or staged per node tile)
     const int parts_c[4] = {1, 2, 3, 6};
     int best_parts = st->sweep_parts;
-    bool best_tiled = st->sweep_tiled;
+    int best_tiled = st->sweep_tiled;
     float best = 1e30f;
     if (st->mode != FELBM_SOLVER_FP64 && st->dm.ell_w > 0) {
         rc = set_schedule(st, 0);
@@ -3237,7 +3272,7 @@ int felbm_autotune(felbm_state* st, int32_t trials, felbm_tune_result* out) {
             if (tiled && st->dm.blk_steps == 0) break;
             for (int k = 0; k < 4 && rc == FELBM_OK; ++k) {
                 st->sweep_parts = parts_c[k];
-                st->sweep_tiled = tiled != 0;
+                st->sweep_tiled = tiled;
                 if (tiled && parts_c[k] != 3) continue;   // the blocked solve has one form
                 drop_graph(st);
                 float ms = 0.0f;
@@ -3246,7 +3281,7 @@ int felbm_autotune(felbm_state* st, int32_t trials, felbm_tune_result* out) {
                 if (ms < best) {
                     best = ms;
                     best_parts = parts_c[k];
-                    best_tiled = tiled != 0;
+                    best_tiled = tiled;
                 }
                 rc = checkpoint_copy(st, nullptr, save, false);
             }
@@ -3256,7 +3291,7 @@ int felbm_autotune(felbm_state* st, int32_t trials, felbm_tune_result* out) {
     st->sweep_tiled = best_tiled;
     drop_graph(st);
     out->sweep_parts = best_parts;
-    out->sweep_tiled = best_tiled ? 1 : 0;
+    out->sweep_tiled = blocked(st, st->dm) ? 1 : 0;
     // 2. batch schedule: CTA per member up to a node threshold (FP32_DEV batches)
     int32_t best_t = 0;
     if (rc == FELBM_OK && st->dev32 && h.G > 1) {
@@ -3419,7 +3454,7 @@ int felbm_adjoint_step(felbm_state* st) {
         k_cheb_start<false><<<ng, nb, 0, s>>>(m, b, a.lam, st->inv_theta);
     else
         k_cheb_start<true><<<ng, nb, 0, s>>>(m, b, a.lam, st->tau[0]);
-    a.lamRHS = enqueue_solve(st, m, b, s, false);
+    a.lamRHS = enqueue_solve(st, m, b, s, false, blocked(st, m));
     k_adj_elem_a<<<tg, tb, 0, s>>>(m, st->phys, b, a);
     k_adj_elem_b<<<tg, tb, 0, s>>>(m, a);
     k_adj_node_d<<<ng, nb, 0, s>>>(m, st->phys, a);
