@@ -1937,8 +1937,12 @@ static void launch_first(felbm_state* st, const DevMesh& m, const Bufs& b, cudaS
     }
 }
 
-// One wave of thread blocks, two to a multiprocessor, at least four fifths full.
-static bool full_wave(int n_blocks, int n_sm) { return n_blocks <= 2 * n_sm && 5 * n_blocks >= 8 * n_sm; }
+// Thread blocks, two to a multiprocessor, in waves that are at least four fifths
+// full altogether.
+static bool full_waves(int n_blocks, int n_sm) {
+    const int slots = 2 * n_sm, waves = (n_blocks + slots - 1) / slots;
+    return 5LL * n_blocks >= 4LL * waves * slots;
+}
 
 // Where the blocked solve of all rows is the faster form (GB300, solve phase of
 // an FP32 step of 10 steps, blocked against one launch per step; rows of 7
@@ -1949,10 +1953,12 @@ static bool full_wave(int n_blocks, int n_sm) { return n_blocks <= 2 * n_sm && 5
 //    on 2,082,816, and with two steps a launch 889 against 1,018.
 //  * With all planes in a thread block and the vectors in L2 it wins in one full
 //    wave (80,400 nodes in 256 blocks: 44 against 45; 128,000: 42 against 55) and
-//    ties where blocks are nearly full (261,726 nodes, 512 of 511: 101 against
-//    103).  Smaller blocks compute too many rows of their layers and a partial
-//    wave leaves multiprocessors idle: 131,584 nodes in 512 blocks of 257: 74
-//    against 61; a batch of 145,852 nodes in 392 blocks: 77 against 63.
+//    wins or ties where blocks are nearly full too (rows of 9, step: 576 blocks of
+//    512, 230 against 254; 261,726 nodes, 512 of 511: 101 against 103).  Smaller
+//    blocks compute too many rows of their layers and a partial wave leaves
+//    multiprocessors idle: 131,584 nodes in 512 blocks of 257: 74 against 61; a
+//    batch of 145,852 nodes in 392 blocks: 77 against 63; rows of 9, 320 blocks
+//    of 512, step: 176 against 152.
 //  * With a plane per thread block it wins or ties: 19 against 31 on 20,200
 //    nodes, 35 against 34 on 65,341.  Rows of more than 9 entries leave one
 //    thread block to a multiprocessor: 33 against 35 on 26,180 nodes (64
@@ -1965,7 +1971,7 @@ static bool blocked_is_faster(const felbm_state* st, const DevMesh& m) {
     if (st->sweeps < 3 || m.blk_steps < (in_l2 ? 3 : 2)) return false;
     if (!in_l2) return true;
     if (m.n_blocks < kSplitPlanesBelow * st->n_sm) return m.ell_w <= 9 || kPlanes * m.n_blocks <= 3 * st->n_sm;
-    return m.ell_w <= 9 && (full_wave(m.n_blocks, st->n_sm) || m.N >= 480 * m.n_blocks);
+    return m.ell_w <= 9 && full_waves(m.n_blocks, st->n_sm) && (m.n_blocks <= 2 * st->n_sm || m.N >= 480 * m.n_blocks);
 }
 
 // Whether the solve of all rows on m runs blocked.

@@ -26,6 +26,13 @@ def _batch():
                     for k, nx in enumerate(np.linspace(44, 88, 64).astype(int))])
 
 
+def _periodic_batch():
+    """20 periodic droplets of 16 blocks of 512 nodes: 320 blocks in two waves, the
+    second nearly empty."""
+    ws = [I.small_free_droplet(n=64, R=12.0, seed=50 + k) for k in range(20)]
+    return {"meshes": [w["mesh"] for w in ws], "C0": np.concatenate([w["C0"] for w in ws]), "phys": ws[0]["phys"]}
+
+
 # workload, node order, solver_iters, launches of the solve phase of one step
 CASES = {
     "a plane per thread block": (lambda: I.small_sessile(nx=64, ny=32, R=12.0), None, 0, 3),       # 2 + field update
@@ -33,6 +40,7 @@ CASES = {
     "full blocks": (lambda: I.small_sessile(nx=723, ny=361, R=90.0), None, 0, 3),
     "beyond L2": (lambda: I.small_sessile(nx=1024, ny=512, R=100.0), None, 0, 2),
     "partial waves": (_batch, None, 0, 9),
+    "partial waves of full blocks": (_periodic_batch, None, 0, 9),
     "small blocks": (lambda: I.small_free_droplet(n=258, R=50.0), None, 0, 9),
     "one step": (lambda: I.small_sessile(nx=64, ny=32, R=12.0), None, 2, 1),
     "one layer": (lambda: I.small_sessile(nx=120, ny=300, R=40.0), "rcm", 0, 9),
