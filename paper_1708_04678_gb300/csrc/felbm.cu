@@ -2155,13 +2155,26 @@ static int solve_launches(const felbm_state* st) {
     return refines * (groups(st->sweeps - 1) + 1) + last + (update ? 0 : 1);
 }
 
-// FP32 states: residuals and their gather in one kernel (k_force32) from this
-// many blocks per multiprocessor on; below, 384 threads a block leave most of
-// the device idle (11,615 nodes: 45 us a step fused, 43 us not; the figures for
-// large meshes stand at the kernel).
-constexpr int kFuseForcesFrom = 1;
+// FP32 states: residuals and their gather in one kernel (k_force32) or in two.
+// One kernel needs the device full, with two thread blocks of 384 threads on a
+// multiprocessor, and few walls: the bounce-back of a wall node is a chain of
+// loads that two thread blocks hide worse than the separate gather's eight.
+// Step of one solve step, us, one kernel against two (GB300):
+//   no walls (rows of 9)  128 blocks 26.8 / 24.7, 160 35.1 / 33.2, 176 34.9 / 35.0, 256 49.5 / 57.5,
+//                         320 72.4 / 69.4, 448 92.4 / 90.8, 512 55.1 / 59.5, 688 140 / 135
+//   walls                 256 blocks, 8,000 x 15 cells (12 % of the nodes) 58.4 / 59.3; batches of 176 to
+//                         1,376 blocks (3 to 8 %) 41.4 / 35.7 to 193 / 181; 450,000 nodes with 0.7, 2 and
+//                         4 %: 165 / 163, 174 / 166, 189 / 173
+//   2,082,816 nodes (0.2 %) 627 / 652
+//   405,900 nodes (0.4 %) in blocks of 396, which fill two of three rounds of threads: 156 / 148
+// Hence: any walls in one full wave, below 1 % of the nodes in more full waves or
+// in one wave of at least 1.15 blocks to a multiprocessor.
 static bool fused_forces(const felbm_state* st, const DevMesh& m) {
-    return st->dev32 && m.max_blk_tri > 0 && m.n_blocks >= kFuseForcesFrom * st->n_sm;
+    if (!st->dev32 || m.max_blk_tri == 0) return false;
+    const int nb = m.n_blocks;
+    const bool one = nb <= 2 * st->n_sm, full = full_waves(nb, st->n_sm);
+    if (100LL * st->hm.E > st->hm.N) return one && full;
+    return full || (one && 20 * nb >= 23 * st->n_sm);
 }
 
 static int step_launches(const felbm_state* st) {
