@@ -2144,14 +2144,25 @@ static void enqueue_mass_solve(felbm_state* st, const Bufs& b, const double* B, 
     k_solve_out<<<grid, kBlock, 0, s>>>(m, x, last, X, k, !last || st->rounds > 1);
 }
 
-static int solve_launches(const felbm_state* st) {
+// The part of the mesh that the launches of a step cover: the members that have
+// no CTA of their own, a prefix of nodes, triangles and blocks (set_schedule).
+static DevMesh launched_part(const felbm_state* st) {
+    DevMesh m = st->dm;
+    m.N = st->tiled_N;
+    m.T = st->tiled_T;
+    m.n_blocks = st->tiled_blocks;
+    return m;
+}
+
+static int solve_launches(const felbm_state* st, const DevMesh& m) {
+    if (m.N == 0) return 0;
     if (st->mode == FELBM_SOLVER_FP64) return st->sweeps - 1;
     const int refines = st->rounds - 1;
-    if (!blocked(st, st->dm)) return st->rounds * (st->sweeps - 1) + refines;
-    const int most = st->dm.blk_steps;
+    if (!blocked(st, m)) return st->rounds * (st->sweeps - 1) + refines;
+    const int most = m.blk_steps;
     const auto groups = [&](int steps) { return (steps + most - 1) / most; };
     const int last = st->check ? groups(st->sweeps - 2) + 1 : groups(st->sweeps - 1);
-    const bool update = fused_update(st, st->dm, st->check ? st->sweeps - 1 : 1);
+    const bool update = fused_update(st, m, st->check ? st->sweeps - 1 : 1);
     return refines * (groups(st->sweeps - 1) + 1) + last + (update ? 0 : 1);
 }
 
@@ -2177,8 +2188,10 @@ static bool fused_forces(const felbm_state* st, const DevMesh& m) {
     return full || (one && 20 * nb >= 23 * st->n_sm);
 }
 
-static int step_launches(const felbm_state* st) {
-    return (st->dev32 ? (fused_forces(st, st->dm) ? 3 : 4) : 5) + solve_launches(st);
+static int step_launches(const felbm_state* st, const DevMesh& m) {
+    const int ctas = st->n_cta > 0 ? 1 : 0;
+    if (m.N == 0) return ctas;
+    return ctas + (st->dev32 ? (fused_forces(st, m) ? 3 : 4) : 5) + solve_launches(st, m);
 }
 
 int set_schedule(felbm_state* st, int32_t max_nodes);
@@ -2204,10 +2217,7 @@ static void enqueue_step(felbm_state* st, cudaStream_t s) {
             cudaEventRecord(st->ev_join, st->side_stream);
         }
         // the rest (a prefix of nodes and triangles): tiled kernels
-        DevMesh mt = m;
-        mt.N = st->tiled_N;
-        mt.T = st->tiled_T;
-        mt.n_blocks = st->tiled_blocks;
+        const DevMesh mt = launched_part(st);
         // collision is folded into the element, RHS and update kernels
         mark(1);
         if (mt.N > 0) {
@@ -2805,8 +2815,9 @@ int felbm_timing_get(felbm_state* st, felbm_step_timing* out) {
     out->rhs_ms = t[4];
     out->solve_ms = t[5];
     out->total_ms = t[0] + t[1] + t[2] + t[3] + t[4] + t[5];
-    out->solve_launches = solve_launches(st);
-    out->launches = step_launches(st);
+    const DevMesh m = launched_part(st);
+    out->solve_launches = solve_launches(st, m);
+    out->launches = step_launches(st, m);
     return FELBM_OK;
 }
 
