@@ -2504,10 +2504,39 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     std::vector<double> grad_p = pad_trid(h.grad, 6), area_p = pad_trid(h.area, 1);
     std::vector<float> grad32_p(grad_p.begin(), grad_p.end()), area32_p(area_p.begin(), area_p.end());
     std::vector<float> inc_bx32(h.inc_bx.begin(), h.inc_bx.end()), inc_by32(h.inc_by.begin(), h.inc_by.end());
+    // node -> triangle incidence (padding: the zero residual row T), and as indices
+    // into the block's triangle list (padding: past its end)
+    const int iw = st->dm.iell_w;
+    std::vector<int32_t> itri((size_t)std::max(iw, 1) * st->dm.Np, h.T);
+    std::vector<float> ibx(itri.size(), 0.0f), iby(itri.size(), 0.0f);
+    for (int32_t i = 0; i < h.N && iw > 0; ++i)
+        for (int32_t k = h.inc_ptr[i]; k < h.inc_ptr[i + 1]; ++k) {
+            const size_t at = (size_t)(k - h.inc_ptr[i]) * st->dm.Np + i;
+            itri[at] = h.inc_tri[k];
+            ibx[at] = inc_bx32[k];
+            iby[at] = inc_by32[k];
+        }
+    std::vector<uint16_t> iloc;
+    if (st->dm.max_blk_tri > 0) {
+        iloc.resize((size_t)iw * st->dm.Np);
+        parallel_for(nblk, 4, []() { return 0; }, [&](int32_t t, int&) {
+            const int32_t* l0 = h.blk_tri.data() + h.blk_tri_ptr[t];
+            const int32_t* l1 = h.blk_tri.data() + h.blk_tri_ptr[t + 1];
+            for (int32_t i = h.blk_ptr[t]; i < h.blk_ptr[t + 1]; ++i)
+                for (int k = 0; k < iw; ++k) {
+                    const size_t at = (size_t)k * st->dm.Np + i;
+                    iloc[at] = (uint16_t)(itri[at] < h.T ? std::lower_bound(l0, l1, itri[at]) - l0 : l1 - l0);
+                }
+        });
+    }
+    // The tables above are all made before the first copy and outlive the last: a
+    // copy from pageable memory may still read them when the call returns, so the
+    // stream is waited for on every way out.
     cudaStream_t s = st->stream;
     const DevMesh& d = st->dm;
     auto fail = [&](cudaError_t e, const char* what) {
         int r = cuda_fail(e, what);
+        cudaStreamSynchronize(s);
         delete st;
         return r;
     };
@@ -2556,48 +2585,24 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     UP(d.inc_by, h.inc_by);
     UP(d.inc_bx32, inc_bx32);
     UP(d.inc_by32, inc_by32);
-    {
-        const int iw = st->dm.iell_w;
-        const size_t Npi = st->dm.Np;
-        std::vector<int32_t> itri((size_t)std::max(iw, 1) * Npi, h.T);
-        std::vector<float> ibx((size_t)std::max(iw, 1) * Npi, 0.0f), iby(ibx.size(), 0.0f);
-        for (int32_t i = 0; i < h.N && iw > 0; ++i)
-            for (int32_t k = h.inc_ptr[i]; k < h.inc_ptr[i + 1]; ++k) {
-                const size_t at = (size_t)(k - h.inc_ptr[i]) * Npi + i;
-                itri[at] = h.inc_tri[k];
-                ibx[at] = inc_bx32[k];
-                iby[at] = inc_by32[k];
-            }
-        std::vector<uint16_t> iloc;
-        if (st->dm.max_blk_tri > 0) {
-            iloc.resize((size_t)iw * Npi);
-            parallel_for(nblk, 4, []() { return 0; }, [&](int32_t t, int&) {
-                const int32_t* l0 = h.blk_tri.data() + h.blk_tri_ptr[t];
-                const int32_t* l1 = h.blk_tri.data() + h.blk_tri_ptr[t + 1];
-                for (int32_t i = h.blk_ptr[t]; i < h.blk_ptr[t + 1]; ++i)
-                    for (int k = 0; k < iw; ++k) {
-                        const int32_t tri = itri[(size_t)k * Npi + i];
-                        iloc[(size_t)k * Npi + i] = (uint16_t)(tri < h.T ? std::lower_bound(l0, l1, tri) - l0 : l1 - l0);
-                    }
-            });
-            UP(d.blk_tri_ptr, h.blk_tri_ptr);
-            UP(d.blk_tri, h.blk_tri);
-            UP(d.iell_loc, iloc);
-            // (the limit holds for every state of the process: the largest any may ask for)
-            const int bytes = (int)force_smem_bytes(kForceTris);
-            const auto allow = [&](auto kern) {
-                if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-            };
-            allow(k_force32<6>);
-            allow(k_force32<8>);
-            allow(k_force32<12>);
-        }
-        UP(d.iell_tri, itri);
-        UP(d.iell_bx32, ibx);
-        UP(d.iell_by32, iby);
-        if (dev32 && e == cudaSuccess) e = cudaMemsetAsync(st->buf.R32 + (size_t)18 * h.T, 0, 18 * sizeof(float), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(st->buf.diag_done, 0, sizeof(unsigned), s);
+    UP(d.iell_tri, itri);
+    UP(d.iell_bx32, ibx);
+    UP(d.iell_by32, iby);
+    if (st->dm.max_blk_tri > 0) {
+        UP(d.blk_tri_ptr, h.blk_tri_ptr);
+        UP(d.blk_tri, h.blk_tri);
+        UP(d.iell_loc, iloc);
+        // (the limit holds for every state of the process: the largest any may ask for)
+        const int bytes = (int)force_smem_bytes(kForceTris);
+        const auto allow = [&](auto kern) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        };
+        allow(k_force32<6>);
+        allow(k_force32<8>);
+        allow(k_force32<12>);
     }
+    if (dev32 && e == cudaSuccess) e = cudaMemsetAsync(st->buf.R32 + (size_t)18 * h.T, 0, 18 * sizeof(float), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(st->buf.diag_done, 0, sizeof(unsigned), s);
     UP(d.wall_a, h.wall_a);
     UP(d.wall_b, h.wall_b);
     UP(d.wall_id, h.wall_id);
