@@ -2319,32 +2319,12 @@ int felbm_workspace_bytes(const felbm_mesh* mesh, const felbm_params* params, si
     return FELBM_OK;
 }
 
-int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double* C0, const double* p0,
-               const double* u0, void* d_workspace, size_t workspace_bytes, void* stream, felbm_state** out) {
-    if (!mesh || !C0 || !out) {
-        set_error("felbm_init: invalid argument");
-        return FELBM_ERR_INVALID_ARG;
-    }
-    *out = nullptr;
-    int rc = check_params(params);
-    if (rc) return rc;
-    const HostMesh& h = mesh->h;
-    for (int32_t e = 0; e < h.E; ++e)
-        if (h.wall_id[e] >= params->n_wall_ids) {
-            set_error("felbm_init: a wall id has no phi_c (n_wall_ids too small)");
-            return FELBM_ERR_INVALID_ARG;
-        }
+// The tables and the first state of a new felbm_state; what it returns or throws
+// leaves st to the caller.  No allocation stands between the first upload and
+// the wait for the stream.
+static int set_up(felbm_state* st, const HostMesh& h, const felbm_params* params, const double* C0, const double* p0,
+                  const double* u0, void* d_workspace, void* stream) {
     const bool dev32 = params->precision == FELBM_FP32_DEV;
-    size_t need = carve(h, dev32, nullptr, nullptr, nullptr);
-    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255)) {
-        set_error("felbm_init: workspace missing, not 256-byte aligned or smaller than felbm_workspace_bytes");
-        return FELBM_ERR_WORKSPACE;
-    }
-    felbm_state* st = new (std::nothrow) felbm_state;
-    if (!st) {
-        set_error("felbm_init: out of host memory");
-        return FELBM_ERR_INVALID_ARG;
-    }
     st->hm = h;
     st->prm = *params;
     st->stream = static_cast<cudaStream_t>(stream);
@@ -2482,7 +2462,6 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
         });
         if (stray) {
             set_error("felbm_init: internal error, a row entry outside its block's layers");
-            delete st;
             return FELBM_ERR_BAD_MESH;
         }
     }
@@ -2535,10 +2514,8 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     cudaStream_t s = st->stream;
     const DevMesh& d = st->dm;
     auto fail = [&](cudaError_t e, const char* what) {
-        int r = cuda_fail(e, what);
         cudaStreamSynchronize(s);
-        delete st;
-        return r;
+        return cuda_fail(e, what);
     };
     cudaError_t e = cudaSuccess;
 #define UP(dst, src) \
@@ -2650,31 +2627,56 @@ int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double*
     if (e != cudaSuccess) return fail(e, "felbm_init: cudaGetDevice");
     // mass at t = 0 (for the drift)
     felbm_diag dg;
-    *out = st;
-    rc = felbm_diagnostics(st, nullptr, &dg);
-    if (rc != FELBM_OK && rc != FELBM_ERR_NONFINITE) {
-        *out = nullptr;
-        delete st;
-        return rc;
-    }
+    int rc = felbm_diagnostics(st, nullptr, &dg);
+    if (rc != FELBM_OK && rc != FELBM_ERR_NONFINITE) return rc;
     st->mass0 = dg.mass;
     st->gmass0.assign(h.G, dg.mass);
     if (h.G > 1) {   // one member: its mass is the mass
         std::vector<felbm_diag> gd(h.G);
         rc = felbm_diagnostics_groups(st, nullptr, h.G, gd.data());
-        if (rc != FELBM_OK && rc != FELBM_ERR_NONFINITE) {
-            *out = nullptr;
-            delete st;
-            return rc;
-        }
+        if (rc != FELBM_OK && rc != FELBM_ERR_NONFINITE) return rc;
         for (int32_t g = 0; g < h.G; ++g) st->gmass0[g] = gd[g].mass;
     }
-    rc = set_schedule(st, 0);
+    return set_schedule(st, 0);
+}
+
+int felbm_init(const felbm_mesh* mesh, const felbm_params* params, const double* C0, const double* p0,
+               const double* u0, void* d_workspace, size_t workspace_bytes, void* stream, felbm_state** out) {
+    if (!mesh || !C0 || !out) {
+        set_error("felbm_init: invalid argument");
+        return FELBM_ERR_INVALID_ARG;
+    }
+    *out = nullptr;
+    int rc = check_params(params);
+    if (rc) return rc;
+    const HostMesh& h = mesh->h;
+    for (int32_t e = 0; e < h.E; ++e)
+        if (h.wall_id[e] >= params->n_wall_ids) {
+            set_error("felbm_init: a wall id has no phi_c (n_wall_ids too small)");
+            return FELBM_ERR_INVALID_ARG;
+        }
+    const bool dev32 = params->precision == FELBM_FP32_DEV;
+    size_t need = carve(h, dev32, nullptr, nullptr, nullptr);
+    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255)) {
+        set_error("felbm_init: workspace missing, not 256-byte aligned or smaller than felbm_workspace_bytes");
+        return FELBM_ERR_WORKSPACE;
+    }
+    felbm_state* st = new (std::nothrow) felbm_state;
+    if (!st) {
+        set_error("felbm_init: out of host memory");
+        return FELBM_ERR_INVALID_ARG;
+    }
+    try {
+        rc = set_up(st, h, params, C0, p0, u0, d_workspace, stream);
+    } catch (const std::exception& ex) {
+        set_error(std::string("felbm_init: ") + ex.what());
+        rc = FELBM_ERR_INVALID_ARG;
+    }
     if (rc != FELBM_OK) {
-        *out = nullptr;
         delete st;
         return rc;
     }
+    *out = st;
     return FELBM_OK;
 }
 
