@@ -2431,30 +2431,27 @@ static int set_up(felbm_state* st, const HostMesh& h, const felbm_params* params
         blk_col.assign((size_t)rows * wc, 0);
         std::atomic<int> stray{0};
         const int32_t Np = st->dm.Np;
-        struct Index {
-            std::vector<int32_t> blk, at;      // a node's index in the list of the block that saw it last
-        };
-        const auto make = [&]() { return Index{std::vector<int32_t>(h.N, -1), std::vector<int32_t>(h.N)}; };
-        parallel_for(nblk, 4, make, [&](int32_t t, Index& ix) {
+        parallel_for(nblk, 4, []() { return NodePlaces(); }, [&](int32_t t, NodePlaces& around) {
             const int32_t s0 = h.blk_ptr[t], ni = h.blk_ptr[t + 1] - s0;
             const int32_t* cnt = h.layer_cnt.data() + (size_t)t * (kBlockSteps + 1);
             const int32_t* halo = h.halo.data() + h.halo_ptr[t];
             const int32_t nr = cnt[h.n_layers - 1], stride = blk_row[t + 1] - blk_row[t];
             float* val = blk_val.data() + (size_t)ellw * blk_row[t];
             uint32_t* col = blk_col.data() + (size_t)wc * blk_row[t];
-            for (int32_t r = 0; r < cnt[h.n_layers]; ++r) {
-                const int32_t i = r < ni ? s0 + r : halo[r - ni];
-                ix.blk[i] = t;
-                ix.at[i] = r;
-            }
+            around.clear();
+            for (int32_t r = ni; r < cnt[h.n_layers]; ++r) around.add(halo[r - ni], r);
             for (int32_t r = 0; r < nr; ++r) {
                 const int32_t i = r < ni ? s0 + r : halo[r - ni];
                 for (int k = 0; k < ellw; ++k) {
                     val[(size_t)k * stride + r] = ell_val[(size_t)k * Np + i];
                     if (k == 0) continue;
                     const int32_t c = ell_col[(size_t)k * Np + i];
-                    if (ix.blk[c] != t) stray = 1;
-                    const uint32_t at = ix.blk[c] == t ? (uint32_t)ix.at[c] : (uint32_t)r;
+                    uint32_t at = (uint32_t)(c - s0);
+                    if (c < s0 || c >= s0 + ni) {
+                        const size_t slot = around.slot(c);
+                        if (around.node[slot] != c) stray = 1;
+                        at = around.node[slot] == c ? (uint32_t)around.place[slot] : (uint32_t)r;
+                    }
                     uint32_t& pair = col[(size_t)((k - 1) / 2) * stride + r];
                     pair = (k & 1) ? at | (uint32_t)r << 16 : (pair & 0xffffu) | at << 16;
                 }

@@ -57,6 +57,30 @@ void parallel_for(int32_t n, int32_t grain, const Make& make, const F& f) {
     if (failed) std::rethrow_exception(failed);
 }
 
+// The nodes around one block and their places in its node list: a hash table of a
+// fixed size, so that what a thread of parallel_for keeps does not grow with the
+// mesh.  Holds up to kBlockNodes + 1 nodes.
+struct NodePlaces {
+    static constexpr int kBits = 12;
+    std::vector<int32_t> node, place;
+    NodePlaces() : node(size_t(1) << kBits, -1), place(size_t(1) << kBits) {}
+    void clear() { std::fill(node.begin(), node.end(), -1); }
+    // the slot that holds node c, or the free one where it would stand
+    size_t slot(int32_t c) const {
+        size_t s = (uint32_t)c * 2654435761u >> (32 - kBits);
+        while (node[s] >= 0 && node[s] != c) s = (s + 1) & (node.size() - 1);
+        return s;
+    }
+    bool add(int32_t c, int32_t at) {        // false: it was there
+        const size_t s = slot(c);
+        if (node[s] == c) return false;
+        node[s] = c;
+        place[s] = at;
+        return true;
+    }
+};
+static_assert(kBlockNodes + 1 < 1 << (NodePlaces::kBits - 1), "the table of NodePlaces stays half empty");
+
 // Host mesh after preprocessing.  Node ids are the internal ids (node tiles
 // of recursive coordinate bisection, reverse Cuthill-McKee order inside a
 // tile); perm[new] = caller id, iperm[caller] = new.

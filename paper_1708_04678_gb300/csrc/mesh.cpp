@@ -496,42 +496,43 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
     // ---- first layer of every tile (its size only), layers of every block ----
     {
         const int32_t ntile = (int32_t)m.tile_ptr.size() - 1, nblk = (int32_t)m.blk_ptr.size() - 1;
-        using Marks = std::vector<int32_t>;                  // the run that saw a node last
-        const auto unmarked = [&]() { return Marks(N, -1); };
-        // the nodes outside run k = [s0, s1) that row i references and that it has not seen
-        const auto visit = [&](int32_t i, int32_t k, int32_t s0, int32_t s1, Marks& mark, std::vector<int32_t>& out) {
-            for (int32_t p = m.row_ptr[i]; p < m.row_ptr[i + 1]; ++p) {
-                const int32_t c = m.col[p];
-                if ((c >= s0 && c < s1) || mark[c] == k) continue;
-                mark[c] = k;
-                out.push_back(c);
-            }
-        };
         std::vector<int32_t> first(ntile);
-        parallel_for(ntile, 4, unmarked, [&](int32_t k, Marks& mark) {
-            std::vector<int32_t> out;
-            for (int32_t i = m.tile_ptr[k]; i < m.tile_ptr[k + 1]; ++i)
-                visit(i, k, m.tile_ptr[k], m.tile_ptr[k + 1], mark, out);
-            first[k] = (int32_t)out.size();
+        using List = std::vector<int32_t>;
+        parallel_for(ntile, 4, []() { return List(); }, [&](int32_t k, List& out) {
+            const int32_t s0 = m.tile_ptr[k], s1 = m.tile_ptr[k + 1];
+            out.clear();
+            for (int32_t p = m.row_ptr[s0]; p < m.row_ptr[s1]; ++p)
+                if (m.col[p] < s0 || m.col[p] >= s1) out.push_back(m.col[p]);
+            std::sort(out.begin(), out.end());
+            first[k] = (int32_t)(std::unique(out.begin(), out.end()) - out.begin());
         });
         m.max_halo = *std::max_element(first.begin(), first.end());
         const int32_t stride = kBlockSteps + 1;
         m.layer_cnt.assign((size_t)nblk * stride, 0);
         std::vector<std::vector<int32_t>> ring(nblk);
         std::vector<int32_t> fits(nblk);
-        parallel_for(nblk, 4, unmarked, [&](int32_t k, Marks& mark) {
+        parallel_for(nblk, 4, []() { return NodePlaces(); }, [&](int32_t k, NodePlaces& seen) {
             const int32_t s0 = m.blk_ptr[k], s1 = m.blk_ptr[k + 1];
             std::vector<int32_t>& h = ring[k];
             h.reserve(kBlockNodes);
             int32_t* cnt = m.layer_cnt.data() + (size_t)k * stride;
             cnt[0] = s1 - s0;
+            seen.clear();
+            const auto full = [&]() { return s1 - s0 + (int64_t)h.size() > kBlockNodes; };
+            // the nodes outside that row i references and that were not seen, until the block is over-full
+            const auto visit = [&](int32_t i) {
+                for (int32_t p = m.row_ptr[i]; p < m.row_ptr[i + 1] && !full(); ++p) {
+                    const int32_t c = m.col[p];
+                    if ((c < s0 || c >= s1) && seen.add(c, 0)) h.push_back(c);
+                }
+            };
             size_t from = 0;
             for (int32_t l = 1; l <= kBlockSteps; ++l) {
                 const size_t to = h.size();
                 if (l == 1)
-                    for (int32_t i = s0; i < s1; ++i) visit(i, k, s0, s1, mark, h);
-                for (size_t q = from; l > 1 && q < to; ++q) visit(h[q], k, s0, s1, mark, h);
-                if (s1 - s0 + (int64_t)h.size() > kBlockNodes) break;
+                    for (int32_t i = s0; i < s1; ++i) visit(i);
+                for (size_t q = from; l > 1 && q < to; ++q) visit(h[q]);
+                if (full()) break;
                 std::sort(h.begin() + to, h.end());
                 from = to;
                 cnt[l] = s1 - s0 + (int32_t)h.size();

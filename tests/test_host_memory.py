@@ -42,3 +42,66 @@ sys.exit(0 if all(rc == -1 and "felbm_init" in msg and p is None for rc, msg, p 
 def test_init_returns_an_error_when_host_memory_runs_out():
     r = subprocess.run([sys.executable, "-c", STARVED], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
+# Largest block of memory that a worker thread of the set-up asks for, with the
+# threads that a host of many cores would start: a preloaded library answers
+# std::thread::hardware_concurrency and watches operator new.  felbm_init stops at
+# its first upload (no device here).
+WATCH = r"""
+#include <atomic>
+#include <cstdlib>
+#include <new>
+#include <thread>
+#include <unistd.h>
+static std::atomic<size_t> biggest{0}, workers{0};
+unsigned std::thread::hardware_concurrency() noexcept { return 16; }
+void* operator new(size_t n) {
+    static thread_local bool seen = false;
+    if (gettid() != getpid()) {
+        if (!seen) workers++;
+        seen = true;
+        size_t b = biggest;
+        while (n > b && !biggest.compare_exchange_weak(b, n)) {}
+    }
+    if (void* p = std::malloc(n ? n : 1)) return p;
+    throw std::bad_alloc();
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, size_t) noexcept { std::free(p); }
+extern "C" size_t biggest_of_workers() { return biggest.exchange(0); }
+extern "C" size_t workers_seen() { return workers.exchange(0); }
+"""
+
+SET_UP = r"""
+import ctypes, sys
+import numpy as np
+from paper_1708_04678_gb300 import felbm as F, inputs as I
+watch = ctypes.CDLL(sys.argv[1])
+watch.biggest_of_workers.restype = watch.workers_seen.restype = ctypes.c_size_t
+w = I.small_sessile(nx=500, ny=250, R=60.0)
+F.lib()
+watch.biggest_of_workers(), watch.workers_seen()
+mesh = F.Mesh.from_dict(w["mesh"])
+print(watch.workers_seen(), watch.biggest_of_workers())
+params = F.params_derive(w["phys"], precision=F.FP32_DEV)
+out, C0 = ctypes.c_void_p(), np.ascontiguousarray(w["C0"])
+rc = F.lib().felbm_init(mesh.handle, ctypes.byref(params), C0.ctypes.data, None, None, 1 << 40,
+                        mesh.workspace_bytes(params), None, ctypes.byref(out))
+assert rc == -3, rc
+print(watch.workers_seen(), watch.biggest_of_workers())
+"""
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the workspace pointer is not a device's")
+def test_scratch_of_the_threads_does_not_grow_with_the_mesh(tmp_path):
+    src, lib = tmp_path / "watch.cpp", tmp_path / "watch.so"
+    src.write_text(WATCH)
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", str(src), "-o", str(lib)], check=True)
+    r = subprocess.run([sys.executable, "-c", SET_UP, str(lib)], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, LD_PRELOAD=str(lib)))
+    assert r.returncode == 0, r.stderr[-2000:]
+    for line in r.stdout.splitlines():
+        workers, biggest = (int(v) for v in line.split())
+        # a word per node would be 502 KB; a block has at most 1,024 nodes and 1,400 triangles
+        assert workers > 0 and biggest < 64 * 1024, r.stdout
