@@ -1333,32 +1333,11 @@ int felbm3d_workspace_bytes(const felbm3d_mesh* mesh, const felbm_params* params
     return FELBM_OK;
 }
 
-int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const double* C0, void* d_workspace,
-                 size_t workspace_bytes, void* stream, felbm3d_state** out) {
-    if (!mesh || !C0 || !out) {
-        set_error("felbm3d_init: invalid argument");
-        return FELBM_ERR_INVALID_ARG;
-    }
-    *out = nullptr;
-    int rc = check_params3(params);
-    if (rc) return rc;
-    const HostMesh3D& h = mesh->h;
-    for (int32_t f = 0; f < h.F; ++f)
-        if (h.wall_id[f] >= params->n_wall_ids) {
-            set_error("felbm3d_init: a wall id has no phi_c (n_wall_ids too small)");
-            return FELBM_ERR_INVALID_ARG;
-        }
+// The tables and the first state of a new felbm3d_state; what it returns or throws
+// leaves st to the caller.
+static int set_up3(felbm3d_state* st, const HostMesh3D& h, const felbm_params* params, const double* C0, void* d_workspace,
+                   size_t need, void* stream) {
     const bool dev32 = params->precision == FELBM_FP32_DEV;
-    const size_t need = carve3(h, dev32, nullptr, nullptr, nullptr);
-    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255)) {
-        set_error("felbm3d_init: workspace missing, not 256-byte aligned or smaller than felbm3d_workspace_bytes");
-        return FELBM_ERR_WORKSPACE;
-    }
-    felbm3d_state* st = new (std::nothrow) felbm3d_state;
-    if (!st) {
-        set_error("felbm3d_init: out of host memory");
-        return FELBM_ERR_INVALID_ARG;
-    }
     st->hm = h;
     st->prm = *params;
     st->stream = static_cast<cudaStream_t>(stream);
@@ -1368,10 +1347,7 @@ int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const dou
         int device = 0;
         cudaError_t qe = cudaGetDevice(&device);
         if (qe == cudaSuccess) qe = cudaDeviceGetAttribute(&st->n_sm, cudaDevAttrMultiProcessorCount, device);
-        if (qe != cudaSuccess) {
-            delete st;
-            return cuda_fail(qe, "felbm3d_init: device");
-        }
+        if (qe != cudaSuccess) return cuda_fail(qe, "felbm3d_init: device");
     }
     carve3(h, dev32, d_workspace, &st->dm, &st->buf);
     Phys3& ph = st->phys;
@@ -1502,20 +1478,50 @@ int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const dou
 #undef UP3
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(st->buf.stage, C0, sizeof(double) * h.N, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) {
-        rc = cuda_fail(e, "felbm3d_init: upload");
-        delete st;
-        return rc;
+    const cudaError_t done = cudaStreamSynchronize(s);     // also after a failed upload: its predecessors read the tables
+    if (e == cudaSuccess) e = done;
+    if (e != cudaSuccess) return cuda_fail(e, "felbm3d_init: upload");
+    if (int rc = init_state_from_stage(st)) return rc;
+    double v[kDiagSlots];
+    DiagReq3 rq{};
+    rq.substrate = -1;
+    rq.dev32 = st->dev32;
+    const int rc = diag_run(st, rq, v);
+    st->mass0 = v[0];
+    return rc;
+}
+
+int felbm3d_init(const felbm3d_mesh* mesh, const felbm_params* params, const double* C0, void* d_workspace,
+                 size_t workspace_bytes, void* stream, felbm3d_state** out) {
+    if (!mesh || !C0 || !out) {
+        set_error("felbm3d_init: invalid argument");
+        return FELBM_ERR_INVALID_ARG;
     }
-    rc = init_state_from_stage(st);
-    if (rc == FELBM_OK) {
-        double v[kDiagSlots];
-        DiagReq3 rq{};
-        rq.substrate = -1;
-        rq.dev32 = st->dev32;
-        rc = diag_run(st, rq, v);
-        st->mass0 = v[0];
+    *out = nullptr;
+    int rc = check_params3(params);
+    if (rc) return rc;
+    const HostMesh3D& h = mesh->h;
+    for (int32_t f = 0; f < h.F; ++f)
+        if (h.wall_id[f] >= params->n_wall_ids) {
+            set_error("felbm3d_init: a wall id has no phi_c (n_wall_ids too small)");
+            return FELBM_ERR_INVALID_ARG;
+        }
+    const bool dev32 = params->precision == FELBM_FP32_DEV;
+    const size_t need = carve3(h, dev32, nullptr, nullptr, nullptr);
+    if (!d_workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(d_workspace) & 255)) {
+        set_error("felbm3d_init: workspace missing, not 256-byte aligned or smaller than felbm3d_workspace_bytes");
+        return FELBM_ERR_WORKSPACE;
+    }
+    felbm3d_state* st = new (std::nothrow) felbm3d_state;
+    if (!st) {
+        set_error("felbm3d_init: out of host memory");
+        return FELBM_ERR_INVALID_ARG;
+    }
+    try {
+        rc = set_up3(st, h, params, C0, d_workspace, need, stream);
+    } catch (const std::exception& ex) {
+        set_error(std::string("felbm3d_init: ") + ex.what());
+        rc = FELBM_ERR_INVALID_ARG;
     }
     if (rc != FELBM_OK) {
         delete st;

@@ -44,6 +44,39 @@ def test_init_returns_an_error_when_host_memory_runs_out():
     assert r.returncode == 0, (r.returncode, r.stdout, r.stderr[-2000:])
 
 
+# The other entries that make tables, in the same way.
+STARVED_OTHERS = r"""
+import ctypes, resource, sys
+import numpy as np
+from paper_1708_04678_gb300 import felbm as F, felbm3d as F3, inputs as I, inputs3d as I3
+
+def starved(call, spare):
+    kb = next(int(l.split()[1]) for l in open("/proc/self/status") if l.startswith("VmSize"))
+    resource.setrlimit(resource.RLIMIT_AS, ((kb << 10) + (spare << 20), resource.RLIM_INFINITY))
+    rc = call()
+    resource.setrlimit(resource.RLIMIT_AS, (resource.RLIM_INFINITY, resource.RLIM_INFINITY))
+    return rc, F.lib().felbm_last_error().decode()
+
+rcs = []
+w = I3.small_sessile_3d(n=40, nz=40)
+mesh = F3.Mesh3D.from_dict(w["mesh"])
+params = F.params_derive(w["phys"])
+C0, out = np.ascontiguousarray(w["C0"]), ctypes.c_void_p()
+args = (mesh.handle, ctypes.byref(params), C0.ctypes.data, 1 << 40, mesh.workspace_bytes(params), None, ctypes.byref(out))
+rcs.append(starved(lambda: F3.lib().felbm3d_init(*args), 1))
+print(rcs)
+sys.exit(0 if all(rc == -1 and "felbm" in msg and not out.value for rc, msg in rcs) else 3)
+"""
+
+
+@pytest.mark.skipif(torch.cuda.is_available(), reason="the workspace pointer is not a device's")
+def test_other_entries_return_an_error_when_host_memory_runs_out():
+    # large blocks straight from the system, so that none comes from freed memory
+    r = subprocess.run([sys.executable, "-c", STARVED_OTHERS], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                       env=dict(os.environ, MALLOC_MMAP_THRESHOLD_="65536"))
+    assert r.returncode == 0, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
 # Largest block of memory that a worker thread of the set-up asks for, with the
 # threads that a host of many cores would start: a preloaded library answers
 # std::thread::hardware_concurrency and watches operator new.  felbm_init stops at
