@@ -691,6 +691,39 @@ static int build_mesh(const double* xy, int32_t N, const int32_t* tri_in, int32_
     return FELBM_OK;
 }
 
+// The members' meshes as one: nodes and triangles one after another.
+static int build_batch(int32_t n_meshes, const felbm_mesh_desc* meshes, int64_t N, int64_t T, int64_t E, HostMesh& m) {
+    std::vector<double> xy(2 * N), npx(N), npy(N);
+    std::vector<int32_t> tri(3 * T), we(2 * E), wid(E);
+    int64_t n0 = 0, t0 = 0, e0 = 0;
+    for (int32_t k = 0; k < n_meshes; ++k) {
+        const felbm_mesh_desc& d = meshes[k];
+        std::copy(d.xy, d.xy + 2 * (size_t)d.n_nodes, xy.begin() + 2 * n0);
+        std::fill(npx.begin() + n0, npx.begin() + n0 + d.n_nodes, d.period_x);
+        std::fill(npy.begin() + n0, npy.begin() + n0 + d.n_nodes, d.period_y);
+        for (int64_t i = 0; i < 3LL * d.n_tri; ++i) {
+            if (d.tri[i] < 0 || d.tri[i] >= d.n_nodes) {
+                set_error("felbm_mesh_create_batch: triangle node id out of range");
+                return FELBM_ERR_INVALID_ARG;
+            }
+            tri[3 * t0 + i] = (int32_t)(d.tri[i] + n0);
+        }
+        for (int64_t i = 0; i < 2LL * d.n_wall_edges; ++i) {
+            if (d.wall_edges[i] < 0 || d.wall_edges[i] >= d.n_nodes) {
+                set_error("felbm_mesh_create_batch: wall edge node id out of range");
+                return FELBM_ERR_INVALID_ARG;
+            }
+            we[2 * e0 + i] = (int32_t)(d.wall_edges[i] + n0);
+        }
+        std::copy(d.wall_id, d.wall_id + d.n_wall_edges, wid.begin() + e0);
+        n0 += d.n_nodes;
+        t0 += d.n_tri;
+        e0 += d.n_wall_edges;
+    }
+    return build_mesh(xy.data(), (int32_t)N, tri.data(), (int32_t)T, E ? we.data() : nullptr, E ? wid.data() : nullptr,
+                      (int32_t)E, npx, npy, m);
+}
+
 }  // namespace felbm
 
 extern "C" {
@@ -768,33 +801,6 @@ int felbm_mesh_create_batch(int32_t n_meshes, const felbm_mesh_desc* meshes, fel
         felbm::set_error("felbm_mesh_create_batch: batch too large for 32-bit indices");
         return FELBM_ERR_INVALID_ARG;
     }
-    std::vector<double> xy(2 * N), npx(N), npy(N);
-    std::vector<int32_t> tri(3 * T), we(2 * E), wid(E);
-    int64_t n0 = 0, t0 = 0, e0 = 0;
-    for (int32_t k = 0; k < n_meshes; ++k) {
-        const felbm_mesh_desc& d = meshes[k];
-        std::copy(d.xy, d.xy + 2 * (size_t)d.n_nodes, xy.begin() + 2 * n0);
-        std::fill(npx.begin() + n0, npx.begin() + n0 + d.n_nodes, d.period_x);
-        std::fill(npy.begin() + n0, npy.begin() + n0 + d.n_nodes, d.period_y);
-        for (int64_t i = 0; i < 3LL * d.n_tri; ++i) {
-            if (d.tri[i] < 0 || d.tri[i] >= d.n_nodes) {
-                felbm::set_error("felbm_mesh_create_batch: triangle node id out of range");
-                return FELBM_ERR_INVALID_ARG;
-            }
-            tri[3 * t0 + i] = (int32_t)(d.tri[i] + n0);
-        }
-        for (int64_t i = 0; i < 2LL * d.n_wall_edges; ++i) {
-            if (d.wall_edges[i] < 0 || d.wall_edges[i] >= d.n_nodes) {
-                felbm::set_error("felbm_mesh_create_batch: wall edge node id out of range");
-                return FELBM_ERR_INVALID_ARG;
-            }
-            we[2 * e0 + i] = (int32_t)(d.wall_edges[i] + n0);
-        }
-        std::copy(d.wall_id, d.wall_id + d.n_wall_edges, wid.begin() + e0);
-        n0 += d.n_nodes;
-        t0 += d.n_tri;
-        e0 += d.n_wall_edges;
-    }
     felbm_mesh* m = new (std::nothrow) felbm_mesh;
     if (!m) {
         felbm::set_error("felbm_mesh_create_batch: out of host memory");
@@ -802,8 +808,7 @@ int felbm_mesh_create_batch(int32_t n_meshes, const felbm_mesh_desc* meshes, fel
     }
     int rc;
     try {
-        rc = felbm::build_mesh(xy.data(), (int32_t)N, tri.data(), (int32_t)T, E ? we.data() : nullptr,
-                               E ? wid.data() : nullptr, (int32_t)E, npx, npy, m->h);
+        rc = felbm::build_batch(n_meshes, meshes, N, T, E, m->h);
     } catch (const std::exception& ex) {
         felbm::set_error(std::string("felbm_mesh_create_batch: ") + ex.what());
         rc = FELBM_ERR_INVALID_ARG;

@@ -64,6 +64,15 @@ params = F.params_derive(w["phys"])
 C0, out = np.ascontiguousarray(w["C0"]), ctypes.c_void_p()
 args = (mesh.handle, ctypes.byref(params), C0.ctypes.data, 1 << 40, mesh.workspace_bytes(params), None, ctypes.byref(out))
 rcs.append(starved(lambda: F3.lib().felbm3d_init(*args), 1))
+m = I.small_sessile(nx=1500, ny=700, R=100.0)["mesh"]
+xy, tri = np.ascontiguousarray(m["xy"], dtype=np.float64), np.ascontiguousarray(m["tri"], dtype=np.int32)
+we, wid = np.ascontiguousarray(m["wall_edges"], dtype=np.int32), np.ascontiguousarray(m["wall_id"], dtype=np.int32)
+d = (F.MeshDesc * 1)()
+d[0].xy, d[0].n_nodes, d[0].tri, d[0].n_tri = xy.ctypes.data, len(xy), tri.ctypes.data, len(tri)
+d[0].wall_edges, d[0].wall_id, d[0].n_wall_edges = we.ctypes.data, wid.ctypes.data, len(we)
+d[0].period_x = float(m["period"][0])
+for spare in (0, 8, 16, 32):
+    rcs.append(starved(lambda: F.lib().felbm_mesh_create_batch(1, d, ctypes.byref(out)), spare))
 print(rcs)
 sys.exit(0 if all(rc == -1 and "felbm" in msg and not out.value for rc, msg in rcs) else 3)
 """
