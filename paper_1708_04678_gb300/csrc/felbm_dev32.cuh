@@ -41,7 +41,7 @@ __device__ __forceinline__ float gamma32(float ux, float uy, float uu15) {
 }
 
 // ------------------------------------------------- chemical potential ------
-// Same arithmetic as k_mu (FP64), FP32 output.
+// The terms of k_mu (FP64), the Laplacian as differences to C_i; FP32 output.
 __device__ __forceinline__ void mu32_node(const DevMesh& m, const Phys& c, const Bufs& b, int i) {
     double Ci = b.C[i];
     double lap = 0.0;
@@ -410,7 +410,8 @@ __global__ void __launch_bounds__(128, 8) k_rhs32(DevMesh m, Phys c, Bufs b, flo
 // k_rhs32 in the same order; the residuals, 72 bytes a triangle written and
 // gathered back through DRAM by those two, never leave the multiprocessor, for
 // about 10 % of the triangles formed twice.  Bound by load latency and L1 (48 %
-// of its wavefronts, 34 % of the issue slots, 24 warps at 80 registers): 337 us
+// of its wavefronts, 34 % of the issue slots, 24 warps at 80 registers, which
+// spill 88 to 100 bytes a thread): 337 us
 // on 2,082,816 nodes against 237 + 144 us for the two kernels, 31 against 22 +
 // 19 us on 131,072 nodes.  Two threads a triangle at 80 or 64 registers: 352
 // and 381 us; 256 threads a block: 416 us.  Residual rows hold the planes of
