@@ -252,8 +252,8 @@ class ClockSampler:
                 "sm_max_mhz": max(mx) if mx else None, "reasons": reasons, "samples": len(self.rows)}
 
 
-SOURCES_2D = ("felbm.cu", "felbm_dev32.cuh", "felbm_block32.cuh", "felbm_adjoint.cuh", "felbm_internal.h", "mesh.cpp", "felbm.h")
-SOURCES_3D = ("felbm3d.cu", "felbm3d_dev32.cuh", "felbm3d_internal.h", "mesh3d.cpp", "felbm_internal.h",
+SOURCES_2D = ("felbm.cu", "felbm_start32.cuh", "felbm_dev32.cuh", "felbm_block32.cuh", "felbm_adjoint.cuh", "felbm_internal.h", "mesh.cpp", "felbm.h")
+SOURCES_3D = ("felbm3d.cu", "felbm_start32.cuh", "felbm3d_dev32.cuh", "felbm3d_internal.h", "mesh3d.cpp", "felbm_internal.h",
               "felbm3d.h", "felbm.h")
 
 

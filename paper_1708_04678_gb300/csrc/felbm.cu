@@ -124,6 +124,7 @@ struct DevMesh {
     const int32_t* iell_tri;  // [iell_w][Np] incident triangle (padding: T, a zero residual row)
     const float* iell_bx32;   // [iell_w][Np] the node's shape gradient in that triangle
     const float* iell_by32;
+    const float2* start32;    // [Np] tau_0 / m_i of the FP32 corrections (Start32)
     const float* inv_lumped32;// [Np]
     const double* lumped;     // [Np]
     const double* inv_vol;    // [Np] 1 / V_i
@@ -286,15 +287,7 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
 }
 
-// A double rounded to a float (nearest, ties to even) through the integer pipe,
-// for the same reason; what is not a normal float takes the instruction.
-__device__ __forceinline__ float narrow(double x) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint32_t e = (hi & 0x7fffffffu) - 0x38100000u;          // exponent above the least of a normal float
-    if (e >= 0x0fe00000u) return (float)x;
-    const uint32_t f = (e + 0x00100000u) << 3 | lo >> 29;
-    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
-}
+#include "felbm_start32.cuh"
 
 constexpr int kBlock = 256;
 constexpr int kWarpBlocksBelow = 512;   // items per multiprocessor (fp64_block)
@@ -545,15 +538,11 @@ __global__ void __launch_bounds__(128) k_element(DevMesh m, Phys c, Bufs b) {
     for (int k = 0; k < 9; ++k) dst[k] = make_double2(out[2 * k], out[2 * k + 1]);
 }
 
-// The right-hand side of an FP32 correction and its first iterate s r, the FP64
-// product rounded once.
-__device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const double (&r)[18], double s) {
+// The right-hand side of an FP32 correction and its first iterate.
+__device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const double (&r)[18], const Start32& start) {
     float r32[18], e[18];
 #pragma unroll
-    for (int q = 0; q < 18; ++q) {
-        r32[q] = narrow(r[q]);
-        e[q] = narrow(r[q] * s);
-    }
+    for (int q = 0; q < 18; ++q) start(r[q], r32[q], e[q]);
     store_all(b.r32, Np, i, r32);
     store_all(b.e1, Np, i, e);
 }
@@ -568,9 +557,9 @@ __device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const 
 // mixed-precision solve, in FP32 together with the FP32 copy of the
 // right-hand side.
 //
-// Bound by the FP64 pipe (108 FMAs, 60 operations on the weights, 18 products for
-// the first iterate a node): 204 us on 520,704 nodes, 256 us with the weights
-// formed direction by direction and conversion instructions.
+// Bound by the FP64 pipe (108 FMAs, 60 operations on the weights a node): 180 us on
+// 520,704 nodes, 602 us on 2,082,816 (Start32 in FP64: 204 and 789); 256 us on
+// 520,704 with the weights formed direction by direction as well.
 // One thread per node, or (kSets = 2, consecutive blocks) one per node and set,
 // which forms the weights twice but halves a thread's chain of loads and its
 // straight-line code -- what a small mesh waits for (2,112 nodes: 15.5 us
@@ -591,7 +580,8 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
     int k = m.inc_ptr[i], t = k < k1 ? m.inc_tri[k] : 0;
     double bxi = k < k1 ? m.inc_bx[k] : 0.0, byi = k < k1 ? m.inc_by[k] : 0.0;
     const int w0 = m.winc_ptr[i], w1 = m.winc_ptr[i + 1];
-    const double s = m.inv_lumped[i] * first_scale;
+    const float2 s32 = kMixed ? m.start32[i] : make_float2(0.0f, 0.0f);
+    const double s = kMixed ? 0.0 : m.inv_lumped[i] * first_scale;
     const double* psi = b.psi + (size_t)9 * set * Np;
     while (k < k1) {
         const double* src = b.R + (size_t)t * 18 + 9 * set;
@@ -649,14 +639,12 @@ __global__ void __launch_bounds__(128) k_rhs(DevMesh m, Phys c, Bufs b, double f
         if (!kMixed) b.x1[(9 * set + q) * Np + i] = acc[q] * s;
     }
     if constexpr (kMixed && kSets == 1) {
-        store_start(b, Np, i, acc, s);
+        store_start(b, Np, i, acc, Start32{s32, m.inv_lumped + i, first_scale});
     } else if constexpr (kMixed) {
+        const Start32 start{s32, m.inv_lumped + i, first_scale};
         float r32[9], e[9];
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            r32[q] = narrow(acc[q]);
-            e[q] = narrow(acc[q] * s);
-        }
+        for (int q = 0; q < 9; ++q) start(acc[q], r32[q], e[q]);
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             const float rp[4] = {r32[4 * p + 1], r32[4 * p + 2], r32[4 * p + 3], r32[4 * p + 4]};
@@ -678,6 +666,7 @@ __global__ void __launch_bounds__(kBlock) k_solve_in(DevMesh m, Bufs b, const do
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m.N) return;
     const int Np = m.Np, o = m.perm[i];
+    const Start32 start{m.start32[i], m.inv_lumped + i, first_scale};
     const double s = m.inv_lumped[i] * first_scale;
     double v[18];
 #pragma unroll
@@ -685,15 +674,18 @@ __global__ void __launch_bounds__(kBlock) k_solve_in(DevMesh m, Bufs b, const do
 #pragma unroll
     for (int p = 0; p < kPlanes; ++p) {
         if (p >= n4 && p != 4) continue;
+        double x[4] = {0.0, 0.0, 0.0, 0.0};
         float r[4], e[4];
 #pragma unroll
         for (int c = 0; c < (p < 4 ? 4 : 2); ++c) {
             const int q = vec_row(p, c);
             b.rhs[q * Np + i] = v[q];
             if (!kMixed) b.x1[q * Np + i] = v[q] * s;
-            r[c] = narrow(v[q]);
-            e[c] = narrow(v[q] * s);
+            x[c] = v[q];
         }
+        if (kMixed)
+#pragma unroll
+            for (int c = 0; c < (p < 4 ? 4 : 2); ++c) start(x[c], r[c], e[c]);
         if (kMixed && p < 4) {
             store_vec(b.r32, Np, p, i, r);
             store_vec(b.e1, Np, p, i, e);
@@ -743,7 +735,7 @@ __global__ void __launch_bounds__(kBlock) k_cheb_start(DevMesh m, Bufs b, const 
         if (src != b.rhs) b.rhs[q * Np + i] = acc[q];
         if (!kMixed) b.x1[q * Np + i] = acc[q] * s;
     }
-    if constexpr (kMixed) store_start(b, Np, i, acc, s);
+    if constexpr (kMixed) store_start(b, Np, i, acc, Start32{m.start32[i], m.inv_lumped + i, first_scale});
 }
 
 // ---------------------------------------------- K6: Chebyshev sweep -------
@@ -961,15 +953,14 @@ __global__ void __launch_bounds__(128) k_sweep32(DevMesh m, Phys c, Bufs b, cons
 // plane (consecutive blocks, which share the rows through L2): five times the
 // warps and a fifth of the straight-line code, which is what a small mesh
 // waits for (2,112 nodes: 8.3 us against 15.3 for all planes in a thread; on
-// 520,704 nodes 252 us, of which the first iterate as an FP64 product takes
-// 40).  Bound by the FP64 pipe; with conversion instructions for the 126 gathered
-// values it took 377 us.
+// 520,704 nodes 212 against 197 us).  Bound by the FP64 pipe; with conversion
+// instructions for the 126 gathered values it took 377 us.
 template <int NV>
 __device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, const float* e,
                                              float* next_first, int first_round, double tau0, int p, int i) {
     const int Np = m.Np, k1 = m.row_ptr[i + 1];
     int k = m.row_ptr[i];
-    const double s = m.inv_lumped[i] * tau0;
+    const Start32 start{m.start32[i], m.inv_lumped + i, tau0};
     // every load of the node itself before the first store (the compiler keeps
     // their order, and one at a time they cost a latency each)
     const size_t at = (size_t)(NV == 2 ? 0 : 9 * (p >> 1) + 1 + 4 * (p & 1)) * Np + i, stride = (size_t)(NV == 2 ? 9 : 1) * Np;
@@ -990,14 +981,15 @@ __device__ __forceinline__ void refine_plane(const DevMesh& m, const Bufs& b, co
 #pragma unroll
         for (int c = 0; c < NV; ++c) acc[c] = fma(mv, widen(ej[c]), acc[c]);
     }
+    double rn[NV];
     float r32[NV], first[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
-        const double ed = widen(ei[c]), rn = ro[c] - acc[c];
+        const double ed = widen(ei[c]);
+        rn[c] = ro[c] - acc[c];
         b.x64[at + c * stride] = first_round ? ed : xo[c] + ed;
-        b.rho64[at + c * stride] = rn;
-        r32[c] = narrow(rn);
-        first[c] = narrow(rn * s);
+        b.rho64[at + c * stride] = rn[c];
+        start(rn[c], r32[c], first[c]);
     }
     store_vec(b.r32, Np, p, i, r32);
     store_vec(next_first, Np, p, i, first);
@@ -1667,6 +1659,7 @@ static size_t carve(const HostMesh& h, bool dev32, void* base, DevMesh* dm, Bufs
     d.blk_tri = cv.take<int32_t>(d.max_blk_tri > 0 ? h.blk_tri.size() : 1);
     d.iell_loc = cv.take<uint16_t>(d.max_blk_tri > 0 ? (size_t)iw * Np : 1);
     d.inv_lumped32 = cv.take<float>(Np);
+    d.start32 = cv.take<float2>(Np);
     d.lumped = cv.take<double>(Np);
     d.inv_vol = cv.take<double>(Np);
     d.inc_ptr = cv.take<int32_t>(h.N + 1);
@@ -2395,6 +2388,7 @@ static int set_up(felbm_state* st, const HostMesh& h, const felbm_params* params
     // host-side derived tables
     const double scale = params->lap_mode == FELBM_LAP_PAPER ? 1.0 : 2.0 / 3.0;
     std::vector<double> inv_vol(h.N), inv_lumped(h.N), lval(h.row_ptr[h.N]);
+    std::vector<float2> start32(h.N);
     std::vector<float> inv_lumped32(h.N), mval32(h.mass.begin(), h.mass.end());
     std::vector<double> wall_phi(h.E);
     for (int32_t e = 0; e < h.E; ++e) wall_phi[e] = params->phi_c[h.wall_id[e]];
@@ -2407,6 +2401,7 @@ static int set_up(felbm_state* st, const HostMesh& h, const felbm_params* params
         inv_vol[i] = 1.0 / (scale * h.patch[i]);
         inv_lumped[i] = 1.0 / h.lumped[i];
         inv_lumped32[i] = (float)inv_lumped[i];
+        start32[i] = split_scale(inv_lumped[i] * st->tau[0]);
         for (int32_t k = h.row_ptr[i]; k < h.row_ptr[i + 1]; ++k) lval[k] = -2.0 * h.stiff[k] * inv_vol[i];
     }
     for (int32_t i = 0; i < h.N && ellw > 0; ++i) {
@@ -2557,6 +2552,7 @@ static int set_up(felbm_state* st, const HostMesh& h, const felbm_params* params
     }
     UP(d.ell_lval, ell_lval);
     UP(d.inv_lumped32, inv_lumped32);
+    UP(d.start32, start32);
     UP(d.lumped, h.lumped);
     UP(d.inv_vol, inv_vol);
     UP(d.inc_ptr, h.inc_ptr);

@@ -121,6 +121,7 @@ struct DevMesh3 {
     const float* ell_val;     // [ell_w][Np]
     const float* mval32;      // [nnz]
     const double* inv_lumped; // [Np]
+    const float2* start32;    // [Np] tau_0 / m_i of the FP32 corrections (Start32)
     const float* inv_lumped32;
     const double* lumped;     // [Np]
     const double* inv_vol;    // [Np] 1 / V_i
@@ -250,15 +251,7 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + bias)), (int)(u << 29));
 }
 
-// A double rounded to a float (nearest, ties to even) through the integer pipe,
-// for the same reason; what is not a normal float takes the instruction.
-__device__ __forceinline__ float narrow(double x) {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const uint32_t e = (hi & 0x7fffffffu) - 0x38100000u;          // exponent above the least of a normal float
-    if (e >= 0x0fe00000u) return (float)x;
-    const uint32_t f = (e + 0x00100000u) << 3 | lo >> 29;
-    return __uint_as_float((hi & 0x80000000u) | (f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29)));
-}
+#include "felbm_start32.cuh"
 
 // ------------------------------------------------------ K1: collision -----
 // Moments of the pre-collision state (C = sum h, p = sum g, rho u = sum e g /
@@ -538,7 +531,6 @@ __global__ void __launch_bounds__(kNodeBlock) k3_rhs(DevMesh3 m, Phys3 c, Bufs3 
             }
         }
     }
-    const double sc = m.inv_lumped[i] * first_scale;
     const size_t r = (size_t)q * Np + i, rh = (size_t)(19 + q) * Np + i;
     b.rhs[r] = g0;
     b.rhs[rh] = h0;
@@ -547,18 +539,21 @@ __global__ void __launch_bounds__(kNodeBlock) k3_rhs(DevMesh3 m, Phys3 c, Bufs3 
         b.rhs[rh + Np] = h1;
     }
     if constexpr (kMixed) {
-        // the first iterate is the FP64 product, rounded once
+        const Start32 start{m.start32[i], m.inv_lumped + i, first_scale};
         const size_t a = (size_t)i * kRow + q;
-        b.r32[a] = narrow(g0);
-        b.r32[a + 20] = narrow(h0);
-        b.e1[a] = narrow(g0 * sc);
-        b.e1[a + 20] = narrow(h0 * sc);
         const size_t a1 = (size_t)i * kRow + (cc == 0 ? 19 : q + 1);      // lane 0: the padding slots, zero
-        b.r32[a1] = narrow(g1);
-        b.r32[a1 + 20] = narrow(h1);
-        b.e1[a1] = narrow(g1 * sc);
-        b.e1[a1 + 20] = narrow(h1 * sc);
+        const double v[4] = {g0, h0, g1, h1};
+        float r32[4], first[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) start(v[k], r32[k], first[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const size_t at = (k < 2 ? a : a1) + (k & 1 ? 20 : 0);
+            b.r32[at] = r32[k];
+            b.e1[at] = first[k];
+        }
     } else {
+        const double sc = m.inv_lumped[i] * first_scale;
         b.x1[r] = g0 * sc;
         b.x1[rh] = h0 * sc;
         if (nd == 2) {
@@ -641,17 +636,18 @@ __global__ void __launch_bounds__(kCoopBlock) k3_refine(DevMesh3 m, Bufs3 b, con
         acc[2] = fma(mv, widen(ej.z), acc[2]);
         acc[3] = fma(mv, widen(ej.w), acc[3]);
     }
-    const double sc = m.inv_lumped[i] * tau0;
+    const Start32 start{m.start32[i], m.inv_lumped + i, tau0};
+    double rn[4];
     float r[4], first[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         r[j] = first[j] = 0.0f;                       // the padding slots stay zero
         if (j >= nq) continue;
-        const double ed = widen(comp(ei, j)), rn = ro[j] - acc[j];
+        const double ed = widen(comp(ei, j));
+        rn[j] = ro[j] - acc[j];
         b.x0[r0 + (size_t)j * Np] = first_round ? ed : xo[j] + ed;
-        b.x1[r0 + (size_t)j * Np] = rn;
-        r[j] = narrow(rn);
-        first[j] = narrow(rn * sc);
+        b.x1[r0 + (size_t)j * Np] = rn[j];
+        start(rn[j], r[j], first[j]);
     }
     reinterpret_cast<float4*>(b.r32 + (size_t)i * kRow)[cc] = make_float4(r[0], r[1], r[2], r[3]);
     reinterpret_cast<float4*>(next_first + (size_t)i * kRow)[cc] = make_float4(first[0], first[1], first[2], first[3]);
@@ -1030,6 +1026,7 @@ static size_t carve3(const HostMesh3D& h, bool dev32, void* base, DevMesh3* dm, 
     d.mval32 = cv.take<float>(nnz);
     d.inv_lumped = cv.take<double>(Np);
     d.inv_lumped32 = cv.take<float>(Np);
+    d.start32 = cv.take<float2>(Np);
     d.lumped = cv.take<double>(Np);
     d.inv_vol = cv.take<double>(Np);
     d.inc_ptr = cv.take<int32_t>(h.N + 1);
@@ -1405,6 +1402,7 @@ static int set_up3(felbm3d_state* st, const HostMesh3D& h, const felbm_params* p
     const double scale = params->lap_mode == FELBM_LAP_PAPER ? 1.0 : 0.75;
     const size_t Np = d.Np, Tp = d.Tp, nnz = h.row_ptr[h.N];
     std::vector<double> inv_vol(h.N), inv_lumped(h.N), lval(nnz), wall_phi(h.F);
+    std::vector<float2> start32(h.N);
     std::vector<float> inv_lumped32(h.N), mval32(h.mass.begin(), h.mass.end());
     std::vector<float> inc_b32(h.inc_b.begin(), h.inc_b.end());
     for (int32_t f = 0; f < h.F; ++f) wall_phi[f] = params->phi_c[h.wall_id[f]];
@@ -1412,6 +1410,7 @@ static int set_up3(felbm3d_state* st, const HostMesh3D& h, const felbm_params* p
         inv_vol[i] = 1.0 / (scale * h.patch[i]);
         inv_lumped[i] = 1.0 / h.lumped[i];
         inv_lumped32[i] = (float)inv_lumped[i];
+        start32[i] = split_scale(inv_lumped[i] * st->tau[0]);
         for (int32_t k = h.row_ptr[i]; k < h.row_ptr[i + 1]; ++k) lval[k] = -3.0 * h.stiff[k] * inv_vol[i];
     }
     const int ellw = d.ell_w;
@@ -1458,6 +1457,7 @@ static int set_up3(felbm3d_state* st, const HostMesh3D& h, const felbm_params* p
     UP3(d.mval32, mval32);
     UP3(d.inv_lumped, inv_lumped);
     UP3(d.inv_lumped32, inv_lumped32);
+    UP3(d.start32, start32);
     UP3(d.lumped, h.lumped);
     UP3(d.inv_vol, inv_vol);
     UP3(d.inc_ptr, h.inc_ptr);

@@ -30,27 +30,32 @@ def _cuda():
     build.build()
 
 
+# sizes of the values, side of a cell: in the range where the product is formed in
+# two floats, below and above it, and a mesh whose tau_0 / m is out of it
+@pytest.mark.parametrize("low,high,side", [(-40, 40, 1.0), (-112, -94, 1.0), (40, 100, 1.0), (-40, 40, 1024.0)])
 @pytest.mark.parametrize("blocked", [True, False])
 @pytest.mark.parametrize("rows", [18, 5])
 @pytest.mark.parametrize("rounds", [1, 2])
-def test_first_iterate_is_the_fp64_product_rounded_once(rounds, rows, blocked):
+def test_first_iterate_is_the_fp64_product_rounded_once(rounds, rows, blocked, low, high, side):
     nx, ny = 24, 16
     w = I.small_sessile(nx=nx, ny=ny, R=5.0, jitter=0.0)
     m = w["mesh"]
-    st = F.State(F.Mesh.from_dict(m), F.params_derive(w["phys"], solver_iters=2, solver_rounds=rounds), w["C0"])
+    mesh = dict(m, xy=m["xy"] * side, period=tuple(side * p for p in m["period"]))
+    st = F.State(F.Mesh.from_dict(mesh), F.params_derive(w["phys"], solver_iters=2, solver_rounds=rounds), w["C0"])
     st.sweep_tiled(blocked)
     node = {(round(x), round(y)): k for k, (x, y) in enumerate(m["xy"])}
     tau = [1.0 / (0.625 + 0.375 * math.cos((2 * j + 1) * math.pi / 4)) for j in (0, 1)]
-    mass, v = 0.5 / 12 + 0.5 / 12, f32(0.5 / 12 + 0.5 / 12)
+    lumped = side * side                                      # powers of two: every product with them is exact
+    mass, v = lumped * (0.5 / 12 + 0.5 / 12), f32(lumped * (0.5 / 12 + 0.5 / 12))
     rng = np.random.default_rng(5)
     for rep in range(4):
         centres = [(4, 5), (10, 8), (16, 6), (22, 9)]
-        val = rng.standard_normal((rows, len(centres))) * 2.0 ** rng.uniform(-40, 40, (rows, len(centres)))
+        val = rng.standard_normal((rows, len(centres))) * 2.0 ** rng.uniform(low, high, (rows, len(centres)))
 
         def step(x0):            # one step at a neighbour whose own iterate and right-hand side are zero
-            return f32(f32(tau[1]) * f32(1.0)) * (-(v * x0))
+            return f32(f32(tau[1]) / f32(lumped)) * (-(v * x0))
 
-        e0 = (val * tau[0]).astype(f32)
+        e0 = (val * (tau[0] / lumped)).astype(f32)
         for c, (x, y) in enumerate(centres):
             B = np.zeros((rows, len(m["xy"])))
             B[:, node[x, y]] = val[:, c]
@@ -59,6 +64,6 @@ def test_first_iterate_is_the_fp64_product_rounded_once(rounds, rows, blocked):
                 at, want = node[x + 1, y + 1], step(e0[:, c])
             else:
                 rho = -(mass * step(e0[:, c]).astype(np.float64))
-                at, want = node[(x + 3) % nx, y + 3], step((rho * tau[0]).astype(f32))
+                at, want = node[(x + 3) % nx, y + 3], step((rho * (tau[0] / lumped)).astype(f32))
             np.testing.assert_array_equal(X[:, at], want.astype(np.float64))
             assert (want != 0).all()
