@@ -557,8 +557,8 @@ __device__ __forceinline__ void store_start(const Bufs& b, int Np, int i, const 
 // mixed-precision solve, in FP32 together with the FP32 copy of the
 // right-hand side.
 //
-// Bound by the FP64 pipe (108 FMAs, 60 operations on the weights a node): 180 us on
-// 520,704 nodes, 602 us on 2,082,816 (Start32 in FP64: 204 and 789); 256 us on
+// Bound by the FP64 pipe (108 FMAs, 60 operations on the weights a node): 162 us on
+// 520,704 nodes, 587 us on 2,082,816 (Start32 in FP64: 204 and 789); 256 us on
 // 520,704 with the weights formed direction by direction as well.
 // One thread per node, or (kSets = 2, consecutive blocks) one per node and set,
 // which forms the weights twice but halves a thread's chain of loads and its

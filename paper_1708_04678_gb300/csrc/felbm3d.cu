@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(128) k3_element(DevMesh3 m, Phys3 c, Bufs3 b) 
 // Ten lanes per node (three nodes per warp): lane c > 0 takes the directions
 // 2c - 1 and 2c, which are opposite, of both sets, so one e.b serves four
 // products and the lanes of a node read a residual row as one contiguous run;
-// lane 0 takes the rest populations.  1,113 us on 262,144 nodes against 1,230 us
+// lane 0 takes the rest populations.  1,086 us on 262,144 nodes against 1,230 us
 // for one thread per node and set; 49 against 95 us on 7,350 nodes.
 template <bool kMixed>
 __global__ void __launch_bounds__(kNodeBlock) k3_rhs(DevMesh3 m, Phys3 c, Bufs3 b, double first_scale) {
@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kNodeBlock) k3_sweep32(DevMesh3 m, Phys3 c, Bu
 // iterate of the next correction, tau_0 rho / m.  x64 = x0, rho64 = x1.  Ten
 // lanes per node (three nodes per warp), lane c the 16-byte vector c of the
 // rows, so a gathered row is one contiguous load; the gathered floats are
-// widened on the integer pipe (the kernel is bound by the FP64 pipe): 486 us on
+// widened on the integer pipe (the kernel is bound by the FP64 pipe): 470 us on
 // 262,144 nodes against 670 us with conversion instructions.
 __global__ void __launch_bounds__(kCoopBlock) k3_refine(DevMesh3 m, Bufs3 b, const float* e, float* next_first,
                                                         int first_round, double tau0) {

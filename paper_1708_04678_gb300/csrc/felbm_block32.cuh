@@ -24,7 +24,7 @@
 //                                    step at a time   blocked
 //   2,082,816 nodes, FP32, 10 steps      1,098 us      758 us
 //     131,072 nodes, FP32, 10 steps        109 us       82 us (rows of 9)
-//     520,704 nodes, FP64, 3 x 14        2,019 us    1,317 us (FP64 refinement included)
+//     520,704 nodes, FP64, 3 x 14        2,019 us    1,280 us (FP64 refinement included)
 //       2,112 nodes, FP64, 3 x 14          164 us       43 us
 // Blocks of 512 nodes at 64 registers put two thread blocks on a
 // multiprocessor, one computing while the other loads.  With blocks of 1,024
